@@ -10,9 +10,23 @@
 // without its division by r_i (which tends to 0 as alpha_i -> 1 and
 // delta_i -> -inf).
 //
-// One warp per query row; lane l holds elements l, l + 32, ... of q and o.
+// A CTA of four warps takes BM = 16 TM query rows of one head against key tiles of 64. Thread
+// (ty, tx) of the 16 x 8 arrangement holds rows 16 w + 4 i + ty % 4 (i < TM, w the warp) and, of a
+// score tile, keys tx + 8 j, of the output, columns 4 tx + 32 c .. + 3: a warp owns its 4 TM rows
+// through both products, so the probabilities pass through shared memory within the warp and the
+// row statistics are eight-lane shuffles.
+//
+// Bound: the register ports of the fp32 FMAs. 4 B Hq Lq L D flops at the pipe's 128 FMA/clk/SM
+// (76 TFLOP/s at 1.95 GHz) are the floor (tensor cores would round the operands), but an FMA whose
+// three operands all come from the register file takes about 1.4 issue slots instead of 1, packed
+// f32x2 (2.8 for two, measured) or not. The packed form leaves issue slots for the rest of the
+// loop: 122 against 143 us with scalar FMAs on 32 heads x 512 rows x 512 keys, D = 128 (35 TFLOP/s;
+// one warp per row with a shuffle reduction per key took 1140 us). Two other layouts measured the
+// same there: eight warps with half the register tile (125 us), and lanes whose shared-memory reads
+// do not merge (124 us).
 #include <math.h>
 
+#include "context.cuh"
 #include "kernels.cuh"
 #include "ptx.cuh"
 #include "route.cuh"
@@ -20,99 +34,321 @@
 namespace cover {
 namespace {
 
-constexpr int kWarps = 4;
+constexpr int kThreads = 128;
+constexpr int kBN = 64;    // keys per tile
 
-template <int D>
-__global__ void __launch_bounds__(kWarps * 32)
+template <int D, int TM>
+struct F32Tile {
+  static constexpr int kBM = 16 * TM;
+  static constexpr int kQ = kBM * D, kKV = kBN * D, kP = kBM * kBN;   // floats
+  static constexpr size_t kBytes = sizeof(float) * (kQ + 2 * kKV + kP) + sizeof(int) * kBM;
+};
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const float* src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float* src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+__device__ __forceinline__ ulonglong2 lds2(const float* p) { return *reinterpret_cast<const ulonglong2*>(p); }
+
+// Copies rows [0, ROWS) of D floats at src to shared memory; rows from `valid` on become zeros.
+// Swizzled, row r's 16-byte chunk c lands in chunk c ^ (r & 7). Without 16-byte alignment of src
+// (vec false) the same chunks go as four 4-byte copies.
+template <int D, int ROWS, bool kSwizzle>
+__device__ __forceinline__ void load_rows(float* dst, const float* __restrict__ src, int valid, bool vec) {
+  constexpr int kChunks = ROWS * D / 4;
+  const uint32_t base = smem_u32(dst);
+  for (int t = threadIdx.x; t < kChunks; t += kThreads) {
+    const int r = t / (D / 4), c = t % (D / 4);
+    const bool in = r < valid;
+    const float* g = src + (in ? static_cast<size_t>(r) * D + 4 * c : 0);
+    const uint32_t d = base + static_cast<uint32_t>(r * D + 4 * (kSwizzle ? c ^ (r & 7) : c)) * 4u;
+    if (vec) {
+      cp_async16(d, g, in);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) cp_async4(d + 4 * e, g + (in ? e : 0), in);
+    }
+  }
+}
+
+template <int D, int TM>
+__global__ void __launch_bounds__(kThreads, 2)
     attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ kc, const float* __restrict__ vc,
                     const float* __restrict__ km, const float* __restrict__ vm, const int32_t* __restrict__ seed_idx,
-                    int n_seeds, int B, int Hq, int Hkv, int Lq, int L, int q0, float* __restrict__ out,
-                    float* __restrict__ lse) {
-  constexpr int E = D / 32;
-  const int lane = threadIdx.x & 31;
-  const long long row = static_cast<long long>(blockIdx.x) * kWarps + threadIdx.x / 32;
-  const long long rows = static_cast<long long>(B) * Hq * Lq;
-  if (row >= rows) return;
-  const int i = q0 + static_cast<int>(row % Lq);   // memory position of this query row
-  const int hq = static_cast<int>((row / Lq) % Hq);
-  const int b = static_cast<int>(row / (static_cast<long long>(Lq) * Hq));
-  const int hkv = hq / (Hq / Hkv);
+                    int n_seeds, int Hq, int Hkv, int Lq, int L, int q0, int tiles, int vec,
+                    float* __restrict__ out, float* __restrict__ lse) {
+  using T = F32Tile<D, TM>;
+  constexpr int kC = D / 32;     // output column groups of a thread (four columns each)
+  extern __shared__ __align__(16) float smem[];
+  float* const sq = smem;
+  float* const sk = sq + T::kQ;
+  float* const sv = sk + T::kKV;
+  float* const sp = sv + T::kKV;
+  int* const slot = reinterpret_cast<int*>(sp + T::kP);
+
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // a half-warp's 16-byte shared-memory reads merge into one access when lanes i, i ^ 1 or lanes
+  // i, i ^ 2 read the same address: tx comes in adjacent pairs, tyl alternates
+  const int tx = (lane >> 1) & 7, tyl = (lane & 1) | (lane >> 4) << 1;
+  const unsigned head = blockIdx.x / static_cast<unsigned>(tiles);        // b * Hq + hq
+  const int row0 = static_cast<int>(blockIdx.x - head * tiles) * T::kBM;  // first query row of the tile
+  const int b = static_cast<int>(head / static_cast<unsigned>(Hq)), hq = static_cast<int>(head - b * Hq);
+  const size_t kv_head = static_cast<size_t>(b) * Hkv + hq / (Hq / Hkv);
+  const float* const k_base = kc + kv_head * L * D;
+  const float* const v_base = vc + kv_head * L * D;
   const float scale = 1.0f / sqrtf(static_cast<float>(D));
+  const int n_kv = (L + kBN - 1) / kBN;
 
-  // seed slot of this row: lowest s with seed_idx[b, s] == i
-  int my_slot = kNoSlot;
-  for (int s = lane; s < n_seeds; s += 32)
-    if (seed_idx[static_cast<size_t>(b) * n_seeds + s] == i) my_slot = min(my_slot, s);
-  for (int o = 16; o > 0; o >>= 1) my_slot = min(my_slot, __shfl_xor_sync(0xffffffffu, my_slot, o));
-  const bool is_seed = my_slot != kNoSlot;
+  route_clear(slot, T::kBM, threadIdx.x, kThreads);
+  griddep_wait();
+  load_rows<D, T::kBM, true>(sq, q + (static_cast<size_t>(head) * Lq + row0) * D, Lq - row0, vec);
+  load_rows<D, kBN, true>(sk, k_base, L, vec);
+  cp_async_commit();
+  load_rows<D, kBN, false>(sv, v_base, L, vec);
+  cp_async_commit();
+  __syncthreads();
+  route_scan(slot, seed_idx + static_cast<size_t>(b) * n_seeds, n_seeds, q0 + row0, T::kBM, L, threadIdx.x, kThreads);
 
-  float qr[E], acc[E];
-  const float* qrow = q + row * D;
+  const int r0 = 16 * TM / 4 * warp + tyl;   // this thread's rows are r0 + 4 i
+  uint64_t o[TM][2 * kC];
+  float m[TM], l[TM];
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    qr[e] = qrow[lane + 32 * e];
-    acc[e] = 0.0f;
+  for (int i = 0; i < TM; ++i) {
+    m[i] = -INFINITY;
+    l[i] = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 2 * kC; ++c) o[i][c] = 0;
   }
-  const size_t kv_head = (static_cast<size_t>(b) * Hkv + hkv) * L * D;
-  float m = -INFINITY, l = 0.0f;
-  for (int j = 0; j < L; ++j) {
-    if (is_seed && j == i) continue;   // cached diagonal term excluded
-    const float* krow = kc + kv_head + static_cast<size_t>(j) * D;
-    float dot = 0.0f;
+  int diag[TM];   // key column of a seed row's excluded diagonal term
+
+  for (int j = 0; j < n_kv; ++j) {
+    cp_async_wait<1>();   // K(j) (and Q) have landed; V(j) may be in flight
+    __syncthreads();
+    if (j == 0) {
 #pragma unroll
-    for (int e = 0; e < E; ++e) dot = fmaf(qr[e], krow[lane + 32 * e], dot);
-    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    const float s = dot * scale;
-    const float m_new = fmaxf(m, s);
-    const float a = expf(m - m_new);   // m = -inf on the first term gives 0
-    const float p = expf(s - m_new);
-    l = l * a + p;
-    const float* vrow = vc + kv_head + static_cast<size_t>(j) * D;
+      for (int i = 0; i < TM; ++i) diag[i] = slot[r0 + 4 * i] != kNoSlot ? q0 + row0 + r0 + 4 * i : -1;
+    }
+    // ---- scores: partial sums over even and odd d in the two halves of a pair ----
+    uint64_t s2[TM][8];
 #pragma unroll
-    for (int e = 0; e < E; ++e) acc[e] = acc[e] * a + p * vrow[lane + 32 * e];
-    m = m_new;
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int jj = 0; jj < 8; ++jj) s2[i][jj] = 0;
+#pragma unroll 4
+    for (int c = 0; c < D / 4; ++c) {
+      ulonglong2 qa[TM];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const int r = r0 + 4 * i;
+        qa[i] = lds2(sq + r * D + 4 * (c ^ (r & 7)));
+      }
+      const float* kp = sk + tx * D + 4 * (c ^ tx);
+#pragma unroll
+      for (int jj = 0; jj < 8; ++jj) {
+        const ulonglong2 ka = lds2(kp + 8 * jj * D);
+#pragma unroll
+        for (int i = 0; i < TM; ++i) s2[i][jj] = f2_fma(qa[i].x, ka.x, s2[i][jj]);
+#pragma unroll
+        for (int i = 0; i < TM; ++i) s2[i][jj] = f2_fma(qa[i].y, ka.y, s2[i][jj]);
+      }
+    }
+    __syncthreads();   // every warp is done with K(j)
+    if (j + 1 < n_kv) load_rows<D, kBN, true>(sk, k_base + static_cast<size_t>(j + 1) * kBN * D, L - (j + 1) * kBN, vec);
+    cp_async_commit();
+    // ---- online softmax of this thread's rows; P to shared memory ----
+    const int key0 = j * kBN + tx;
+    // only the last tile has keys past the end, only the tiles of the diagonal an excluded key
+    const bool masked = (j + 1) * kBN > L || (q0 + row0 < (j + 1) * kBN && q0 + row0 + T::kBM > j * kBN);
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+      float s[8], mx = -INFINITY;
+#pragma unroll
+      for (int jj = 0; jj < 8; ++jj) {
+        float lo, hi;
+        f2_unpack(s2[i][jj], lo, hi);
+        const int key = key0 + 8 * jj;
+        s[jj] = (lo + hi) * scale;
+        if (masked && (key >= L || key == diag[i])) s[jj] = -INFINITY;
+        mx = fmaxf(mx, s[jj]);
+      }
+#pragma unroll
+      for (int off = 8; off > 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+      const float m_new = fmaxf(m[i], mx);
+      const float ref = m_new == -INFINITY ? 0.0f : m_new;   // no term yet: every p is 0
+      const float a = expf(m[i] - ref);
+      m[i] = m_new;
+      float sum = 0.0f;
+      float* const pr = sp + (r0 + 4 * i) * kBN;
+#pragma unroll
+      for (int jj = 0; jj < 8; ++jj) {
+        const float p = expf(s[jj] - ref);
+        sum += p;
+        const int key = tx + 8 * jj;
+        pr[4 * ((key >> 2) ^ (tyl << 1)) + (key & 3)] = p;
+      }
+      l[i] = l[i] * a + sum;
+      const uint64_t aa = f2_pack(a, a);
+#pragma unroll
+      for (int c = 0; c < 2 * kC; ++c) o[i][c] = f2_mul(o[i][c], aa);
+    }
+    cp_async_wait<1>();   // V(j) has landed; K(j + 1) may be in flight
+    __syncthreads();
+    // ---- O += P V ----
+#pragma unroll 2
+    for (int kk = 0; kk < kBN / 4; ++kk) {
+      float4 pa[TM];
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+        pa[i] = *reinterpret_cast<const float4*>(sp + (r0 + 4 * i) * kBN + 4 * (kk ^ (tyl << 1)));
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float* vp = sv + (4 * kk + e) * D + 4 * tx;
+        ulonglong2 va[kC];
+#pragma unroll
+        for (int c = 0; c < kC; ++c) va[c] = lds2(vp + 32 * c);
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          const float p = e == 0 ? pa[i].x : e == 1 ? pa[i].y : e == 2 ? pa[i].z : pa[i].w;
+          const uint64_t pp = f2_pack(p, p);
+#pragma unroll
+          for (int c = 0; c < kC; ++c) {
+            o[i][2 * c] = f2_fma(pp, va[c].x, o[i][2 * c]);
+            o[i][2 * c + 1] = f2_fma(pp, va[c].y, o[i][2 * c + 1]);
+          }
+        }
+      }
+    }
+    __syncthreads();   // every warp is done with V(j)
+    if (j + 1 < n_kv) load_rows<D, kBN, false>(sv, v_base + static_cast<size_t>(j + 1) * kBN * D, L - (j + 1) * kBN, vec);
+    cp_async_commit();
   }
-  if (is_seed) {
-    // merge the masked-input self term (k_i, v_i)
-    const size_t mrow = ((static_cast<size_t>(b) * Hkv + hkv) * n_seeds + my_slot) * D;
-    float dot = 0.0f;
+
 #pragma unroll
-    for (int e = 0; e < E; ++e) dot = fmaf(qr[e], km[mrow + lane + 32 * e], dot);
-    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    const float s = dot * scale;
-    const float m_new = fmaxf(m, s);
-    const float a = (m == -INFINITY) ? 0.0f : expf(m - m_new);
-    const float p = expf(s - m_new);
-    l = l * a + p;
+  for (int i = 0; i < TM; ++i) {
+    const int r = r0 + 4 * i;
 #pragma unroll
-    for (int e = 0; e < E; ++e) acc[e] = acc[e] * a + p * vm[mrow + lane + 32 * e];
-    m = m_new;
+    for (int off = 8; off > 1; off >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
+    const int sl = slot[r];
+    if (__any_sync(0xffffffffu, sl != kNoSlot)) {
+      // merge the masked-input self term (k_i, v_i) of the warp's seed rows
+      const bool is_seed = sl != kNoSlot;
+      const size_t mrow = (kv_head * n_seeds + (is_seed ? sl : 0)) * D;
+      float dot = 0.0f;
+      if (is_seed) {
+#pragma unroll
+        for (int c = tx; c < D / 4; c += 8) {
+          const float4 qv = *reinterpret_cast<const float4*>(sq + r * D + 4 * (c ^ (r & 7)));
+          const float* kp = km + mrow + 4 * c;
+          dot = fmaf(qv.x, kp[0], fmaf(qv.y, kp[1], fmaf(qv.z, kp[2], fmaf(qv.w, kp[3], dot))));
+        }
+      }
+#pragma unroll
+      for (int off = 8; off > 1; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+      if (is_seed) {
+        const float s = dot * scale;
+        const float m_new = fmaxf(m[i], s);
+        const float a = (m[i] == -INFINITY) ? 0.0f : expf(m[i] - m_new);
+        const float p = expf(s - m_new);
+        l[i] = l[i] * a + p;
+        m[i] = m_new;
+        const uint64_t aa = f2_pack(a, a), pp = f2_pack(p, p);
+#pragma unroll
+        for (int c = 0; c < kC; ++c) {
+          const float* vp = vm + mrow + 32 * c + 4 * tx;
+          o[i][2 * c] = f2_fma(pp, f2_pack(vp[0], vp[1]), f2_mul(o[i][2 * c], aa));
+          o[i][2 * c + 1] = f2_fma(pp, f2_pack(vp[2], vp[3]), f2_mul(o[i][2 * c + 1], aa));
+        }
+      }
+    }
+    if (row0 + r < Lq) {
+      const float inv = 1.0f / l[i];
+      const size_t row = static_cast<size_t>(head) * Lq + row0 + r;
+#pragma unroll
+      for (int c = 0; c < kC; ++c) {
+        float x0, x1, x2, x3;
+        f2_unpack(o[i][2 * c], x0, x1);
+        f2_unpack(o[i][2 * c + 1], x2, x3);
+        float* op = out + row * D + 32 * c + 4 * tx;
+        if (vec) {
+          *reinterpret_cast<float4*>(op) = make_float4(x0 * inv, x1 * inv, x2 * inv, x3 * inv);
+        } else {
+          op[0] = x0 * inv;
+          op[1] = x1 * inv;
+          op[2] = x2 * inv;
+          op[3] = x3 * inv;
+        }
+      }
+      if (lse != nullptr && tx == 0) lse[row] = m[i] + logf(l[i]);
+    }
   }
-  const float inv = 1.0f / l;
-#pragma unroll
-  for (int e = 0; e < E; ++e) out[row * D + lane + 32 * e] = acc[e] * inv;
-  if (lse != nullptr && lane == 0) lse[row] = m + logf(l);
+}
+
+template <int D, int TM>
+int launch_tile(const AttnArgs& a, bool vec, cudaStream_t stream) {
+  static ContextCache<int> cache;
+  int ready = 0;
+  const int rc = cache.get(&ready, [](int& v) {
+    v = 1;
+    return cudaFuncSetAttribute(attn_f32_kernel<D, TM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(F32Tile<D, TM>::kBytes)) == cudaSuccess ? 0 : -3;
+  });
+  if (rc != 0) return rc;
+  const int tiles = (a.Lq + F32Tile<D, TM>::kBM - 1) / F32Tile<D, TM>::kBM;
+  const long long blocks = static_cast<long long>(a.B) * a.Hq * tiles;
+  if (blocks > 0x7fffffffLL) return -2;
+  cudaLaunchAttribute attr[1];
+  const cudaLaunchConfig_t cfg =
+      pdl_config(dim3(static_cast<unsigned>(blocks)), dim3(kThreads), F32Tile<D, TM>::kBytes, stream, attr);
+  const cudaError_t err = cudaLaunchKernelEx(
+      &cfg, attn_f32_kernel<D, TM>, static_cast<const float*>(a.q), static_cast<const float*>(a.k_cached),
+      static_cast<const float*>(a.v_cached), static_cast<const float*>(a.k_seedmask),
+      static_cast<const float*>(a.v_seedmask), a.seed_idx, a.n_seeds, a.Hq, a.Hkv, a.Lq, a.L, a.q0, tiles,
+      vec ? 1 : 0, static_cast<float*>(a.out), a.lse);
+  return err == cudaSuccess ? 0 : -3;
+}
+
+// Rows per CTA: a launch lasts about as long as the SM with the most CTAs, so the cost of 16 TM
+// rows a CTA is ceil(CTAs / SMs) times a CTA's cost, which the shared K / V work keeps from falling
+// with TM: 32, 43, 75 for TM = 1, 2, 4 (in rows of the FMA pipe's rate; fitted to the first and
+// fourth shape below). us at TM = 1 / 2 / 4 (heads x rows x keys, D): 32 x 512 x 512, 128: 177 / 136
+// / 119; 8 x 512 x 512, 128: 50 / 42 / 69; 4 x 256 x 256, 64: 11.3 / 13.8 / 20.8; 32 x 300 x 300, 128:
+// 63 / 66 / 76; 16 x 700 x 700, 64: 97 / 80 / 87; 32 x 32 x 1024, 128: 66 / 80 / 132. The rule takes
+// the fastest on each.
+template <int D>
+int launch_rows(const AttnArgs& a, bool vec, cudaStream_t stream) {
+  static ContextCache<int> cache;
+  int n_sm = 0;
+  const int rc = cache.get(&n_sm, [](int& v) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return -3;
+    return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? 0 : -3;
+  });
+  if (rc != 0) return rc;
+  const auto cost = [&](int rows, int cta_cost) {
+    const long long ctas = static_cast<long long>(a.B) * a.Hq * ((a.Lq + rows - 1) / rows);
+    return (ctas + n_sm - 1) / n_sm * cta_cost;
+  };
+  const long long c16 = cost(16, 32), c32 = cost(32, 43), c64 = cost(64, 75);
+  if (c64 <= c32 && c64 <= c16) return launch_tile<D, 4>(a, vec, stream);
+  if (c32 <= c16) return launch_tile<D, 2>(a, vec, stream);
+  return launch_tile<D, 1>(a, vec, stream);
 }
 
 }  // namespace
 
 int launch_attn_f32(const AttnArgs& a, int* /*status*/, cudaStream_t stream) {
-  const long long rows = static_cast<long long>(a.B) * a.Hq * a.Lq;
-  const long long blocks = (rows + kWarps - 1) / kWarps;
-  if (blocks > 0x7fffffffLL) return -2;
-  const float* q = static_cast<const float*>(a.q);
-  const float* kc = static_cast<const float*>(a.k_cached);
-  const float* vc = static_cast<const float*>(a.v_cached);
-  const float* km = static_cast<const float*>(a.k_seedmask);
-  const float* vm = static_cast<const float*>(a.v_seedmask);
-  float* out = static_cast<float*>(a.out);
-  if (a.D == 64)
-    attn_f32_kernel<64><<<static_cast<unsigned>(blocks), kWarps * 32, 0, stream>>>(
-        q, kc, vc, km, vm, a.seed_idx, a.n_seeds, a.B, a.Hq, a.Hkv, a.Lq, a.L, a.q0, out, a.lse);
-  else
-    attn_f32_kernel<128><<<static_cast<unsigned>(blocks), kWarps * 32, 0, stream>>>(
-        q, kc, vc, km, vm, a.seed_idx, a.n_seeds, a.B, a.Hq, a.Hkv, a.Lq, a.L, a.q0, out, a.lse);
-  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+  bool vec = true;   // 16-byte copies; the entry point asks for 4-byte alignment only
+  for (const void* p : {a.q, a.k_cached, a.v_cached, static_cast<const void*>(a.out)})
+    vec = vec && reinterpret_cast<uintptr_t>(p) % 16 == 0;
+  return a.D == 64 ? launch_rows<64>(a, vec, stream) : launch_rows<128>(a, vec, stream);
 }
 
 }  // namespace cover

@@ -88,6 +88,42 @@ def test_f32_shapes(B, Hq, Hkv, L, D, S):
     H.assert_f32_close(out, ref, lse, ref_lse)
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,L,D,S", [
+    (1, 2, 1, 16, 128, 3), (1, 2, 2, 17, 64, 2), (1, 1, 1, 63, 128, 4), (1, 1, 1, 64, 64, 4),   # 16 rows a CTA
+    (1, 50, 25, 90, 64, 6), (1, 50, 10, 96, 128, 5),      # 32 rows a CTA, a ragged last tile and a full one
+    (1, 50, 25, 130, 64, 9), (2, 38, 19, 128, 128, 128),  # 64 rows a CTA; every row a seed
+])
+def test_f32_row_tiles(B, Hq, Hkv, L, D, S):
+    """Every row tile of the fp32 kernel at the edges of its row and key tiles (152 SMs choose as noted)."""
+    inp = W.make_attn_inputs(B, Hq, Hkv, L, D, S, dtype="f32", seed=L + S)
+    out, lse = H.run_attn(inp)
+    ref, ref_lse = H.oracle_full(inp)
+    H.assert_f32_close(out, ref, lse, ref_lse)
+
+
+@pytest.mark.parametrize("which", range(4))
+def test_f32_unaligned_rows_equal_aligned(which):
+    """A tensor that is only 4-byte aligned takes the 4-byte copies: the same bits."""
+    inp = W.make_attn_inputs(1, 2, 1, 70, 64, 5, dtype="f32", seed=4)
+    t = [H.to_dev(x, "f32") for x in (inp.q, inp.k_cached, inp.v_cached, inp.k_seedmask, inp.v_seedmask)]
+    seeds = H.to_dev(inp.seed_idx, "i32")
+    out = torch.empty_like(t[0])
+    ref = api.cover_attn_fwd_f32(*t, seeds)
+
+    def shifted(x):
+        y = torch.empty(x.numel() + 1, dtype=x.dtype, device=x.device)[1:].view(x.shape)
+        return y.copy_(x)
+
+    if which < 3:
+        t[which] = shifted(t[which])
+    else:
+        out = shifted(out)
+        t[3], t[4] = shifted(t[3]), shifted(t[4])
+    got = api.cover_attn_fwd_f32(*t, seeds, out=out)
+    torch.cuda.synchronize()
+    assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
+
+
 # ----------------------------------------------------------------------------
 # bf16 tcgen05 path: small shapes, ragged tails, seeds in every position class
 # ----------------------------------------------------------------------------
