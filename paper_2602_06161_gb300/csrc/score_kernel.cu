@@ -1,7 +1,7 @@
 // score_kernel.cu - fused per-position scoring over the vocabulary and top-k
 // seed selection.
 //
-// Per row (one CTA per row, the row streamed once from HBM):
+// Per row (one CTA, or one cluster, per row; the row streamed once from HBM):
 //   greedy token y_hat = argmax p and confidence c = max p       (Section 3)
 //   entropy H = -sum p ln p                                       (Section 6.1)
 //   uncertainty u = -log p(y), Score = u (1 + d_in)/(1 + d_out)   (Section 5.3)
@@ -26,18 +26,19 @@
 // (n_t pi_t), and selects ceil(sqrt(n_t pi_t)) new seeds among the rows that
 // were not seeds and have ReMasks left, with the same 64-bit key sort.
 //
-// Two ways to stream a row:
-//  * score_bulk_kernel (rows 16-byte aligned, V % 8 == 0): a producer warp
-//    issues cp.async.bulk copies of 16 KB chunks into a 3-stage shared-memory
-//    ring (mbarrier full / empty), 8 consumer warps reduce from shared memory;
-//    bytes in flight do not cost registers, and 4 CTAs share an SM.
-//  * score_kernel (any V): 16-byte non-allocating global loads, scalar head and
-//    tail for rows that do not start on a 16-byte boundary.
+// Streaming: a producer warp issues cp.async.bulk copies of 16 KB chunks of the row's aligned
+// 16-byte vectors into a 3-stage shared-memory ring (mbarrier full / empty), 8 consumer warps
+// reduce from shared memory; bytes in flight do not cost registers, and 4 CTAs share an SM. The
+// up to 14 elements outside the aligned vectors (V or the row's offset not a multiple of 8) are
+// read by the producer warp's other lanes, so every V takes this path: a kernel of 16-byte register
+// loads for such rows took 57.9 us on 1024 rows of V = 126465 against 50.1 us. With few
+// rows each is split over the CTAs of a cluster (row_split), whose slice sums its first CTA adds.
 #include <math.h>
 #include <stdint.h>
 
 #include <algorithm>
 
+#include "cluster.cuh"
 #include "context.cuh"
 #include "kernels.cuh"
 #include "ptx.cuh"
@@ -45,10 +46,7 @@
 namespace cover {
 namespace {
 
-constexpr int kThreads = 512;              // register-load kernel
-constexpr int kWarps = kThreads / 32;
-constexpr int kUnroll = 4;
-constexpr int kConsumerWarps = 8;          // bulk kernel: consumers + 1 producer warp
+constexpr int kConsumerWarps = 8;          // consumers + 1 producer warp
 constexpr int kBulkThreads = (kConsumerWarps + 1) * 32;
 constexpr int kChunkElems = 8192;          // 16 KB of bf16 per bulk copy
 constexpr int kChunkBytes = kChunkElems * 2;
@@ -60,6 +58,8 @@ constexpr int kRowLoads = 4;                // rows whose state a thread loads a
 constexpr int kRoundsMax = 32;              // selections up to this size by rounds or warp sorts (top_select)
 constexpr int kRoundsFew = 8;               // selections up to this size by per-warp rounds (top_rounds)
 constexpr int kMaxWarps = 16;               // every kernel here runs at most 512 threads
+constexpr int kMaxSplit = 8;                // CTAs a row is split over (the portable cluster size)
+constexpr int kMinSlice = 2048;             // elements of a row a CTA gets at least
 
 struct RowAcc {
   float m;     // running maximum logit of this thread's elements
@@ -143,6 +143,14 @@ struct RowOut {
   float q;      // (sum t 2^t) / Z
 };
 
+// A row's (or a row slice's) sums as unevaluated pairs (value, rounding error).
+struct alignas(8) RowSum {
+  float M;        // maximum; -inf for an empty slice
+  int yhat;       // first index attaining it
+  float zh, zl;   // sum 2^t re-referenced to M log2(e)
+  float sh, sl;   // sum t 2^t
+};
+
 // a + b = s + e exactly (Knuth's TwoSum)
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = a + b;
@@ -154,7 +162,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // kStride elements apart; the loads are issued by the threads that hold their warp's maximum
 // before the block-wide maximum is known, so their latency overlaps the reduction.
 constexpr int kMaxBatch = 4;
-static_assert(kVecPerThread <= kMaxBatch && kUnroll <= kMaxBatch, "batches hold at most four vectors");
+static_assert(kVecPerThread <= kMaxBatch, "batches hold at most four vectors");
 
 template <int kStride>
 __device__ __forceinline__ void load_batch(const RowAcc& a, const uint16_t* row, uint4 (&w)[kMaxBatch]) {
@@ -181,7 +189,7 @@ __device__ __forceinline__ int first_index_of(const RowAcc& a, float M, const ui
 }
 
 template <int NW, int kStride>
-__device__ __forceinline__ RowOut row_reduce(const RowAcc& a, const uint16_t* row, float* red_m, int* red_i,
+__device__ __forceinline__ RowSum row_reduce(const RowAcc& a, const uint16_t* row, float* red_m, int* red_i,
                                              float2* red_z, float2* red_s) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float m = a.m;
@@ -195,13 +203,12 @@ __device__ __forceinline__ RowOut row_reduce(const RowAcc& a, const uint16_t* ro
   float M = red_m[0];
 #pragma unroll
   for (int i = 1; i < NW; ++i) M = fmaxf(M, red_m[i]);
-  const float Mref = M * kLog2e;
-  // partials re-referenced to the row maximum, summed across the warp in fp32
+  // partials re-referenced to the row maximum (to the unrounded M log2 e), summed across the warp in fp32
   // with error-free TwoSum pairs (value, rounding error), then across the warps
   // the same way by thread 0
   float z = 0.0f, ze = 0.0f, sv = 0.0f, se = 0.0f;
   if (a.m != -INFINITY) {
-    const float d = a.mref - Mref;
+    const float d = fmaf(-M, kLog2e, a.mref);
     const float f = ex2_approx(d);
     const float zz = a.z - a.zc;
     const float ss = a.s - a.sc;
@@ -228,7 +235,7 @@ __device__ __forceinline__ RowOut row_reduce(const RowAcc& a, const uint16_t* ro
     red_s[warp] = make_float2(sv, se);
   }
   __syncthreads();
-  RowOut r{M, 0x7fffffff, 0.0f, 0.0f};
+  RowSum r{M, 0x7fffffff, 0.0f, 0.0f, 0.0f, 0.0f};
   if (tid == 0) {
     int I = red_i[0];
 #pragma unroll
@@ -236,24 +243,70 @@ __device__ __forceinline__ RowOut row_reduce(const RowAcc& a, const uint16_t* ro
     r.yhat = I;
     // the warps' (value, error) pairs added with TwoSum in fp32 (no fp64: this GPU's fp64 adds
     // have long latencies, and this runs at the end of every row with no copy in flight)
-    float zh = red_z[0].x, zl = red_z[0].y, sh = red_s[0].x, sl = red_s[0].y;
+    r.zh = red_z[0].x, r.zl = red_z[0].y, r.sh = red_s[0].x, r.sl = red_s[0].y;
 #pragma unroll
     for (int w = 1; w < NW; ++w) {
       float t, e;
-      two_sum(zh, red_z[w].x, t, e);
-      zl += e + red_z[w].y;
-      zh = t;
-      two_sum(sh, red_s[w].x, t, e);
-      sl += e + red_s[w].y;
-      sh = t;
+      two_sum(r.zh, red_z[w].x, t, e);
+      r.zl += e + red_z[w].y;
+      r.zh = t;
+      two_sum(r.sh, red_s[w].x, t, e);
+      r.sl += e + red_s[w].y;
+      r.sh = t;
     }
-    // S / Z with one correction step on the pairs: q = sh / zh, then the residual of
-    // (sh + sl) - q (zh + zl) divided by zh
-    const float q0 = sh / zh;
-    const float res = fmaf(-q0, zh, sh) + (sl - q0 * zl);
-    r.q = q0 + res / zh;
-    r.Z = zh + zl;
   }
+  return r;
+}
+
+// S / Z with one correction step on the pairs: q = sh / zh, then the residual of
+// (sh + sl) - q (zh + zl) divided by zh
+__device__ __forceinline__ RowOut row_finish(const RowSum& r) {
+  const float q0 = r.sh / r.zh;
+  const float res = fmaf(-q0, r.zh, r.sh) + (r.sl - q0 * r.zl);
+  return {r.M, r.yhat, r.zh + r.zl, q0 + res / r.zh};
+}
+
+// The sum of the row slices in part[0 .. C), on the lanes of one warp: every lane returns it.
+// Each slice's pairs move to the row maximum (S by the error-free product d zh), then a tree
+// of TwoSums adds them, so a split row keeps the accuracy of an unsplit one.
+template <int C>
+__device__ __forceinline__ RowSum row_combine(const RowSum* part, int lane) {
+  RowSum r = part[lane & (C - 1)];
+  float M = r.M;
+#pragma unroll
+  for (int o = C / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  int y = r.M == M ? r.yhat : 0x7fffffff;
+  if (r.M != -INFINITY) {
+    // d + dl = (r.M - M) log2 e to twice the precision: its rounding would shift the whole slice
+    const float d = __fmul_rn(r.M - M, kLog2e);   // <= 0
+    const float dl = fmaf(r.M - M, kLog2e, -d);
+    float f = ex2_approx(d);
+    f = fmaf(f, 0.6931471805599453f * dl, f);
+    const float p = d * r.zh;
+    float sh, se;
+    two_sum(r.sh, p, sh, se);
+    const float sl = se + fmaf(d, r.zh, -p) + fmaf(d, r.zl, r.sl) + dl * r.zh;
+    r.sh = f * sh;
+    r.sl = fmaf(f, sh, -r.sh) + f * sl;
+    const float zh = r.zh;
+    r.zh = f * zh;
+    r.zl = fmaf(f, zh, -r.zh) + f * r.zl;
+  }
+#pragma unroll
+  for (int o = C / 2; o > 0; o >>= 1) {
+    y = min(y, __shfl_xor_sync(0xffffffffu, y, o));
+    const float zh2 = __shfl_xor_sync(0xffffffffu, r.zh, o), zl2 = __shfl_xor_sync(0xffffffffu, r.zl, o);
+    const float sh2 = __shfl_xor_sync(0xffffffffu, r.sh, o), sl2 = __shfl_xor_sync(0xffffffffu, r.sl, o);
+    float t, e;
+    two_sum(r.zh, zh2, t, e);
+    r.zl += zl2 + e;
+    r.zh = t;
+    two_sum(r.sh, sh2, t, e);
+    r.sl += sl2 + e;
+    r.sh = t;
+  }
+  r.M = M;
+  r.yhat = y;
   return r;
 }
 
@@ -1212,61 +1265,7 @@ __device__ __forceinline__ void acc_batch(RowAcc& a, const uint4 (&w)[U], int i0
 
 
 // ---------------------------------------------------------------------------
-// register-load kernel (any V)
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads, 2) score_kernel(const ScoreParams P) {
-  extern __shared__ __align__(16) uint64_t keys[];
-  __shared__ float red_m[kWarps];
-  __shared__ int red_i[kWarps];
-  __shared__ float2 red_z[kWarps], red_s[kWarps];
-  __shared__ int s_last;
-  // programmatic dependent launch: wait for the stream's previous kernel, let the next one be
-  // scheduled
-  griddep_wait();
-  griddep_launch_dependents();
-
-  const int n = blockIdx.x;
-  const int tid = threadIdx.x;
-  const int V = P.V;
-  const size_t row_off = static_cast<size_t>(n) * V;
-  const uint16_t* row = P.logits + row_off;
-  RowAcc a{-INFINITY, 0x7fffffff, 0, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-
-  // elements before the first 16-byte boundary of the row
-  const int head = min(static_cast<int>((8 - (row_off & 7)) & 7), V);
-  const int nvec = (V - head) / 8;
-  const int tail0 = head + nvec * 8;
-  if (tid < head) acc_scalar(a, bf16_to_f32(row[tid]), tid);
-  const uint4* vrow = reinterpret_cast<const uint4*>(row + head);
-  int v = tid;
-  for (; v + (kUnroll - 1) * kThreads < nvec; v += kUnroll * kThreads) {
-    uint4 w[kUnroll];
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) w[u] = ld_stream(vrow + v + u * kThreads);
-    acc_batch<kUnroll>(a, w, head + v * 8);
-  }
-  for (; v < nvec; v += kThreads) {
-    uint4 w[1] = {ld_stream(vrow + v)};
-    acc_batch<1>(a, w, head + v * 8);
-  }
-  if (tail0 + tid < V) acc_scalar(a, bf16_to_f32(row[tail0 + tid]), tail0 + tid);
-
-  const RowOut r = row_reduce<kWarps, kThreads * 8>(a, row, red_m, red_i, red_z, red_s);
-  if (tid == 0)
-    s_last = row_write(r, n, row, V, P.per_seq, P.decide ? P.dec.tok : P.cur_tok, P.d_in, P.d_out, P.topk,
-                       P.maxprob, P.entropy, P.argmax, P.score, P.counters, P.decide ? P.dec.ws_u : nullptr,
-                       P.decide ? P.dec.ws_lnz : nullptr);
-  __syncthreads();
-  if (s_last) {
-    if (P.decide)
-      segment_decide(keys, n / P.per_seq, P.per_seq, P.sort_n, P);
-    else
-      segment_topk(keys, n / P.per_seq, P.per_seq, P.sort_n, P.topk, P.score, P.eligible, P.topk_idx, P.topk_score);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// bulk-copy kernel (rows 16-byte aligned)
+// row kernel: bulk copies of a row, or of a row's slice in each CTA of a cluster
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile(
@@ -1276,6 +1275,18 @@ __device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint3
       : "memory");
 }
 
+// Writes r to *dst of the cluster's CTA `rank` (dst: this CTA's copy of the same variable).
+__device__ __forceinline__ void cluster_store_row_sum(RowSum* dst, uint32_t rank, const RowSum& r) {
+  const uint32_t d = cluster_map(smem_u32(dst), rank);
+  asm volatile(
+      "st.shared::cluster.v2.f32 [%0], {%1, %2};\n\t"
+      "st.shared::cluster.v2.f32 [%0 + 8], {%3, %4};\n\t"
+      "st.shared::cluster.v2.f32 [%0 + 16], {%5, %6};" ::"r"(d),
+      "f"(r.M), "f"(__int_as_float(r.yhat)), "f"(r.zh), "f"(r.zl), "f"(r.sh), "f"(r.sl)
+      : "memory");
+}
+
+template <int C>
 __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const ScoreParams P, int* status) {
   extern __shared__ __align__(128) uint8_t dsmem[];   // ring, reused for top-k keys
   __shared__ uint64_t bar_full[kRingStages], bar_empty[kRingStages];
@@ -1283,16 +1294,28 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
   __shared__ int red_i[kConsumerWarps + 1];
   __shared__ float2 red_z[kConsumerWarps + 1], red_s[kConsumerWarps + 1];
   __shared__ int s_last, s_abort;
+  __shared__ RowSum s_part[C];   // the cluster's slice sums, in its first CTA
+  if (C > 1) cluster_arrive();   // completed before the slice sums are sent: every CTA has started
   // programmatic dependent launch: wait for the stream's previous kernel, let the next one be
   // scheduled
   griddep_wait();
   griddep_launch_dependents();
 
-  const int n = blockIdx.x;
+  const int n = blockIdx.x / C;
+  const int rank = C > 1 ? static_cast<int>(cluster_ctarank()) : 0;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int V = P.V;
-  const uint16_t* row = P.logits + static_cast<size_t>(n) * V;
-  const int nchunks = (V + kChunkElems - 1) / kChunkElems;
+  const size_t row_off = static_cast<size_t>(n) * V;
+  const uint16_t* row = P.logits + row_off;
+  // the row's aligned 16-byte vectors go through the ring, the few elements before and after
+  // them are read directly
+  const int head = min(static_cast<int>((8 - (row_off & 7)) & 7), V);
+  const int row_vec = (V - head) / 8;
+  const int slice = C > 1 ? (row_vec + C - 1) / C : row_vec;
+  const int first = head + min(rank * slice, row_vec) * 8;   // first element of this CTA's slice
+  const int elems_all = min(slice, row_vec - min(rank * slice, row_vec)) * 8;
+  const int nchunks = (elems_all + kChunkElems - 1) / kChunkElems;
+  const uint16_t* src_row = row + first;
   uint8_t* ring = dsmem;
 
   if (warp == kConsumerWarps && lane == 0) {
@@ -1305,10 +1328,10 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
     s_abort = 0;
     fence_mbar_init();
     for (int c = 0; c < kRingStages && c < nchunks; ++c) {
-      const int elems = min(kChunkElems, V - c * kChunkElems);
+      const int elems = min(kChunkElems, elems_all - c * kChunkElems);
       mbar_arrive_expect_tx(&bar_full[c], static_cast<uint32_t>(elems * 2));
-      bulk_load(ring + c * kChunkBytes, row + static_cast<size_t>(c) * kChunkElems, static_cast<uint32_t>(elems * 2),
-                &bar_full[c]);
+      bulk_load(ring + c * kChunkBytes, src_row + static_cast<size_t>(c) * kChunkElems,
+                static_cast<uint32_t>(elems * 2), &bar_full[c]);
     }
   }
   __syncthreads();
@@ -1324,13 +1347,17 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
           s_abort = 1;
           break;
         }
-        const int elems = min(kChunkElems, V - c * kChunkElems);
+        const int elems = min(kChunkElems, elems_all - c * kChunkElems);
         mbar_arrive_expect_tx(&bar_full[st], static_cast<uint32_t>(elems * 2));
-        bulk_load(ring + st * kChunkBytes, row + static_cast<size_t>(c) * kChunkElems,
+        bulk_load(ring + st * kChunkBytes, src_row + static_cast<size_t>(c) * kChunkElems,
                   static_cast<uint32_t>(elems * 2), &bar_full[st]);
       }
       // every copy issued has been consumed once the consumers pass their last
       // full-barrier wait; nothing is left in flight at the final barrier
+    } else if (rank == 0 && lane <= 16) {
+      // the elements outside the aligned vectors: lanes 1 .. 8 before them, 9 .. 16 after them
+      const int i = lane <= 8 ? lane - 1 : head + row_vec * 8 + lane - 9;
+      if (lane <= 8 ? i < head : i < V) acc_scalar(a, bf16_to_f32(row[i]), i);
     }
   } else {
     for (int c = 0; c < nchunks; ++c) {
@@ -1343,7 +1370,7 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
         }
         break;
       }
-      const int elems = min(kChunkElems, V - c * kChunkElems);
+      const int elems = min(kChunkElems, elems_all - c * kChunkElems);
       const uint4* src = reinterpret_cast<const uint4*>(ring + st * kChunkBytes);
       const int nv = elems / 8;
       constexpr int kStride = kConsumerWarps * 32;
@@ -1351,11 +1378,11 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
         uint4 w[kVecPerThread];
 #pragma unroll
         for (int u = 0; u < kVecPerThread; ++u) w[u] = src[tid + u * kStride];
-        acc_batch<kVecPerThread>(a, w, c * kChunkElems + tid * 8);
+        acc_batch<kVecPerThread>(a, w, first + c * kChunkElems + tid * 8);
       } else {
         for (int v = tid; v < nv; v += kStride) {
           uint4 w[1] = {src[v]};
-          acc_batch<1>(a, w, c * kChunkElems + v * 8);
+          acc_batch<1>(a, w, first + c * kChunkElems + v * 8);
         }
       }
       __syncwarp();
@@ -1367,10 +1394,22 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
     for (int c = max(0, nchunks - kRingStages); c < nchunks; ++c)
       mbar_wait(&bar_full[c % kRingStages], (c / kRingStages) & 1, nullptr, 1000000ull);
   }
+  __syncwarp();
 
-  const RowOut r = row_reduce<kConsumerWarps + 1, kConsumerWarps * 32 * 8>(a, row, red_m, red_i, red_z, red_s);
+  RowSum r = row_reduce<kConsumerWarps + 1, kConsumerWarps * 32 * 8>(a, row, red_m, red_i, red_z, red_s);
+  if (C > 1) {
+    // every CTA sends its slice's sums to the cluster's first, which adds them
+    __syncwarp();
+    cluster_wait();
+    if (tid == 0) cluster_store_row_sum(&s_part[rank], 0, r);
+    __syncwarp();
+    cluster_arrive();
+    if (rank != 0) return;
+    cluster_wait();
+    if (warp == 0) r = row_combine<C>(s_part, lane);
+  }
   if (tid == 0)
-    s_last = row_write(r, n, row, V, P.per_seq, P.decide ? P.dec.tok : P.cur_tok, P.d_in, P.d_out, P.topk,
+    s_last = row_write(row_finish(r), n, row, V, P.per_seq, P.decide ? P.dec.tok : P.cur_tok, P.d_in, P.d_out, P.topk,
                        P.maxprob, P.entropy, P.argmax, P.score, P.counters, P.decide ? P.dec.ws_u : nullptr,
                        P.decide ? P.dec.ws_lnz : nullptr);
   __syncthreads();
@@ -1386,7 +1425,7 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
 // Section 5.3 selection as its own launch (one CTA per segment), after the
 // update phase and the d_in / d_out pass.
 constexpr int kSelectThreads = 512;
-static_assert(kThreads <= 32 * kMaxWarps && kBulkThreads <= 32 * kMaxWarps && kSelectThreads <= 32 * kMaxWarps,
+static_assert(kBulkThreads <= 32 * kMaxWarps && kSelectThreads <= 32 * kMaxWarps,
               "top_rounds keeps a list per warp for at most kMaxWarps warps");
 __global__ void __launch_bounds__(kSelectThreads) seed_select_kernel(const DecideArgs d, const float* d_in,
                                                                     const float* d_out, float* score, int per_seq,
@@ -1423,49 +1462,70 @@ __global__ void __launch_bounds__(kSelectThreads) seed_select_kernel(const Decid
 
 namespace {
 
+template <int C>
+int launch_rows(const ScoreParams& P, int N, size_t smem, int* status, cudaStream_t stream) {
+  // the ring's shared-memory limit is a function attribute of the current context
+  static ContextCache<int> setup;
+  int unused = 0;
+  const int rc = setup.get(&unused, [](int&) {
+    return cudaFuncSetAttribute(score_bulk_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(kRingStages * kChunkBytes)) == cudaSuccess ? 0 : -3;
+  });
+  if (rc != 0) return rc;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = C;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(N) * C);
+  cfg.blockDim = dim3(kBulkThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = C > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, score_bulk_kernel<C>, P, status) == cudaSuccess ? 0 : -3;
+}
+
+// CTAs a row is split over. A row alone on an SM is bound by its own CTA (12 us at V = 126464), so
+// few rows are split until the launch holds two CTAs per SM. Beyond that the SMs' issue rate is
+// shared anyway and every further CTA only adds its start and reduction. us at 1 / 2 / 4 / 8 CTAs a
+// row, V = 126464: 32 rows 12.5 / 9.2 / 7.4 / 6.8, 64 rows 12.7 / 9.5 / 8.5 / 8.9, 128 rows 13.6 / 12.0
+// / 12.4 / 15.9, 152 rows 14.7 / 13.4 / 17.3 / 20.2, 200 rows 17.8 / 18.4 / 22.1 / 24.2. V = 32000:
+// 32 rows 6.4 / 6.3 / 5.9 / 5.5, 128 rows 7.0 / 7.2 / 7.7 / 11.5: halves of a short row do not pay.
+int row_split(int N, int V, int n_sm) {
+  int c = kMaxSplit;
+  while (c > 1 && (static_cast<long long>(N) * c > 2LL * n_sm || V < c * kMinSlice || (c == 2 && V < 65536))) c >>= 1;
+  return c;
+}
+
 int launch_score_impl(const ScoreArgs& a, const DecideArgs* d, int* status, cudaStream_t stream) {
+  static ContextCache<int> sms;
+  int n_sm = 0;
+  const int rc = sms.get(&n_sm, [](int& v) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return -3;
+    return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? 0 : -3;
+  });
+  if (rc != 0) return rc;
   const int per = a.N / a.n_seq;
   int sort_n = 1;
   while (sort_n < per) sort_n <<= 1;
   ScoreParams P{static_cast<const uint16_t*>(a.logits), a.V, per, a.cur_tok, a.d_in, a.d_out, a.eligible,
                 a.topk, sort_n, a.maxprob, a.entropy, a.argmax, a.score, a.topk_idx, a.topk_score, a.counters,
                 d != nullptr ? 1 : 0, d != nullptr ? *d : DecideArgs{}};
-  // top-k keys; the decision step also keeps a float score per row behind them. At least one key
-  // per thread of the register-load kernel: the one-row-per-thread selection publishes up to
-  // 32 keys per warp.
-  const size_t key_slots = static_cast<size_t>(std::max(sort_n, kThreads));
-  const size_t keys_bytes = d != nullptr ? (sizeof(uint64_t) + sizeof(float)) * key_slots
-                            : a.topk > 0 ? sizeof(uint64_t) * key_slots : 0;
-  const bool aligned_rows = (a.V % 8) == 0 && (reinterpret_cast<uintptr_t>(a.logits) % 16) == 0;
-  if (aligned_rows) {
-    const size_t smem = std::max(keys_bytes, static_cast<size_t>(kRingStages) * kChunkBytes);
-    // the ring's shared-memory limit is a function attribute of the current context
-    static ContextCache<int> setup;
-    int unused = 0;
-    const int rc = setup.get(&unused, [](int&) {
-      return cudaFuncSetAttribute(score_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(kRingStages * kChunkBytes)) == cudaSuccess ? 0 : -3;
-    });
-    if (rc != 0) return rc;
-    cudaLaunchAttribute attr[1];
-    const cudaLaunchConfig_t cfg = pdl_config(dim3(a.N), dim3(kBulkThreads), smem, stream, attr);
-    if (cudaLaunchKernelEx(&cfg, score_bulk_kernel, P, status) != cudaSuccess) return -3;
-  } else {
-    // decision keys of the longest segment: 4096 x 12 bytes, above the 48 KB a launch gets
-    // without opting in (with the static shared memory)
-    static ContextCache<int> setup_reg;
-    int unused = 0;
-    const int rc = setup_reg.get(&unused, [](int&) {
-      return cudaFuncSetAttribute(score_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>((sizeof(uint64_t) + sizeof(float)) * kMaxPerSeq)) == cudaSuccess
-                 ? 0 : -3;
-    });
-    if (rc != 0) return rc;
-    cudaLaunchAttribute attr[1];
-    const cudaLaunchConfig_t cfg = pdl_config(dim3(a.N), dim3(kThreads), keys_bytes, stream, attr);
-    if (cudaLaunchKernelEx(&cfg, score_kernel, P) != cudaSuccess) return -3;
+  // top-k keys (at most 4096 x 8 bytes) reuse the ring; so does the decision step, which keeps a
+  // float score per row behind them (4096 x 12 bytes, exactly the ring)
+  static_assert((sizeof(uint64_t) + sizeof(float)) * kMaxPerSeq <= kRingStages * kChunkBytes, "keys fit the ring");
+  const size_t smem = static_cast<size_t>(kRingStages) * kChunkBytes;
+  switch (row_split(a.N, a.V, n_sm)) {
+    case 8: return launch_rows<8>(P, a.N, smem, status, stream);
+    case 4: return launch_rows<4>(P, a.N, smem, status, stream);
+    case 2: return launch_rows<2>(P, a.N, smem, status, stream);
+    default: return launch_rows<1>(P, a.N, smem, status, stream);
   }
-  return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
 }  // namespace

@@ -56,6 +56,22 @@ def test_score_shapes(N, V, n_seq, k):
     check(inp, run_score(inp), f"N{N} V{V}")
 
 
+@pytest.mark.parametrize("N,V", [
+    (5, 16387), (38, 20001),      # eight CTAs a row, the last slice short; the most rows on 152 SMs
+    (39, 20001), (76, 8193),      # four
+    (77, 65544), (152, 65537),    # two
+    (153, 65544),                 # one
+])
+def test_score_split_rows(N, V):
+    """Rows split over a cluster: sums and, with the maximum in several slices, its first index."""
+    inp = W.make_score_inputs(N, V, 1, 4, seed=V, with_cur_tok=True, spike_frac=0.3)
+    x = inp.logits
+    for r in range(0, N, 2):
+        x[r, [V // 9, V // 2, V - 1 - r % 7]] = W.f32_to_bf16_bits(np.full(3, 20.0, np.float32))
+    x[1, 0] = x[1, V - 1] = W.f32_to_bf16_bits(np.full(1, 21.0, np.float32))[0]
+    check(inp, run_score(inp), f"N{N} V{V}")
+
+
 def test_score_side_inputs_and_eligibility():
     inp = W.make_score_inputs(96, 5003, 3, 10, seed=7, with_cur_tok=True, with_dio=True, eligible_frac=0.4)
     check(inp, run_score(inp))
