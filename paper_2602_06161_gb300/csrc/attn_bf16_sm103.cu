@@ -54,7 +54,7 @@ constexpr int kD = 128;
 constexpr int kBM = 128;                  // rows per Q tile
 constexpr int kBN = 128;                  // keys per KV tile
 constexpr int kNQ = 2;                    // Q tiles per CTA
-constexpr int kRowsPerCta = kNQ * kBM;
+constexpr int kRowsPerCta = kNQ * kBM;    // rows a CTA has tables for
 constexpr int kStages = 2;
 constexpr int kTileBytes = kBM * kD * 2;  // 32 KB
 constexpr int kBoxBytes = kTileBytes / 2; // one 64-column, 128-byte-swizzled box
@@ -105,10 +105,12 @@ struct FastDiv {
 
 // The persistent grid's unit space: n_reg whole units, n_split split ones, and the divisors
 // that decompose a unit index (n_mblk row blocks per head, Hq heads) and map a query head to
-// its KV head (Hq / Hkv query heads per KV head).
+// its KV head (Hq / Hkv query heads per KV head). A window of grouped-query heads may be launched
+// packed: the G Lq rows of a KV head's query heads, contiguous in q and out, are then the rows of
+// one head, and row P of it sits at memory position q0 + P % period (period = Lq; else all rows).
 struct UnitGrid {
   int n_reg, n_split;
-  FastDiv mblk, hq, group;
+  FastDiv mblk, hq, group, period;
 };
 
 // Iteration it of this CTA. Units c, c + grid, ... below n_reg are whole units. When the
@@ -141,9 +143,10 @@ __device__ __forceinline__ bool work_of(int it, const UnitGrid& ug, Unit& w) {
   return true;
 }
 
-// first query row of Q tile t of a unit
+// first query row of Q tile t of a unit of kUnitRows rows
+template <int kUnitRows>
 __device__ __forceinline__ int tile_row0(const Unit& w, int t) {
-  return w.mblk * kRowsPerCta + (w.split ? w.ts : t) * kBM;
+  return w.mblk * kUnitRows + (w.split ? w.ts : t) * kBM;
 }
 
 struct AttnSmem {
@@ -200,8 +203,8 @@ __device__ __forceinline__ void raise_abort(AttnSmem& sm, int* status, int site)
   sm.abort = 1;
 }
 
-// NQ: Q tiles holding query rows (1 for a window of at most 128 rows, else 2).
-// kWindow: query row r sits at memory position q0 + r of an Lk-long memory;
+// NQ: Q tiles of a unit (1 or 2 for a window, 2 otherwise).
+// kWindow: query row r sits at memory position q0 + r % period of an Lk-long memory;
 // otherwise Lq = Lk and q0 = 0 are compile-time facts.
 // kFault: the self-test instance that takes its wait limit and a planted missing load from
 // `flt`; the production instances wait up to one second and load every tile.
@@ -221,12 +224,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = tid >> 5, lane = tid & 31;
   const int nkv = (Lk + kBN - 1) / kBN;
   constexpr int nqt = NQ;
+  constexpr int kUnitRows = NQ * kBM;
   const uint64_t wait_ns = kFault ? flt.wait_ns : kWaitLimitNs;
   const int Lq = kWindow ? Lq_arg : Lk;
   const int q0 = kWindow ? q0_arg : 0;
   const int tail_valid = Lk - (nkv - 1) * kBN;   // valid keys in the last KV tile (1..128)
-  // a window of at most 128 rows has one Q tile; with an even number of KV tiles its units are
-  // all split, so the second softmax warpgroup takes half of every unit's keys
+  // one-tile units of a window are all split when the number of KV tiles is even, so the second
+  // softmax warpgroup takes half of every unit's keys
   constexpr bool kSplitAll = kWindow && NQ == 1;
   const bool all_split = kSplitAll && ug.n_split > 0;
 
@@ -300,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int sig = (n * nkv + nkv - 1) & 1;
         const uint8_t* stage = t == 0 ? sm.k[sig] : sm.v[sig];
         for (int wq = 0; wq < 4; ++wq) {
-          const int wrow = tile_row0(wn, t) + wq * 32;
+          const int wrow = tile_row0<kUnitRows>(wn, t) + wq * 32;
           if (wrow < Lq) {   // rows at or past Lq fall outside the tensor and are not written
             tma_store_4d(&tm_o, stage + wq * 8192, 0, wrow, wn.hq, wn.b);
             tma_store_4d(&tm_o, stage + wq * 8192 + 4096, 64, wrow, wn.hq, wn.b);
@@ -322,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             return false;
           mbar_arrive_expect_tx(&sm.bar_q_full[t], kTileBytes);
           for (int h = 0; h < 2; ++h)
-            tma_load_4d(sm.q[t] + h * kBoxBytes, &tm_q, &sm.bar_q_full[t], 64 * h, tile_row0(w, t), w.hq, w.b);
+            tma_load_4d(sm.q[t] + h * kBoxBytes, &tm_q, &sm.bar_q_full[t], 64 * h, tile_row0<kUnitRows>(w, t), w.hq, w.b);
           last_qit[t] = it;
           return true;
         };
@@ -412,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           Unit wn;
           if (work_of<kSplitAll>(it + 1, ug, wn))
             for (int t = 0; t < (wn.split ? 1 : nqt); ++t)
-              for (int h = 0; h < 2; ++h) tma_prefetch_l2_4d(&tm_q, 64 * h, tile_row0(wn, t), wn.hq, wn.b);
+              for (int h = 0; h < 2; ++h) tma_prefetch_l2_4d(&tm_q, 64 * h, tile_row0<kUnitRows>(wn, t), wn.hq, wn.b);
         }
         ++G;
         if (nkv > 1) {
@@ -453,12 +457,23 @@ __global__ void __launch_bounds__(kThreads, 1)
         break;
       }
       if (lane == 0) sm.unit[sb] = w;
-      // slot[t * 128 + r] belongs to query row tile_row0(w, t) + r, at memory position q0 + that
-      const int rows = w.split ? kBM : kRowsPerCta;
+      // slot[t * 128 + r] belongs to query row tile_row0<kUnitRows>(w, t) + r, at memory position q0 + that
+      const int rows = w.split ? kBM : kUnitRows, row0 = tile_row0<kUnitRows>(w, 0);
+      const int32_t* seeds_b = seed_idx + static_cast<size_t>(w.b) * n_seeds;
       route_clear(sm.slot[sb], rows, lane, 32);
       __syncwarp();
-      route_scan(sm.slot[sb], seed_idx + static_cast<size_t>(w.b) * n_seeds, n_seeds, q0 + tile_row0(w, 0), rows,
-                 Lk, lane, 32);
+      if (kWindow) {
+        // the rows at a seed's position, one per packed head
+        const int period = static_cast<int>(ug.period.d), end = min(row0 + rows, Lq);
+        for (int sd = lane; sd < n_seeds; sd += 32) {
+          const int at = __ldg(seeds_b + sd) - q0;
+          if (at < 0 || at >= period) continue;
+          for (int P = at; P < end; P += period)
+            if (P >= row0) atomicMin(sm.slot[sb] + (P - row0), sd);
+        }
+      } else {
+        route_scan(sm.slot[sb], seeds_b, n_seeds, row0, rows, Lk, lane, 32);
+      }
       if (w.split) {
         // both warpgroups of a split unit work on the same rows
         __syncwarp();
@@ -495,7 +510,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int rc = 0; rc < kBM; rc += 32) {
           const int rr = rc + lane;
           const int sl = sm.slot[sb][t * kBM + rr];
-          const bool seed_row = sl != kNoSlot && tile_row0(w, t) + rr < Lq;
+          const bool seed_row = sl != kNoSlot && tile_row0<kUnitRows>(w, t) + rr < Lq;
           uint32_t pending = __ballot_sync(0xffffffffu, seed_row);
           while (pending != 0u) {
             // up to four seed rows at a time, their loads in flight together
@@ -731,21 +746,26 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = warp_wait(&sm.bar_slot_full[sb], (it >> 1) & 1, &sm.abort, wait_ns);
           if (!ok) break;
           const Unit w = sm.unit[sb];
-          const int grow = tile_row0(w, qt) + r;
+          const int grow = tile_row0<kUnitRows>(w, qt) + r;
           const int jbase = w.split ? qt * (nkv >> 1) : 0;
           steps = w.split ? nkv >> 1 : nkv;
           tail_j = tail_valid < kBN ? nkv - 1 - jbase : -1;   // -1: no ragged tile
           my_slot = sm.slot[sb][qt * kBM + r];
           if (grow >= Lq) my_slot = kNoSlot;
-          // the diagonal of a square launch is column r of KV tile row0 / 128 of the row's Q tile;
-          // in a window a warp's 32 consecutive rows meet their diagonals in at most two KV tiles
-          diag_j = (kWindow ? (q0 + grow) / kBN : tile_row0(w, qt) / kBN) - jbase;
-          diag_c = kWindow ? (q0 + grow) % kBN : r;
+          // the diagonal of a square launch is column r of KV tile row0 / 128 of the row's Q tile
+          int pos = 0;
+          if (kWindow) {
+            const uint32_t P = static_cast<uint32_t>(grow);
+            pos = q0 + static_cast<int>(P - ug.period.div(P) * ug.period.d);
+          }
+          diag_j = (kWindow ? pos / kBN : tile_row0<kUnitRows>(w, qt) / kBN) - jbase;
+          diag_c = kWindow ? pos % kBN : r;
         }
         const bool is_seed = my_slot != kNoSlot;
         const bool warp_seed = __any_sync(0xffffffffu, is_seed);
-        const int dj_lo = kWindow ? __shfl_sync(0xffffffffu, diag_j, 0) : diag_j;
-        const int dj_hi = kWindow ? __shfl_sync(0xffffffffu, diag_j, 31) : diag_j;
+        // in a window: the KV steps that hold the diagonals of the warp's seed rows (none: lo > hi)
+        const int dj_lo = kWindow ? __reduce_min_sync(0xffffffffu, is_seed ? diag_j : 0x7fffffff) : diag_j;
+        const int dj_hi = kWindow ? __reduce_max_sync(0xffffffffu, is_seed ? diag_j : -0x7fffffff) : diag_j;
         const int g0 = it * nkv;   // the CTA's KV steps before this unit
         // this warpgroup's steps before this unit (half a unit's KV tiles each when all are split)
         const int sbase = all_split ? it * (nkv >> 1) : g0;
@@ -767,7 +787,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int c = 0; c < kBN; ++c)
               if (c >= valid) s[c] = -INFINITY;
           }
-          if (warp_seed && (j == dj_lo || j == dj_hi)) {
+          if (kWindow ? j >= dj_lo && j <= dj_hi : warp_seed && j == diag_j) {
             // exclusion of the cached diagonal term of a seed row
             const bool here = is_seed && j == diag_j;
             if (!kWindow) {
@@ -876,7 +896,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int e = 0; e < 32; ++e) oh[32 * c + e] = __uint_as_float(x0[e]) * a0 + __uint_as_float(x1[e]) * a1;
           }
-          const int grow = tile_row0(w, 0) + r;
+          const int grow = tile_row0<kUnitRows>(w, 0) + r;
           if (is_seed) {
             const float s_self = sm.sself[sb][r];
             const int vi = sm.vidx[sb][r];
@@ -950,7 +970,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int c = 0; c < 4; ++c) tmem_ld_wait(oraw[c]);
         float* o = reinterpret_cast<float*>(&oraw[0][0]);
-        const int grow = tile_row0(w, qt) + r;
+        const int grow = tile_row0<kUnitRows>(w, qt) + r;
         if (warp_seed) {
           ok = warp_wait(&sm.bar_sself_full[sb], (it >> 1) & 1, &sm.abort, wait_ns);
           if (!ok) break;
@@ -1052,26 +1072,91 @@ FastDiv make_fastdiv(uint32_t d) {
 
 }  // namespace
 
-int launch_attn_bf16_sm103(const AttnArgs& a, int* status, cudaStream_t stream) {
+namespace {
+
+// Units, split or not, of a window launch: `pack` query heads in common Q tiles, nq Q tiles a unit.
+struct WindowPlan {
+  bool pack;
+  int nq;
+  double us;
+};
+
+// The cheapest of the four plans by a launch-time model. A unit takes about 1.7 us per KV step of a
+// softmax warpgroup (half of the KV tiles in a one-tile unit, whose keys its two warpgroups split;
+// that takes an even number of tiles, and an odd one keeps the square launch's bits) and 2 us
+// around them, and the persistent grid runs rounds of n_sm units. On equal cost the units stay
+// unpacked, whose rows spread over more SMs. us measured, unpacked with one / two tiles a unit and
+// packed with one / two (B, heads, keys, rows):
+//   8, 32/8, 2048, 64:  38.7 / 61.3 / 21.5 / 33.0    12, 32/8, 2000, 17: 55.4 / 88.3 / 21.9 / 35.3
+//   8, 28/4, 1024, 32:  23.5 / 35.4 / 13.1 / 19.2    6, 28/4, 1500, 100: 30.6 / 47.4 / 18.1 / 26.1
+//   4, 28/4, 1024, 32:  13.0 / 19.5 / 13.0 / 19.3    8, 32/8, 1100, 64:  34.7 / 41.8 / 20.0 / 22.2
+//   2, 32/32, 2048, 200: 21.1 / 32.9                 3, 32/32, 2048, 200: 38.7 / 36.6
+// (before, a window was unpacked, with one tile a unit up to 128 rows and two above).
+WindowPlan plan_window(const AttnArgs& a, int n_sm) {
+  const int G = a.Hq / a.Hkv, nkv = (a.L + kBN - 1) / kBN;
+  const bool even = nkv % 2 == 0;
+  WindowPlan best{false, a.Lq <= kBM ? 1 : 2, 0.0};
+  const auto us = [&](bool pack, int nq) {
+    const long long rows = pack ? static_cast<long long>(G) * a.Lq : a.Lq;
+    const long long units = (rows + nq * kBM - 1) / (nq * kBM) * a.B * (pack ? a.Hkv : a.Hq);
+    const int steps = nq == 1 && even ? nkv / 2 : nkv;
+    return static_cast<double>((units + n_sm - 1) / n_sm) * (2.0 + 1.7 * steps) + 3.0;
+  };
+  best.us = us(best.pack, best.nq);
+  const auto consider = [&](bool pack, int nq) {
+    const double t = us(pack, nq);
+    if (t < best.us) best = WindowPlan{pack, nq, t};
+  };
+  if (even || a.Lq <= kBM) consider(false, 1);
+  consider(false, 2);
+  if (G > 1 && static_cast<long long>(G) * a.Lq <= 0x7fffffffLL / 2) {
+    consider(true, 2);
+    consider(true, 1);
+  }
+  return best;
+}
+
+}  // namespace
+
+double window_square_us(const AttnArgs& a, int n_sm) { return plan_window(a, n_sm).us; }
+
+int launch_attn_bf16_sm103(const AttnArgs& args, int* status, cudaStream_t stream) {
+  static ContextCache<int> sms;
+  int n_sm = 0;
+  const int rc_sm = sms.get(&n_sm, [](int& v) {
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+                   cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v >= 1 ? 0 : -3;
+  });
+  if (rc_sm != 0) return rc_sm;
+  AttnArgs a = args;
+  const bool window = a.Lq != a.L || a.q0 != 0;
+  const int period = a.Lq;
+  int nq = kNQ;
+  if (window) {
+    const WindowPlan plan = plan_window(a, n_sm);
+    nq = plan.nq;
+    if (plan.pack) {
+      // the query heads of a KV head as the rows of one head
+      a.Lq *= a.Hq / a.Hkv;
+      a.Hq = a.Hkv;
+    }
+  }
   CUtensorMap tq, tk, tv, to;
   if (!make_bf16_map_4d(&tq, a.q, kD, a.Lq, a.Hq, a.B, kBM) ||
       !make_bf16_map_4d(&to, a.out, kD, a.Lq, a.Hq, a.B, 32) ||
       !make_bf16_map_4d(&tk, a.k_cached, kD, a.L, a.Hkv, a.B, kBN) ||
       !make_bf16_map_4d(&tv, a.v_cached, kD, a.L, a.Hkv, a.B, kBN))
     return -3;
-  const int n_mblk = (a.Lq + kRowsPerCta - 1) / kRowsPerCta;
+  const int n_mblk = (a.Lq + nq * kBM - 1) / (nq * kBM);
   const long long n_units = static_cast<long long>(n_mblk) * a.Hq * a.B;
   const int nkv = (a.L + kBN - 1) / kBN;
   const size_t smem = sizeof(AttnSmem) + 1024;
-  // per context: the SM count, and the kernels' shared-memory limit set (a function attribute
-  // holds only in the context it was set in)
+  // per context: the kernels' shared-memory limit set (a function attribute holds only in the
+  // context it was set in)
   static ContextCache<int> setup;
-  int n_sm = 0;
-  const int rc = setup.get(&n_sm, [&](int& v) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
-      return -3;
+  int unused = 0;
+  const int rc = setup.get(&unused, [&](int&) {
     for (auto fn : {attn_bf16_kernel<2, false, false>, attn_bf16_kernel<1, true, false>,
                     attn_bf16_kernel<2, true, false>, attn_bf16_kernel<2, false, true>,
                     attn_bf16_kernel<1, true, true>, attn_bf16_kernel<2, true, true>}) {
@@ -1091,10 +1176,9 @@ int launch_attn_bf16_sm103(const AttnArgs& a, int* status, cudaStream_t stream) 
   // The last round of units would leave at least half of the SMs idle: split its units
   // (square launches with an even number of KV tiles), two CTAs per unit.
   const long long rounds = n_units / n_sm, n_last = n_units % n_sm;
-  const bool window = a.Lq != a.L || a.q0 != 0;
-  // A window of at most 128 rows has one Q tile per unit; with an even number of KV tiles every
-  // unit is split inside its CTA (both softmax warpgroups on the two halves of the keys).
-  const bool split_all = window && a.Lq <= kBM && nkv >= 2 && nkv % 2 == 0;
+  // One-tile units of a window are split inside their CTAs when the number of KV tiles is even
+  // (both softmax warpgroups on the two halves of the keys).
+  const bool split_all = nq == 1 && nkv % 2 == 0;
   const int n_split = split_all ? static_cast<int>(n_units)
                       : (!window && nkv >= 2 && nkv % 2 == 0 && n_last > 0 && 2 * n_last <= n_sm)
                           ? static_cast<int>(n_last) : 0;
@@ -1103,10 +1187,11 @@ int launch_attn_bf16_sm103(const AttnArgs& a, int* status, cudaStream_t stream) 
                                    : (rounds > 0 ? n_sm : (n_split > 0 ? 2 * n_split : n_units));
   const float scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(kD));
   const UnitGrid ug{n_reg, n_split, make_fastdiv(static_cast<uint32_t>(n_mblk)),
-                    make_fastdiv(static_cast<uint32_t>(a.Hq)), make_fastdiv(static_cast<uint32_t>(a.Hq / a.Hkv))};
+                    make_fastdiv(static_cast<uint32_t>(a.Hq)), make_fastdiv(static_cast<uint32_t>(a.Hq / a.Hkv)),
+                    make_fastdiv(static_cast<uint32_t>(period))};
   const bool fault = a.fault_cta >= 0 || a.wait_ns > 0;
   auto kernel = !window       ? (fault ? attn_bf16_kernel<2, false, true> : attn_bf16_kernel<2, false, false>)
-                : a.Lq <= kBM ? (fault ? attn_bf16_kernel<1, true, true> : attn_bf16_kernel<1, true, false>)
+                : nq == 1     ? (fault ? attn_bf16_kernel<1, true, true> : attn_bf16_kernel<1, true, false>)
                               : (fault ? attn_bf16_kernel<2, true, true> : attn_bf16_kernel<2, true, false>);
   // programmatic dependent launch: the prologue overlaps the previous kernel's tail
   cudaLaunchAttribute attr[1];

@@ -643,24 +643,14 @@ int win_setup(WinSetup* out, size_t smem) {
   });
 }
 
-// Predicted microseconds of one call on each kernel, fitted to calls measured back to back on
+// Predicted microseconds of one call, fitted to calls measured back to back on
 // GB300 (Dream-shaped windows of 16 to 128 rows over 1024 keys, batches of 1 to 8, memories of
 // 2048 to 8192 keys; within 15 % on every shape measured): a packed CTA takes about 7 us plus
-// 1.5 us per KV step, and the clusters beyond those resident at once run in further waves; the
-// square kernel's window path takes about 5 us plus 1.7 us per KV step of one softmax warpgroup
-// for each round of its persistent grid.
+// 1.5 us per KV step, and the clusters beyond those resident at once run in further waves (the
+// square kernel's prediction: window_square_us).
 double packed_us(const WinShape& w, const WinSetup& su) {
   const long long waves = (w.clusters + su.max_clusters[w.nsplit] - 1) / su.max_clusters[w.nsplit];
   return static_cast<double>(waves) * (7.0 + 1.5 * w.T);
-}
-
-double square_us(const AttnArgs& a, const WinShape& w, const WinSetup& su) {
-  const long long units = static_cast<long long>((a.Lq + 255) / 256) * a.Hq * a.B;
-  const long long rounds = (units + su.n_sm - 1) / su.n_sm;
-  // a window of at most 128 rows with an even number of KV tiles splits each unit's keys over
-  // the two softmax warpgroups
-  const int steps = (a.Lq <= kBM && w.nkv % 2 == 0) ? w.nkv / 2 : w.nkv;
-  return 5.0 + static_cast<double>(rounds) * steps * 1.7;
 }
 
 bool packed_supported(const AttnArgs& a) {
@@ -690,7 +680,7 @@ WindowChoice window_gqa_model(const AttnArgs& a, int n_sm, const int* max_cluste
   // a cluster of nsplit CTAs that cannot be resident leaves only the square kernel
   c.resident = su.max_clusters[w.nsplit] >= 1;
   c.packed_us = c.resident ? packed_us(w, su) : 0.0;
-  c.square_us = square_us(a, w, su);
+  c.square_us = window_square_us(a, n_sm);
   c.packed = c.resident && c.packed_us < c.square_us;
   return c;
 }

@@ -29,6 +29,8 @@ struct AttnArgs {
 };
 
 int launch_attn_bf16_sm103(const AttnArgs& a, int* status, cudaStream_t stream);
+// Predicted microseconds of a window on it, on a GPU with n_sm SMs (host arithmetic).
+double window_square_us(const AttnArgs& a, int n_sm);
 
 // Prefix-cache windows of grouped-query heads (attn_window_gqa.cu): the G = Hq / Hkv query heads
 // of a KV head packed into common Q tiles, the keys split over a cluster of up to 8 CTAs.

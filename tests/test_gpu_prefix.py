@@ -62,6 +62,29 @@ def test_window_bf16(B, Hq, Hkv, Lk, Lq, q0, S, inside):
     assert np.abs(lse - ref_lse).max() <= H.TOL_LSE
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,Lk,Lq,q0,S,inside", [
+    (5, 32, 8, 512, 64, 400, 12, 6),        # 160 units in two rounds unpacked: packed, 256 rows in one-tile units
+    (5, 32, 8, 500, 45, 411, 12, 8),        # 180 packed rows: a tile and a ragged one, heads meeting in a warp
+    (6, 28, 4, 640, 33, 97, 10, 6),         # an odd number of KV tiles: packed without a split
+    (9, 24, 3, 256, 3, 251, 5, 2),          # 24 packed rows, several heads of a position in one warp
+    (20, 16, 2, 130, 1, 64, 3, 1),          # one row per head; 40 packed units against 320
+    (1, 3, 3, 512, 200, 250, 8, 5),         # MHA: one-tile split units of a window above 128 rows
+    (2, 4, 4, 768, 256, 512, 9, 9),         # the same, every tile full
+])
+def test_window_plans(B, Hq, Hkv, Lk, Lq, q0, S, inside):
+    """The launch plans of a window: packed grouped-query heads, one-tile units beyond 128 rows."""
+    q, kc, vc, km, vm, seeds = _case(B, Hq, Hkv, Lk, 128, S, q0, Lq, "bf16", Lk + Lq, inside)
+    dev = [H.to_dev(np.ascontiguousarray(q[:, :, q0:q0 + Lq]), "bf16"), H.to_dev(kc, "bf16"), H.to_dev(vc, "bf16"),
+           H.to_dev(km, "bf16"), H.to_dev(vm, "bf16"), H.to_dev(seeds, "i32")]
+    # the fault entry with nothing planted: this kernel whichever one the window call would take
+    out, lse = api.cover_debug_attn_fault(*dev, q0=q0, fault_cta=-1, fault_entry=-1, limit_us=1000000)
+    torch.cuda.synchronize()
+    assert api.cover_device_status() == 0
+    f = W.bf16_bits_to_f64
+    ref, ref_lse = oracle.override_attention_window(f(q[:, :, q0:q0 + Lq]), f(kc), f(vc), f(km), f(vm), seeds, q0)
+    H.assert_bf16_close(out.float().cpu().numpy(), ref, lse.cpu().numpy(), ref_lse)
+
+
 @pytest.mark.parametrize("D,Lk,Lq,q0", [(64, 100, 30, 70), (128, 77, 20, 3)])
 def test_window_f32(D, Lk, Lq, q0):
     q, kc, vc, km, vm, seeds = _case(2, 4, 2, Lk, D, 6, q0, Lq, "f32", D + Lk, 3)
