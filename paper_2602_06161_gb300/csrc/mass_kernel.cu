@@ -12,25 +12,33 @@
 // keys contribute, so the pass covers a per x per block of each head.
 //
 // Both sums become row sums held in registers by computing the block twice on
-// the tensor cores, once per orientation, in two kinds of CTA per (b, hq, tile):
-//   rows CTA    S  = Q_t K_j^T for every key tile j: thread = query row of tile
-//               t, sums its weights over the drafted keys (d_out partial);
-//   columns CTA S' = K_t Q_j^T for every query tile j: thread = key of tile t,
-//               sums exp(s - lse(q)) over the masked queries q, whose lse is
-//               staged per column in shared memory (+inf for a query that is
-//               not masked, so its weight is exactly 0) (d_in partial).
-// The resident tile (Q_t or K_t) is loaded once; the other operand streams
-// through a two-stage ring, and S double-buffers in tensor memory so a tile's
-// product overlaps the previous tile's exponentials. A 32-column chunk with no
-// drafted key (rows) or no masked query (columns) is skipped as a whole (its
-// predicate is the same for every thread). Each CTA writes one partial per
-// row of its tile; a second kernel adds the partials of the Hq heads in a
-// fixed order (deterministic) and divides by the head count.
+// the tensor cores, once per orientation, in 128 x 128 tiles:
+//   row product     S  = Q_t K_j^T: thread = query row of tile t, sums its weights
+//                   over the drafted keys of tile j (d_out partial);
+//   column product  S' = K_t Q_j^T: thread = key of tile t, sums exp(s - lse(q)) over
+//                   the masked queries q of tile j, whose lse is staged per column
+//                   in shared memory (negated; -inf for a query that is not masked,
+//                   so its weight is exactly 0) (d_in partial).
+// A product whose tile j has no drafted key (rows) or no masked query (columns) is left out, and
+// a 32-column chunk without one is skipped, as is a group of four keys without a drafted one (a step
+// drafts few; the predicates are the same for every thread). Each CTA writes one partial per row of
+// its tiles; a second kernel adds the partials of the Hq heads in a fixed order (deterministic) and
+// divides by the head count.
 //
-// Warps: 0-3 rows / keys of the tile (thread = tensor-memory lane), 4 issues
-// the TMA loads (lane 0), 5 allocates tensor memory and issues the products
-// (lane 0). About 100 KB of shared memory and 256 tensor-memory columns per CTA,
-// so two CTAs share an SM.
+// A CTA keeps Q_t and K_t of NT tiles of one head resident: they serve as the A operands of both
+// orientations and as the B operands of the products among themselves; the block's other tiles
+// stream through a two-slot ring. Each of the two warpgroups of the math threads takes the products
+// of one tile (NT = 2) or of one orientation (NT = 1) from two tensor-memory buffers, so a product
+// overlaps the previous one's exponentials.
+//
+// Bound: latency and, with many heads, reading Q and K once (8 x 32 heads x 256 rows: 34 MB, 5 us).
+// With NT = 2 a head's 256-row block is one CTA that reads it once, instead of four CTAs (one per
+// tile and orientation) reading three tiles each: 29.1 -> 19.4 us there (both launches), 16.6 ->
+// 10.2 us with 4 x 32 heads. What is left is a CTA's chain (column data, tile loads, four products
+// and their exponentials, about 8 us) in ceil(CTAs / SMs) waves.
+//
+// Warps: 0-7 rows / keys of the tiles (thread = tensor-memory lane), 8 issues the TMA loads (lane
+// 0), 9 allocates tensor memory and issues the products (lane 0).
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -45,47 +53,46 @@ namespace {
 
 constexpr int kD = 128;
 constexpr int kT = 128;                     // rows / keys per tile
-constexpr int kThreads = 192;
-constexpr int kMathThreads = 128;
-constexpr int kTmaWarp = 4;
-constexpr int kMmaWarp = 5;
+constexpr int kMathThreads = 256;           // two warpgroups
+constexpr int kTmaWarp = 8;
+constexpr int kMmaWarp = 9;
+constexpr int kThreads = 320;
 constexpr int kTileBytes = kT * kD * 2;     // 32 KB
 constexpr int kBoxBytes = kTileBytes / 2;   // one 64-column, 128-byte-swizzled box
 constexpr int kMaxPer = kMassMaxPer;        // per-column staging must fit in shared memory
+constexpr int kSlots = 2;                   // ring slots of the streamed tiles
+constexpr int kMaxTilesPair = 32;           // tiles of a block up to which two are resident
 
-// 128-byte aligned, so the per-column arrays that follow it start 16-byte aligned (float4 reads)
-struct alignas(128) MassSmem {
-  uint8_t x[kTileBytes];                    // resident operand: Q_t (rows) or K_t (columns)
-  uint8_t y[2][kTileBytes];                 // streamed operand: K_j (rows) or Q_j (columns)
-  uint64_t bar_x;
-  uint64_t bar_y_full[2];
-  uint64_t bar_y_empty[2];
-  uint64_t bar_s_full[2];
-  uint64_t bar_s_empty[2];
+struct alignas(128) MassCtrl {
+  uint64_t bar_q[2], bar_k[2];              // resident Q / K tile has landed
+  uint64_t bar_ring_full[kSlots], bar_ring_empty[kSlots];
+  uint64_t bar_s_full[2][2];                // [warpgroup][buffer]
+  uint64_t bar_s_empty[2][2];
   uint64_t bar_drain;
   uint32_t tmem_base;
   int abort;
-  int slot[kT];                             // seed slot of the resident tile's positions
-  // followed by the per-column data of the whole block (dynamic size):
-  //   uint32_t bits[n_t * 4]  drafted keys (rows) / masked queries (columns)
-  //   float colv[n_t * 128]   columns: log2-scaled lse of a masked query, else +inf
+  int slot[2 * kT];                         // seed slot of the resident tiles' positions
 };
 
-static_assert(sizeof(MassSmem) % 16 == 0, "per-column arrays must start 16-byte aligned");
-
-__device__ __forceinline__ uint32_t* col_bits(MassSmem& sm) { return reinterpret_cast<uint32_t*>(&sm + 1); }
-__device__ __forceinline__ float* col_vals(MassSmem& sm, int n_t) {
-  return reinterpret_cast<float*>(col_bits(sm) + n_t * 4);
+// Shared memory: NT Q tiles | NT K tiles | kSlots ring slots (when the block has more than NT tiles) |
+// MassCtrl | per-column data of the whole block:
+//   uint32_t bits[2][n_t * 4]  drafted keys, masked queries
+//   float colv[n_t * 128]      the negated log2-scaled lse of a masked query, else -inf
+size_t mass_smem_bytes(int NT, int n_t) {
+  return static_cast<size_t>(2 * NT + (n_t > NT ? kSlots : 0)) * kTileBytes + sizeof(MassCtrl) +
+         static_cast<size_t>(n_t) * (8 * sizeof(uint32_t) + kT * sizeof(float)) + 1024;
 }
 
-// q_row . k_row over the 128 dimensions, both bf16 rows in global memory.
-__device__ __forceinline__ float dot_row(const __nv_bfloat16* qrow, const __nv_bfloat16* krow) {
-  const uint4* qv = reinterpret_cast<const uint4*>(qrow);
+// q . k over the 128 dimensions: q is row r of a 128-byte-swizzled tile in shared memory, k a row
+// in global memory.
+__device__ __forceinline__ float dot_row(const uint8_t* qtile, int r, const __nv_bfloat16* krow) {
   const uint4* kv = reinterpret_cast<const uint4*>(krow);
   float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
   for (int ch = 0; ch < 16; ++ch) {
-    const uint4 a = __ldg(qv + ch), b = __ldg(kv + ch);
+    const uint4 a = *reinterpret_cast<const uint4*>(qtile + (ch >> 3) * kBoxBytes + r * 128 +
+                                                    (((ch & 7) ^ (r & 7)) << 4));
+    const uint4 b = __ldg(kv + ch);
     const __nv_bfloat162* ap = reinterpret_cast<const __nv_bfloat162*>(&a);
     const __nv_bfloat162* bp = reinterpret_cast<const __nv_bfloat162*>(&b);
 #pragma unroll
@@ -98,95 +105,119 @@ __device__ __forceinline__ float dot_row(const __nv_bfloat16* qrow, const __nv_b
   return (d[0] + d[1]) + (d[2] + d[3]);
 }
 
-// blockIdx.x = (b * Hq + hq) * n_t + t; blockIdx.y = 0 rows CTA, 1 columns CTA.
-__global__ void __launch_bounds__(kThreads, 2)
+// blockIdx.x = (b * Hq + hq) * n_g + g: tiles NT g .. of head (b, hq).
+template <int NT>
+__global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
     mass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k_seedmask,
-                const int32_t* __restrict__ seed_idx, int n_seeds, const float* __restrict__ lse, int Hq, int Hkv,
-                int L, int pos0, int per, int n_t, const int32_t* __restrict__ tok, const uint8_t* __restrict__ flags,
-                int mask_id, float scale_log2, float* __restrict__ part_in, float* __restrict__ part_out,
-                int* status) {
+                const __nv_bfloat16* __restrict__ k_seedmask, const int32_t* __restrict__ seed_idx, int n_seeds,
+                const float* __restrict__ lse, int Hq, int Hkv, int L, int pos0, int per, int n_t, int n_g,
+                const int32_t* __restrict__ tok, const uint8_t* __restrict__ flags, int mask_id, float scale_log2,
+                float* __restrict__ part_in, float* __restrict__ part_out, int* status) {
   extern __shared__ uint8_t smem_raw[];
-  MassSmem& sm = *reinterpret_cast<MassSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* const base =
+      reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* const xq = base;
+  uint8_t* const xk = base + NT * kTileBytes;
+  uint8_t* const ring = base + 2 * NT * kTileBytes;
+  MassCtrl& sm = *reinterpret_cast<MassCtrl*>(ring + (n_t > NT ? kSlots * kTileBytes : 0));
+  uint32_t* const bits = reinterpret_cast<uint32_t*>(&sm + 1);   // [kind][n_t * 4]
+  float* const colv = reinterpret_cast<float*>(bits + 8 * n_t);
 
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
-  const bool cols = blockIdx.y != 0;
-  const int t = static_cast<int>(blockIdx.x) % n_t;
-  const int bh = static_cast<int>(blockIdx.x) / n_t;   // b * Hq + hq
+  const int bh = static_cast<int>(blockIdx.x) / n_g;   // b * Hq + hq
+  const int t0 = (static_cast<int>(blockIdx.x) - bh * n_g) * NT;
+  const int nw = min(NT, n_t - t0);                    // resident tiles
   const int hq = bh % Hq, b = bh / Hq;
   const int hkv = hq / (Hq / Hkv);
-  uint32_t* bits = col_bits(sm);
-  float* colv = col_vals(sm, n_t);
-  // launched as a programmatic dependent of the stream's previous kernel: wait for its results;
-  // the reduction kernel behind this one may be scheduled now, it waits for this grid's results
-  griddep_wait();
-  griddep_launch_dependents();
+  // tensor-memory buffers of a warpgroup (one for a one-tile block, so that two CTAs share an SM)
+  const int nbuf = n_t == 1 ? 1 : 2;
+  const uint32_t tmem_cols = 2u * static_cast<uint32_t>(nbuf) * kT;
+  // the block's tiles in the order they are taken: the resident ones first
+  auto tile_of = [&](int jj) {
+    if (jj < nw) return t0 + jj;
+    const int o = jj - nw;
+    return o < t0 ? o : o + nw;
+  };
+  // whether tile j has a drafted key (kind 0, row products) / a masked query (kind 1, column products)
+  auto needed = [&](int kind, int j) {
+    const uint4 w = reinterpret_cast<const uint4*>(bits + kind * 4 * n_t)[j];
+    return (w.x | w.y | w.z | w.w) != 0u;
+  };
 
-  const CUtensorMap* tm_x = cols ? &tm_k : &tm_q;
-  const CUtensorMap* tm_y = cols ? &tm_q : &tm_k;
-  const int hx = cols ? hkv : hq, hy = cols ? hq : hkv;
   if (warp == kTmaWarp && lane == 0) {
-    // the TMA thread initialises the barriers and issues the resident tile and the first two
-    // streamed tiles at once, so their latency overlaps the rest of the prologue
-    mbar_init(&sm.bar_x, 1);
     for (int s = 0; s < 2; ++s) {
-      mbar_init(&sm.bar_y_full[s], 1);
-      mbar_init(&sm.bar_y_empty[s], 1);
-      mbar_init(&sm.bar_s_full[s], 1);
-      mbar_init(&sm.bar_s_empty[s], kMathThreads / 32);
+      mbar_init(&sm.bar_q[s], 1);
+      mbar_init(&sm.bar_k[s], 1);
+      mbar_init(&sm.bar_ring_full[s], 1);
+      mbar_init(&sm.bar_ring_empty[s], 1);
+      for (int u = 0; u < 2; ++u) {
+        mbar_init(&sm.bar_s_full[s][u], 1);
+        mbar_init(&sm.bar_s_empty[s][u], 4);
+      }
     }
     mbar_init(&sm.bar_drain, 1);
     sm.abort = 0;
     fence_mbar_init();
-    tma_prefetch_desc(tm_x);
-    tma_prefetch_desc(tm_y);
-    mbar_arrive_expect_tx(&sm.bar_x, kTileBytes);
-    for (int h = 0; h < 2; ++h) tma_load_4d(sm.x + h * kBoxBytes, tm_x, &sm.bar_x, 64 * h, pos0 + t * kT, hx, b);
-    for (int j = 0; j < 2 && j < n_t; ++j) {
-      mbar_arrive_expect_tx(&sm.bar_y_full[j], kTileBytes);
-      for (int h = 0; h < 2; ++h)
-        tma_load_4d(sm.y[j] + h * kBoxBytes, tm_y, &sm.bar_y_full[j], 64 * h, pos0 + j * kT, hy, b);
-    }
+    tma_prefetch_desc(&tm_q);
+    tma_prefetch_desc(&tm_k);
   }
   if (warp == kMmaWarp) {
-    tmem_alloc(&sm.tmem_base, 256);
+    tmem_alloc(&sm.tmem_base, tmem_cols);
     tmem_relinquish();
   }
-  route_clear(sm.slot, kT, tid, kThreads);
+  route_clear(sm.slot, 2 * kT, tid, kThreads);
+  // launched as a programmatic dependent of the stream's previous kernel: wait for its results;
+  // the reduction kernel behind this one may be scheduled now, it waits for this grid's results
+  griddep_wait();
+  griddep_launch_dependents();
+  if (warp == kTmaWarp && lane == 0) {
+    // the resident tiles are issued at once, so their latency overlaps the rest of the prologue
+    for (int w = 0; w < nw; ++w)
+      for (int kind = 0; kind < 2; ++kind) {
+        uint64_t* bar = kind == 0 ? &sm.bar_q[w] : &sm.bar_k[w];
+        mbar_arrive_expect_tx(bar, kTileBytes);
+        for (int h = 0; h < 2; ++h)
+          tma_load_4d((kind == 0 ? xq : xk) + w * kTileBytes + h * kBoxBytes, kind == 0 ? &tm_q : &tm_k, bar, 64 * h,
+                      pos0 + (t0 + w) * kT, kind == 0 ? hq : hkv, b);
+      }
+  }
   // the first seed entry of this thread, loaded now so that its latency overlaps the column data's
   const int32_t* seeds_b = seed_idx + static_cast<size_t>(b) * n_seeds;
   const int seed0 = tid < n_seeds ? __ldg(seeds_b + tid) : -1;
-  // rows CTAs: the log2-scaled lse of the thread's own query (thread = row of the tile)
-  float own = 0.0f;
-  if (!cols && tid < kMathThreads && t * kT + tid < per)
-    own = lse[static_cast<size_t>(bh) * L + pos0 + t * kT + tid] * 1.4426950408889634f;
-  // per-column data of the whole block: rows CTAs need the drafted keys, columns CTAs the masked
-  // queries and their lse; one warp per 32 columns
+  // per-column data of the whole block: the drafted keys, the masked queries and their lse; one
+  // warp per 32 columns
   for (int w = warp; w < n_t * 4; w += kThreads / 32) {
     const int c = w * 32 + lane;
     const bool in = c < per;
     const size_t srow = static_cast<size_t>(b) * per + c;
-    bool on;
-    if (!cols) {
-      on = in && (flags[srow] & 2u) != 0;
-    } else {
-      on = in && tok[srow] == mask_id;
-      colv[c] = on ? lse[static_cast<size_t>(bh) * L + pos0 + c] * 1.4426950408889634f : INFINITY;
+    const bool drafted = in && (flags[srow] & 2u) != 0;
+    const bool masked = in && tok[srow] == mask_id;
+    const float l2 = in ? lse[static_cast<size_t>(bh) * L + pos0 + c] * 1.4426950408889634f : 0.0f;
+    colv[c] = masked ? -l2 : -INFINITY;
+    const uint32_t d = __ballot_sync(0xffffffffu, drafted), m = __ballot_sync(0xffffffffu, masked);
+    if (lane == 0) {
+      bits[w] = d;
+      bits[4 * n_t + w] = m;
     }
-    const uint32_t word = __ballot_sync(0xffffffffu, on);
-    if (lane == 0) bits[w] = word;
   }
+  // the log2-scaled lse of a math thread's own query (thread = row of its tile)
+  const int g = (warp >> 2) & 1;                       // warpgroup
+  const int my = NT == 2 ? g : 0;                      // its resident tile
+  const int r = tid & (kT - 1);                        // tensor-memory lane
+  const int i = (t0 + my) * kT + r;                    // response index of this thread's query / key
+  const bool valid = warp < kMathThreads / 32 && my < nw && i < per;
+  const float own = valid ? lse[static_cast<size_t>(bh) * L + pos0 + i] * 1.4426950408889634f : 0.0f;
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   {
-    // seed routing of the resident tile's positions (the lowest slot naming a position wins)
-    const int row0 = pos0 + t * kT;
-    if (seed0 >= row0 && seed0 < row0 + kT && seed0 < L) atomicMin(sm.slot + (seed0 - row0), tid);
+    // seed routing of the resident tiles' positions (the lowest slot naming a position wins)
+    const int row0 = pos0 + t0 * kT, rows = nw * kT;
+    if (seed0 >= row0 && seed0 < row0 + rows && seed0 < L) atomicMin(sm.slot + (seed0 - row0), tid);
     for (int sidx = tid + kThreads; sidx < n_seeds; sidx += kThreads) {
       const int p = __ldg(seeds_b + sidx);
-      if (p >= row0 && p < row0 + kT && p < L) atomicMin(sm.slot + (p - row0), sidx);
+      if (p >= row0 && p < row0 + rows && p < L) atomicMin(sm.slot + (p - row0), sidx);
     }
   }
   __syncthreads();
@@ -194,49 +225,80 @@ __global__ void __launch_bounds__(kThreads, 2)
 
   if (warp == kTmaWarp) {
     if (lane == 0) {
-      int last = min(n_t, 2) - 1;
+      int n = 0;   // tiles streamed so far
       bool ok = true;
-      for (int j = 2; j < n_t; ++j) {
-        const int st = j & 1;
-        if (!mbar_wait(&sm.bar_y_empty[st], ((j - 2) >> 1) & 1, &sm.abort)) {
-          ok = false;
-          break;
+      for (int jj = nw; jj < n_t && ok; ++jj) {
+        const int j = tile_of(jj);
+        for (int kind = 0; kind < 2 && ok; ++kind) {
+          if (!needed(kind, j)) continue;
+          // a row product streams K_j, a column product Q_j
+          const int st = n % kSlots, use = n / kSlots;
+          ok = use == 0 || mbar_wait(&sm.bar_ring_empty[st], (use - 1) & 1, &sm.abort);
+          if (!ok) break;
+          mbar_arrive_expect_tx(&sm.bar_ring_full[st], kTileBytes);
+          for (int h = 0; h < 2; ++h)
+            tma_load_4d(ring + st * kTileBytes + h * kBoxBytes, kind == 0 ? &tm_k : &tm_q, &sm.bar_ring_full[st],
+                        64 * h, pos0 + j * kT, kind == 0 ? hkv : hq, b);
+          ++n;
         }
-        mbar_arrive_expect_tx(&sm.bar_y_full[st], kTileBytes);
-        for (int h = 0; h < 2; ++h)
-          tma_load_4d(sm.y[st] + h * kBoxBytes, tm_y, &sm.bar_y_full[st], 64 * h, pos0 + j * kT, hy, b);
-        last = j;
       }
       if (!ok) {
         report_status(status, kStatusTimeout, 60);
         sm.abort = 1;
-        // let every copy already issued land before the CTA's shared memory is released
-        mbar_wait(&sm.bar_x, 0, nullptr);
-        for (int jj = max(0, last - 1); jj <= last; ++jj) mbar_wait(&sm.bar_y_full[jj & 1], (jj >> 1) & 1, nullptr);
       }
+      // let every copy issued land before the CTA's shared memory is released: the resident tiles
+      // whose products were left out, the rest on an abort
+      for (int w = 0; w < nw; ++w) {
+        mbar_wait(&sm.bar_q[w], 0, nullptr);
+        mbar_wait(&sm.bar_k[w], 0, nullptr);
+      }
+      for (int e = max(0, n - kSlots); e < n; ++e) mbar_wait(&sm.bar_ring_full[e % kSlots], (e / kSlots) & 1, nullptr);
     }
   } else if (warp == kMmaWarp) {
     if (lane == 0) {
       constexpr uint32_t id_s = idesc_bf16_f32(kT, kT, false, false);
       constexpr uint64_t kTileDesc = kTileBytes >> 4;
-      bool ok = mbar_wait(&sm.bar_x, 0, &sm.abort);
-      tc_fence_after_sync();
-      const uint64_t dx = sdesc_sw128(smem_u32(sm.x), 16, 1024);
-      const uint64_t dy0 = sdesc_sw128(smem_u32(sm.y[0]), 16, 1024);
-      for (int j = 0; j < n_t && ok; ++j) {
-        const int st = j & 1;
-        ok = mbar_wait(&sm.bar_y_full[st], (j >> 1) & 1, &sm.abort);
-        if (ok && j >= 2) ok = mbar_wait(&sm.bar_s_empty[st], ((j - 2) >> 1) & 1, &sm.abort);
-        if (!ok) break;
-        tc_fence_after_sync();
-        // S_st = X . Y(j)^T, both K-major with 128-byte swizzle
+      const uint64_t dq = sdesc_sw128(smem_u32(xq), 16, 1024);
+      const uint64_t dk = sdesc_sw128(smem_u32(xk), 16, 1024);
+      const uint64_t dr = sdesc_sw128(smem_u32(ring), 16, 1024);
+      int n = 0;              // streamed tiles taken
+      int k[2] = {0, 0};      // products issued to each warpgroup
+      bool ok = true;
+      for (int jj = 0; jj < n_t && ok; ++jj) {
+        const int j = tile_of(jj);
+        for (int kind = 0; kind < 2 && ok; ++kind) {
+          if (!needed(kind, j)) continue;
+          // B: K_j (rows) or Q_j (columns), resident or streamed
+          uint64_t db;
+          if (jj < nw) {
+            ok = mbar_wait(kind == 0 ? &sm.bar_k[jj] : &sm.bar_q[jj], 0, &sm.abort);
+            db = (kind == 0 ? dk : dq) + jj * kTileDesc;
+          } else {
+            ok = mbar_wait(&sm.bar_ring_full[n % kSlots], (n / kSlots) & 1, &sm.abort);
+            db = dr + (n % kSlots) * kTileDesc;
+          }
+          for (int w = 0; w < nw && ok; ++w) {
+            const int wg = NT == 2 ? w : kind;
+            const int buf = k[wg] % nbuf, use = k[wg] / nbuf;
+            ok = mbar_wait(kind == 0 ? &sm.bar_q[w] : &sm.bar_k[w], 0, &sm.abort) &&
+                 (use == 0 || mbar_wait(&sm.bar_s_empty[wg][buf], (use - 1) & 1, &sm.abort));
+            if (!ok) break;
+            tc_fence_after_sync();
+            // S = A . B^T, both K-major with 128-byte swizzle
+            const uint64_t da = (kind == 0 ? dq : dk) + w * kTileDesc;
 #pragma unroll
-        for (int ks = 0; ks < kD / 16; ++ks) {
-          const uint64_t off = static_cast<uint64_t>(((ks >> 2) * kBoxBytes + (ks & 3) * 32) >> 4);
-          umma_ss(tbase + st * kT, dx + off, dy0 + st * kTileDesc + off, id_s, ks > 0 ? 1u : 0u);
+            for (int ks = 0; ks < kD / 16; ++ks) {
+              const uint64_t off = static_cast<uint64_t>(((ks >> 2) * kBoxBytes + (ks & 3) * 32) >> 4);
+              umma_ss(tbase + (wg * nbuf + buf) * kT, da + off, db + off, id_s, ks > 0 ? 1u : 0u);
+            }
+            umma_commit(&sm.bar_s_full[wg][buf]);
+            ++k[wg];
+          }
+          if (jj >= nw) {
+            umma_commit(&sm.bar_ring_empty[n % kSlots]);
+            ++n;
+          }
         }
-        umma_commit(&sm.bar_s_full[st]);
-        umma_commit(&sm.bar_y_empty[st]);
       }
       if (!ok) {
         report_status(status, kStatusTimeout, 61);
@@ -246,78 +308,92 @@ __global__ void __launch_bounds__(kThreads, 2)
       umma_commit(&sm.bar_drain);
       mbar_wait(&sm.bar_drain, 0, nullptr);
     }
-  } else {
-    // ---------------- rows / keys of the resident tile ----------------
-    const int r = tid;                                 // tensor-memory lane
-    const uint32_t trow = tbase + (static_cast<uint32_t>(warp * 32) << 16);
-    const int i = t * kT + r;                          // response index of this thread's query / key
-    const bool valid = i < per;
-    const size_t qrow = (static_cast<size_t>(bh) * L + pos0 + i) * kD;
-    // the diagonal entry of a seed query uses its masked-input key (leave-one-out view)
-    const int my_slot = valid ? sm.slot[r] : kNoSlot;
-    float p_self = 0.0f;
-    if (my_slot != kNoSlot) {
-      const float lse2 = cols ? colv[i] : own;         // +inf for a query that is not masked: weight 0
-      const float dot = dot_row(q + qrow, k_seedmask + ((static_cast<size_t>(b) * Hkv + hkv) * n_seeds + my_slot) * kD);
-      p_self = ex2_approx(dot * scale_log2 - lse2);
-    }
-    float acc = 0.0f;
+  } else if (my < nw) {
+    // ---------------- rows / keys of the resident tiles ----------------
+    const uint32_t trow = tbase + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+    // the diagonal entry of a seed query uses its masked-input key (leave-one-out view): its score
+    // replaces the cached one before the exponentials
+    const int my_slot = valid ? sm.slot[my * kT + r] : kNoSlot;
+    const bool warp_seed = __any_sync(0xffffffffu, my_slot != kNoSlot);
+    float s_self = 0.0f;
     bool ok = true;
-    for (int j = 0; j < n_t; ++j) {
-      const int st = j & 1;
-      ok = mbar_wait(&sm.bar_s_full[st], (j >> 1) & 1, &sm.abort);
-      if (!__all_sync(0xffffffffu, ok)) {
-        ok = false;
-        break;
-      }
-      tc_fence_after_sync();
-      const int diag = (j == t && my_slot != kNoSlot) ? r : -1;   // column of the seed diagonal
-      float a4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-      // two halves of 64 columns keep half of the tile in registers at a time
+    if (warp_seed) {
+      ok = mbar_wait(&sm.bar_q[my], 0, &sm.abort);
+      if (ok && my_slot != kNoSlot)
+        s_self = dot_row(xq + my * kTileBytes, r,
+                         k_seedmask + ((static_cast<size_t>(b) * Hkv + hkv) * n_seeds + my_slot) * kD);
+      ok = __all_sync(0xffffffffu, ok);
+    }
+    const uint64_t scale2 = f2_pack(scale_log2, scale_log2), nown2 = f2_pack(-own, -own);
+    float acc[2] = {0.0f, 0.0f};   // rows, columns
+    int k = 0;
+    for (int jj = 0; jj < n_t && ok; ++jj) {
+      const int j = tile_of(jj);
 #pragma unroll
-      for (int hf = 0; hf < 2; ++hf) {
-        uint32_t raw[2][32];
-#pragma unroll
-        for (int c = 0; c < 2; ++c) tmem_ld32(trow + st * kT + 64 * hf + 32 * c, raw[c]);
-#pragma unroll
-        for (int c = 0; c < 2; ++c) tmem_ld_wait(raw[c]);
-        if (hf == 1) {
-          tc_fence_before_sync();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&sm.bar_s_empty[st]);
-        }
-        const float* s = reinterpret_cast<const float*>(&raw[0][0]);
-#pragma unroll
-        for (int cc = 0; cc < 2; ++cc) {
-          const int c32 = 2 * hf + cc;
-          const uint32_t word = bits[j * 4 + c32];    // the same for every thread: uniform branch
+      for (int kind = 0; kind < 2; ++kind) {
+        if (!needed(kind, j) || (NT == 1 && kind != g) || !ok) continue;
+        const int buf = k % nbuf;
+        ok = __all_sync(0xffffffffu, mbar_wait(&sm.bar_s_full[g][buf], (k / nbuf) & 1, &sm.abort));
+        if (!ok) break;
+        ++k;
+        tc_fence_after_sync();
+        const int diag = my_slot != kNoSlot ? r : -1;   // column of the seed diagonal in tile t0 + my
+        uint64_t a2[2] = {0, 0};
+        // a quarter of the tile in registers at a time
+#pragma unroll 1
+        for (int c32 = 0; c32 < 4; ++c32) {
+          const uint32_t word = bits[(kind * n_t + j) * 4 + c32];   // the same for every thread
+          uint32_t raw[32];
+          if (word != 0u) {
+            tmem_ld32(trow + (g * nbuf + buf) * kT + 32 * c32, raw);
+            tmem_ld_wait(raw);
+          }
+          if (c32 == 3) {
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.bar_s_empty[g][buf]);
+          }
           if (word == 0u) continue;
-          if (!cols) {
+          float* s = reinterpret_cast<float*>(raw);
+          if (warp_seed && j == t0 + my) {
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
-              const int c = c32 * 32 + e;
-              float p = ex2_approx(fmaf(s[cc * 32 + e], scale_log2, -own));
-              if (c == diag) p = p_self;
-              a4[e & 3] += ((word >> e) & 1u) ? p : 0.0f;
-            }
-          } else {
-            const float4* cv = reinterpret_cast<const float4*>(colv + j * kT + c32 * 32);
+            for (int c = 0; c < 32; ++c)
+              if (32 * c32 + c == diag) s[c] = s_self;
+          }
 #pragma unroll
-            for (int e4 = 0; e4 < 8; ++e4) {
-              const float4 v = cv[e4];
-              const float vv[4] = {v.x, v.y, v.z, v.w};
+          for (int e4 = 0; e4 < 8; ++e4) {
+            const uint32_t nib = (word >> (4 * e4)) & 15u;
+            if (kind == 0 && nib == 0u) continue;
+            const float* s4 = s + 4 * e4;
+            float p[4];
+            if (kind == 0) {
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const int c = c32 * 32 + e4 * 4 + e;
-                float p = ex2_approx(fmaf(s[cc * 32 + e4 * 4 + e], scale_log2, -vv[e]));
-                if (c == diag) p = p_self;
-                a4[e] += p;
+              for (int e = 0; e < 4; e += 2) {
+                float x, y;
+                f2_unpack(f2_fma(f2_pack(s4[e], s4[e + 1]), scale2, nown2), x, y);
+                p[e] = (nib >> e) & 1u ? ex2_approx(x) : 0.0f;
+                p[e + 1] = (nib >> (e + 1)) & 1u ? ex2_approx(y) : 0.0f;
               }
+            } else {
+              // the queries' negated lse, -inf where not masked (weight 0)
+              const float4 v = *reinterpret_cast<const float4*>(colv + j * kT + 32 * c32 + 4 * e4);
+              float x, y;
+              f2_unpack(f2_fma(f2_pack(s4[0], s4[1]), scale2, f2_pack(v.x, v.y)), x, y);
+              p[0] = ex2_approx(x);
+              p[1] = ex2_approx(y);
+              f2_unpack(f2_fma(f2_pack(s4[2], s4[3]), scale2, f2_pack(v.z, v.w)), x, y);
+              p[2] = ex2_approx(x);
+              p[3] = ex2_approx(y);
             }
+            a2[0] = f2_add(a2[0], f2_pack(p[0], p[1]));
+            a2[1] = f2_add(a2[1], f2_pack(p[2], p[3]));
           }
         }
+        float a4[4];
+        f2_unpack(a2[0], a4[0], a4[1]);
+        f2_unpack(a2[1], a4[2], a4[3]);
+        acc[kind] += (a4[0] + a4[1]) + (a4[2] + a4[3]);
       }
-      acc += (a4[0] + a4[1]) + (a4[2] + a4[3]);
     }
     if (!ok) {
       if (lane == 0 && !sm.abort) {
@@ -325,36 +401,74 @@ __global__ void __launch_bounds__(kThreads, 2)
         sm.abort = 1;
       }
     } else if (valid) {
-      (cols ? part_in : part_out)[static_cast<size_t>(bh) * per + i] = acc;
+      const size_t o = static_cast<size_t>(bh) * per + i;
+      if (NT == 2 || g == 0) part_out[o] = acc[0];
+      if (NT == 2 || g == 1) part_in[o] = acc[1];
     }
   }
 
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
-  if (warp == kMmaWarp) tmem_dealloc(tbase, 256);
+  if (warp == kMmaWarp) tmem_dealloc(tbase, tmem_cols);
 }
 
-// d_in / d_out of row n = b * per + i: the partial sums of the Hq heads in a fixed order,
-// divided by the head count.
-__global__ void mass_reduce_kernel(const float* __restrict__ part_in, const float* __restrict__ part_out, int B,
-                                   int Hq, int per, float* __restrict__ d_in, float* __restrict__ d_out) {
+// d_in / d_out of row n = b * per + i: the partial sums of the Hq heads in a fixed order, divided
+// by the head count. A CTA takes 32 rows; warp w adds heads w, w + 8, ..., then the eight sums are
+// added in order (one thread per row walking all heads was a chain of Hq loads).
+constexpr int kReduceWarps = 8;
+__global__ void __launch_bounds__(32 * kReduceWarps)
+    mass_reduce_kernel(const float* __restrict__ part_in, const float* __restrict__ part_out, int B, int Hq, int per,
+                       float* __restrict__ d_in, float* __restrict__ d_out) {
+  __shared__ float sums[2][kReduceWarps][32];
   // launched as a programmatic dependent of mass_kernel: wait until its partial sums are complete
   // and visible
   griddep_wait();
   griddep_launch_dependents();
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= B * per) return;
-  const int b = n / per, i = n % per;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = blockIdx.x * 32 + lane;
+  const bool in = n < B * per;
+  const int b = in ? n / per : 0, i = in ? n - b * per : 0;
   float si = 0.0f, so = 0.0f;
-  for (int h = 0; h < Hq; ++h) {
+#pragma unroll 4
+  for (int h = warp; h < Hq; h += kReduceWarps) {
     const size_t o = (static_cast<size_t>(b) * Hq + h) * per + i;
     si += part_in[o];
     so += part_out[o];
   }
-  const float inv = 1.0f / static_cast<float>(Hq);
-  d_in[n] = si * inv;
-  d_out[n] = so * inv;
+  sums[0][warp][lane] = si;
+  sums[1][warp][lane] = so;
+  __syncthreads();
+  if (warp < 2 && in) {
+    float t = sums[warp][0][lane];
+#pragma unroll
+    for (int w = 1; w < kReduceWarps; ++w) t += sums[warp][w][lane];
+    (warp == 0 ? d_in : d_out)[n] = t * (1.0f / static_cast<float>(Hq));
+  }
+}
+
+template <int NT>
+int launch_tiles(const MassArgs& a, int n_t, const CUtensorMap& tq, const CUtensorMap& tk, float* part_in,
+                 float* part_out, int* status, cudaStream_t stream) {
+  // the shared-memory limit is a function attribute of the current context
+  static ContextCache<int> setup;
+  int unused = 0;
+  const int rc = setup.get(&unused, [](int&) {
+    const size_t most = mass_smem_bytes(NT, NT == 2 ? kMaxTilesPair : (kMaxPer + kT - 1) / kT);
+    return cudaFuncSetAttribute(mass_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(most)) == cudaSuccess ? 0 : -3;
+  });
+  if (rc != 0) return rc;
+  const int n_g = (n_t + NT - 1) / NT;
+  const long long grid = static_cast<long long>(n_g) * a.Hq * a.B;
+  if (grid > 0x7fffffffLL) return -2;
+  const float scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(kD));
+  cudaLaunchAttribute attr[1];
+  const cudaLaunchConfig_t cfg =
+      pdl_config(dim3(static_cast<unsigned>(grid)), dim3(kThreads), mass_smem_bytes(NT, n_t), stream, attr);
+  return cudaLaunchKernelEx(&cfg, mass_kernel<NT>, tq, tk, static_cast<const __nv_bfloat16*>(a.k_seedmask), a.seed_idx,
+                            a.n_seeds, a.lse, a.Hq, a.Hkv, a.L, a.pos0, a.per, n_t, n_g, a.tok, a.flags, a.mask_id,
+                            scale_log2, part_in, part_out, status) == cudaSuccess ? 0 : -3;
 }
 
 }  // namespace
@@ -369,38 +483,29 @@ int launch_attn_mass(const MassArgs& a, int* status, cudaStream_t stream) {
   if (!make_bf16_map_4d(&tq, a.q, kD, a.L, a.Hq, a.B, kT) || !make_bf16_map_4d(&tk, a.k_cached, kD, a.L, a.Hkv, a.B, kT))
     return -3;
   const int n_t = (a.per + kT - 1) / kT;
-  const long long grid = static_cast<long long>(n_t) * a.Hq * a.B;
-  if (grid > 0x7fffffffLL) return -2;
+  if (static_cast<long long>(n_t) * a.Hq * a.B > 0x7fffffffLL) return -2;
   float* part_in = static_cast<float*>(a.workspace);
   float* part_out = part_in + static_cast<size_t>(a.B) * a.Hq * a.per;
-  const size_t smem = sizeof(MassSmem) + 1024 + static_cast<size_t>(n_t) * (4 * sizeof(uint32_t) + kT * sizeof(float));
-  // the shared-memory limit is a function attribute of the current context
-  static ContextCache<int> setup;
-  int unused = 0;
-  const int rc = setup.get(&unused, [](int&) {
-    const size_t most = sizeof(MassSmem) + 1024 + static_cast<size_t>((kMaxPer + kT - 1) / kT) *
-                                                      (4 * sizeof(uint32_t) + kT * sizeof(float));
-    return cudaFuncSetAttribute(mass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most)) ==
-                   cudaSuccess ? 0 : -3;
+  static ContextCache<int> sms;
+  int n_sm = 0;
+  int rc = sms.get(&n_sm, [](int& v) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return -3;
+    return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? 0 : -3;
   });
   if (rc != 0) return rc;
-  const float scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(kD));
-  {
-    cudaLaunchAttribute attr[1];
-    const cudaLaunchConfig_t cfg =
-        pdl_config(dim3(static_cast<unsigned>(grid), 2), dim3(kThreads), smem, stream, attr);
-    if (cudaLaunchKernelEx(&cfg, mass_kernel, tq, tk, static_cast<const __nv_bfloat16*>(a.q),
-                           static_cast<const __nv_bfloat16*>(a.k_seedmask), a.seed_idx, a.n_seeds, a.lse, a.Hq, a.Hkv,
-                           a.L, a.pos0, a.per, n_t, a.tok, a.flags, a.mask_id, scale_log2, part_in, part_out,
-                           status) != cudaSuccess)
-      return -3;
-  }
-  if (cudaGetLastError() != cudaSuccess) return -3;
+  // Tiles per CTA: two while the tiles outnumber the SMs; below that one tile a CTA spreads over
+  // more SMs. us at NT = 1 / 2 (B, heads, rows): 4, 32, 256: 16.8 / 10.9; 1, 32 / 32, 1024: 34.9 /
+  // 23.7; 2, 32 / 8, 256 (128 tiles): 9.5 / 10.2; 1, 28 / 4, 512 (112 tiles): 12.0 / 14.4.
+  const bool pair = n_t > 1 && n_t <= kMaxTilesPair && static_cast<long long>(n_t) * a.Hq * a.B > n_sm;
+  rc = pair ? launch_tiles<2>(a, n_t, tq, tk, part_in, part_out, status, stream)
+            : launch_tiles<1>(a, n_t, tq, tk, part_in, part_out, status, stream);
+  if (rc != 0) return rc;
   // the reduction may launch while the partial sums are still being written (programmatic
   // dependent launch); it waits on the device for them, so its launch latency is hidden
   const int rows = a.B * a.per;
   cudaLaunchAttribute attr[1];
-  const cudaLaunchConfig_t cfg = pdl_config(dim3(static_cast<unsigned>((rows + 255) / 256)), dim3(256), 0, stream, attr);
+  const cudaLaunchConfig_t cfg = pdl_config(dim3(static_cast<unsigned>((rows + 31) / 32)), dim3(32 * kReduceWarps), 0, stream, attr);
   return cudaLaunchKernelEx(&cfg, mass_reduce_kernel, static_cast<const float*>(part_in),
                             static_cast<const float*>(part_out), a.B, a.Hq, a.per, a.d_in, a.d_out) == cudaSuccess
              ? 0 : -3;

@@ -85,6 +85,34 @@ def test_mass_against_oracle(B, Hq, Hkv, L, S, pos0, per):
     assert np.all(np.abs(d_out - ref_out.ravel()) <= _mass_tol(ref_out.ravel())), np.abs(d_out - ref_out.ravel()).max()
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,L,pos0,per", [
+    (20, 4, 2, 300, 40, 256),     # 160 tiles of queries: two resident tiles a CTA (one up to 152)
+    (18, 3, 3, 420, 30, 390),     # four tiles, the last ragged, streamed past two resident ones
+    (17, 3, 1, 300, 0, 300),      # three tiles: a CTA with one of its two
+])
+@pytest.mark.parametrize("where", ["first", "none", "last"])
+def test_mass_resident_pairs_and_skipped_products(B, Hq, Hkv, L, pos0, per, where):
+    """Two resident tiles a CTA; drafted keys and masked queries in one tile only, or none drafted."""
+    inp = W.make_attn_inputs(B, Hq, Hkv, L, 128, 6, dtype="bf16", seed=L + per, seed_lo=0, seed_hi=L)
+    tok, flags = np.zeros((B, per), np.int32), np.zeros((B, per), np.uint8)
+    if where == "first":
+        flags[:, [3, 64, 127]] = 2
+        tok[:, per - 40:] = 7
+    else:
+        tok[:, 1:90:2] = 7
+        if where == "last":
+            flags[:, per - 1] = 2
+    masked, drafted = tok == 7, (flags & 2) != 0
+    d_in, d_out = run_mass(inp, tok.ravel(), flags.ravel(), pos0, per)
+    pick = [0, B - 1]
+    ref_in, ref_out = oracle_mass(inp, masked, drafted, pos0, batches=pick)
+    for got, ref in ((d_in, ref_in), (d_out, ref_out)):
+        for k, b in enumerate(pick):
+            assert np.all(np.abs(got[b * per:(b + 1) * per] - ref[k]) <= _mass_tol(ref[k]))
+    if where == "none":
+        assert not d_out.any()
+
+
 def test_mass_whole_memory_sums_to_the_masked_count():
     # with every position a response position each masked row spreads mass 1 over the keys
     B, Hq, Hkv, L, S = 2, 4, 2, 640, 16
