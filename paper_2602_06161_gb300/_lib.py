@@ -15,6 +15,12 @@ _P = ctypes.c_void_p
 _I = ctypes.c_int
 _lock = threading.Lock()
 _lib = None
+_native = None
+
+# the entry points that the native marshalling (_binding) calls, in the order it binds them
+_BOUND = ("cover_attn_fwd", "cover_attn_fwd_f32", "cover_attn_fwd_prefix", "cover_attn_fwd_prefix_f32",
+          "cover_score_fwd", "cover_score_decide_fwd", "cover_attn_mass_fwd", "cover_seed_kv_gather",
+          "cover_seed_kv_override")
 
 # name -> (restype, argtypes)
 _SIGNATURES = {
@@ -75,6 +81,17 @@ def load(build_if_needed: bool = True):
             fn.argtypes = args
         _lib = lib
         return lib
+
+
+def native():
+    """The native argument marshalling, bound to the loaded library's entry points."""
+    global _native
+    if _native is None:
+        lib = load()
+        from . import _binding
+        _binding.bind([ctypes.cast(getattr(lib, name), _P).value for name in _BOUND])
+        _native = _binding
+    return _native
 
 
 def exported_symbols():

@@ -1,4 +1,5 @@
-"""Builds libcover.so (the C-ABI kernel library) in-tree with nvcc for sm_103a.
+"""Builds libcover.so (the C-ABI kernel library) in-tree with nvcc for sm_103a, and beside it
+_binding.so (the Python calls' native argument marshalling) with the host compiler.
 
 Each translation unit compiles in parallel; the objects link into
 ``paper_2602_06161_gb300/libcover.so``. The CUDA runtime is linked statically
@@ -19,6 +20,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libcover.so")
+BINDING = os.path.join(PKG, "_binding.so")
 
 SOURCES = ["cover_api.cu", "context.cu", "tmap.cu", "route_kernel.cu", "attn_f32.cu", "attn_bf16_sm103.cu", "attn_window_gqa.cu",
            "score_kernel.cu", "kv_kernel.cu", "mass_kernel.cu", "debug_kernels.cu"]
@@ -33,18 +35,39 @@ def nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
-def _stale(lib: str) -> bool:
-    if not os.path.exists(lib):
+def _stale() -> bool:
+    if not os.path.exists(LIB) or not os.path.exists(BINDING):
         return True
-    t = os.path.getmtime(lib)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [
         os.path.join(INCLUDE, f) for f in os.listdir(INCLUDE)] + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _build_binding() -> None:
+    import sysconfig
+
+    import torch
+
+    root = os.path.dirname(torch.__file__)
+    tmp = BINDING + ".tmp"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    for inc in (os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+                os.path.join(os.path.dirname(os.path.dirname(nvcc())), "include"), sysconfig.get_paths()["include"]):
+        cmd += ["-isystem", inc]
+    lib = os.path.join(root, "lib")
+    cmd += ["-I", INCLUDE, os.path.join(CSRC, "binding.cpp"), "-o", tmp, "-L" + lib, "-Wl,-rpath," + lib,
+            "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"binding.cpp failed:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, BINDING)
+
+
 def build(force: bool = False, verbose_ptxas: bool = False, quiet: bool = True) -> str:
     """Compile (if stale) and return the path of libcover.so."""
-    if not force and not _stale(LIB):
+    if not force and not _stale():
         return LIB
     os.makedirs(BUILD, exist_ok=True)
     cc = nvcc()
@@ -57,8 +80,10 @@ def build(force: bool = False, verbose_ptxas: bool = False, quiet: bool = True) 
         r = subprocess.run(cmd, capture_output=True, text=True)
         return src, obj, r
 
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    with cf.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
+        binding = ex.submit(_build_binding)
         results = list(ex.map(compile_one, SOURCES))
+        binding.result()
     logs = []
     for src, obj, r in results:
         if r.returncode != 0:

@@ -1,0 +1,43 @@
+"""The native argument marshalling takes only calls of plain CUDA tensors: any other form is handed
+back (None) with nothing launched, and the Python path raises its errors as it always did."""
+import pytest
+import torch
+
+from paper_2602_06161_gb300 import _lib, api
+
+
+def _qkv(dtype=torch.bfloat16):
+    return [torch.zeros(1, 2, 16, 128, dtype=dtype) for _ in range(3)]
+
+
+def test_cpu_tensors_are_handed_back_and_refused():
+    q, k, v = _qkv()
+    n = _lib.native()
+    assert n.attn(0, q, k, v, None, None, None, 0, None, None, True, None) is None
+    assert n.attn(2, q, k, v, None, None, None, 0, None, None, True, None) is None
+    assert n.kv(1, k, v, torch.zeros(1, 2, dtype=torch.int32), k, v, None) is None
+    with pytest.raises(ValueError, match="q must be a CUDA tensor"):
+        api.cover_attn_fwd(q, k, v)
+    with pytest.raises(TypeError, match="q must be torch.float32"):
+        api.cover_attn_fwd_f32(q, k, v)
+    with pytest.raises(ValueError, match="logits must be a CUDA tensor"):
+        api.cover_score_fwd(torch.zeros(4, 8, dtype=torch.bfloat16), 1, 1)
+
+
+@pytest.mark.parametrize("args", [(None,) * 12, (0, 1, 2, 3, None, None, None, 0, None, None, True, None),
+                                  ("0",) + (None,) * 11])
+def test_other_objects_are_handed_back(args):
+    assert _lib.native().attn(*args) is None
+
+
+def test_wrong_number_of_arguments():
+    for fn in ("attn", "score", "decide", "mass", "kv"):
+        with pytest.raises(TypeError):
+            getattr(_lib.native(), fn)(1, 2)
+    with pytest.raises(ValueError):
+        _lib.native().bind([1, 2])
+
+
+def test_not_a_tensor():
+    with pytest.raises(TypeError, match="q must be a torch.Tensor"):
+        api.cover_attn_fwd([1.0], None, None)
