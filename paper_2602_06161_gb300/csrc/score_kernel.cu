@@ -57,7 +57,9 @@ constexpr int kMaxPerSeq = 4096;            // rows per segment (the entry point
 constexpr int kRowLoads = 4;                // rows whose state a thread loads at once (general paths)
 constexpr int kRoundsMax = 32;              // selections up to this size by rounds or warp sorts (top_select)
 constexpr int kRoundsFew = 8;               // selections up to this size by per-warp rounds (top_rounds)
-constexpr int kMaxWarps = 16;               // every kernel here runs at most 512 threads
+constexpr int kMaxWarps = 32;               // the selection kernels run up to 1024 threads
+constexpr int kMaxThreads = 32 * kMaxWarps;
+constexpr int kRankWarps = 16;              // top_small ranks the published keys of up to this many warps
 constexpr int kMaxSplit = 8;                // CTAs a row is split over (the portable cluster size)
 constexpr int kMinSlice = 2048;             // elements of a row a CTA gets at least
 
@@ -334,6 +336,7 @@ __device__ __forceinline__ bool row_write(const RowOut& r, int n, const uint16_t
     // decision step: the seed score is formed after the state update
     ws_u[n] = u;
     ws_lnz[n] = lnZ;
+    if (counters == nullptr) return false;   // the decisions have a launch of their own
   } else {
     score[n] = u * (1.0f + din) / (1.0f + dout);
     if (topk <= 0) return false;
@@ -349,6 +352,7 @@ __device__ __forceinline__ bool row_write(const RowOut& r, int n, const uint16_t
   return old == static_cast<unsigned>(per_seq - 1);
 }
 
+constexpr int kDecideFused = 1, kDecideApart = 2;
 struct ScoreParams {
   const uint16_t* logits;
   int V, per_seq;
@@ -364,7 +368,7 @@ struct ScoreParams {
   int32_t* topk_idx;
   float* topk_score;
   uint32_t* counters;
-  int decide;          // 1: run the decision step instead of the top-k
+  int decide;          // kDecideFused: the last CTA of a segment decides; kDecideApart: decide_kernel does
   DecideArgs dec;
 };
 
@@ -910,12 +914,32 @@ __device__ __forceinline__ int rank_below(const uint64_t* keys, int n, uint64_t 
 // The k largest (k <= 32) of the CTA's keys, one per thread (distinct, 0 = none). Each warp sorts
 // its keys and publishes its k largest in cand[warp * k ..]; a key can be among the CTA's k
 // largest only if it is among its warp's, and the number of larger published keys is its rank,
-// exact while below k (a warp publishes at most k). Returns, for the key this lane holds after
-// its warp's sort (*held), its slot 0 .. k-1 among the CTA's k largest, else -1. All threads of
-// the CTA call it; cand holds blockDim.x keys.
+// exact while below k (a warp publishes at most k). With many warps the
+// sorted lists are merged pairwise instead (log2(warps) barriers), since ranking against every
+// published key would cost warps * k reads a thread. Returns, for the key this lane then holds
+// (*held), its slot 0 .. k-1 among the CTA's k largest, else -1. All threads of the CTA call it;
+// cand holds blockDim.x keys.
 __device__ __forceinline__ int top_small(uint64_t key, int k, uint64_t* cand, uint64_t* held) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const uint64_t sorted = warp_sort_desc(key, lane);
+  uint64_t sorted = warp_sort_desc(key, lane);
+  if (nw > kRankWarps) {
+    cand[threadIdx.x] = sorted;
+    for (int n = nw; n > 1;) {
+      // the upper half's lists go into the lower half's
+      const int half = (n + 1) >> 1;
+      __syncthreads();
+      if (warp + half < n) {
+        uint64_t mine[1] = {sorted};
+        const uint64_t other[1] = {cand[(warp + half) * 32 + lane]};
+        warp_merge_desc<1>(mine, other, lane);
+        sorted = mine[0];
+        cand[threadIdx.x] = sorted;
+      }
+      n = half;
+    }
+    *held = sorted;
+    return warp == 0 && lane < k && sorted != 0 ? lane : -1;
+  }
   if (lane < k) cand[warp * k + lane] = sorted;
   __syncthreads();
   int slot = -1;
@@ -937,7 +961,7 @@ __device__ void select_fast(uint64_t* keys, int seg, int per_seq, const DecideAr
   __shared__ long long s_fx[32];
   __shared__ uint32_t s_emax;
   __shared__ int s_elig;
-  __shared__ uint8_t s_mark[512];   // blockDim <= 512
+  __shared__ uint8_t s_mark[kMaxThreads];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int n = seg * per_seq + tid;
   float sc = -INFINITY;
@@ -1025,7 +1049,7 @@ __device__ void select_fast(uint64_t* keys, int seg, int per_seq, const DecideAr
 __device__ void decide_fast(uint64_t* keys, int seg, int per_seq, const ScoreParams& P) {
   __shared__ unsigned long long s_fallback;
   __shared__ int s_cnt[3];
-  __shared__ uint8_t s_draft[512];   // blockDim <= 512
+  __shared__ uint8_t s_draft[kMaxThreads];
   const DecideArgs& d = P.dec;
   const int tid = threadIdx.x, lane = tid & 31;
   const bool in = tid < per_seq;
@@ -1410,7 +1434,8 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
   }
   if (tid == 0)
     s_last = row_write(row_finish(r), n, row, V, P.per_seq, P.decide ? P.dec.tok : P.cur_tok, P.d_in, P.d_out, P.topk,
-                       P.maxprob, P.entropy, P.argmax, P.score, P.counters, P.decide ? P.dec.ws_u : nullptr,
+                       P.maxprob, P.entropy, P.argmax, P.score, P.decide == kDecideApart ? nullptr : P.counters,
+                       P.decide ? P.dec.ws_u : nullptr,
                        P.decide ? P.dec.ws_lnz : nullptr);
   __syncthreads();
   if (s_last) {
@@ -1420,6 +1445,19 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
       segment_topk(reinterpret_cast<uint64_t*>(ring), n / P.per_seq, P.per_seq, P.sort_n, P.topk, P.score,
                    P.eligible, P.topk_idx, P.topk_score);
   }
+}
+
+// One step's decisions as their own launch (one CTA per segment) behind the row kernel, for segments
+// of more rows than that kernel's CTAs have threads: up to 1024 rows then have a thread each, where
+// the last CTA of a segment made five passes over its rows. Segments of up to kBulkThreads rows
+// stay in the row kernel, where the last CTA starts on them at once.
+// 1 x 1024 rows of 152064 logits: 70.6 -> 62.0 us (54.0 us for the rows alone), and 92 -> 68 us in a
+// decoding step, whose other launches leave the row state in L2 only.
+__global__ void __launch_bounds__(kMaxThreads) decide_kernel(const ScoreParams P) {
+  extern __shared__ __align__(16) uint64_t dec_keys[];
+  griddep_wait();
+  griddep_launch_dependents();
+  segment_decide(dec_keys, blockIdx.x, P.per_seq, P.sort_n, P);
 }
 
 // Section 5.3 selection as its own launch (one CTA per segment), after the
@@ -1515,17 +1553,32 @@ int launch_score_impl(const ScoreArgs& a, const DecideArgs* d, int* status, cuda
   while (sort_n < per) sort_n <<= 1;
   ScoreParams P{static_cast<const uint16_t*>(a.logits), a.V, per, a.cur_tok, a.d_in, a.d_out, a.eligible,
                 a.topk, sort_n, a.maxprob, a.entropy, a.argmax, a.score, a.topk_idx, a.topk_score, a.counters,
-                d != nullptr ? 1 : 0, d != nullptr ? *d : DecideArgs{}};
+                d == nullptr ? 0 : per > kBulkThreads ? kDecideApart : kDecideFused, d != nullptr ? *d : DecideArgs{}};
   // top-k keys (at most 4096 x 8 bytes) reuse the ring; so does the decision step, which keeps a
   // float score per row behind them (4096 x 12 bytes, exactly the ring)
   static_assert((sizeof(uint64_t) + sizeof(float)) * kMaxPerSeq <= kRingStages * kChunkBytes, "keys fit the ring");
   const size_t smem = static_cast<size_t>(kRingStages) * kChunkBytes;
+  int rl = 0;
   switch (row_split(a.N, a.V, n_sm)) {
-    case 8: return launch_rows<8>(P, a.N, smem, status, stream);
-    case 4: return launch_rows<4>(P, a.N, smem, status, stream);
-    case 2: return launch_rows<2>(P, a.N, smem, status, stream);
-    default: return launch_rows<1>(P, a.N, smem, status, stream);
+    case 8: rl = launch_rows<8>(P, a.N, smem, status, stream); break;
+    case 4: rl = launch_rows<4>(P, a.N, smem, status, stream); break;
+    case 2: rl = launch_rows<2>(P, a.N, smem, status, stream); break;
+    default: rl = launch_rows<1>(P, a.N, smem, status, stream);
   }
+  if (rl != 0 || P.decide != kDecideApart) return rl;
+  const int threads = std::min((per + 31) / 32 * 32, kMaxThreads);
+  const size_t keys = (sizeof(uint64_t) + sizeof(float)) * static_cast<size_t>(std::max(sort_n, threads));
+  static ContextCache<int> setup;
+  int unused = 0;
+  const int rc2 = setup.get(&unused, [](int&) {
+    return cudaFuncSetAttribute(decide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>((sizeof(uint64_t) + sizeof(float)) * kMaxPerSeq)) == cudaSuccess
+               ? 0 : -3;
+  });
+  if (rc2 != 0) return rc2;
+  cudaLaunchAttribute attr[1];
+  const cudaLaunchConfig_t cfg = pdl_config(dim3(static_cast<unsigned>(a.n_seq)), dim3(threads), keys, stream, attr);
+  return cudaLaunchKernelEx(&cfg, decide_kernel, P) == cudaSuccess ? 0 : -3;
 }
 
 }  // namespace

@@ -201,6 +201,16 @@ def test_decide_both_sides_of_the_fast_path(per, V):
         check(di, p, run_decide(di, p), what=f"per {per} V {V} B {p['draft_budget']}")
 
 
+@pytest.mark.parametrize("per,n_seq", [(513, 2), (600, 3), (1024, 1), (1025, 2)])
+def test_decide_in_a_launch_of_its_own(per, n_seq):
+    # segments longer than the row kernel's CTAs have threads are decided by a launch of their own: the
+    # selections merge the sorted lists of 17, 19 and 32 warps; 1025 rows take its general path
+    di = W.make_decide_inputs(n_seq * per, 1000, n_seq, seed=per + 2, block_len=64)
+    for p in (_params(draft_budget=32, tau_draft=0.05, max_seeds=32), _params(draft_budget=1, tau_draft=0.05, max_seeds=3),
+              _params(draft_budget=33, tau_draft=0.02, max_seeds=40)):
+        check(di, p, run_decide(di, p), what=f"per {per}")
+
+
 @pytest.mark.parametrize("per", [256, 512, 513, 1024, 2049])
 def test_update_then_select_both_paths(per):
     # the split order (update phase, then the selection launch with the caller's d_in / d_out):
