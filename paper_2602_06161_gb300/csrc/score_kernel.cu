@@ -1292,9 +1292,14 @@ __device__ __forceinline__ void acc_batch(RowAcc& a, const uint4 (&w)[U], int i0
 // row kernel: bulk copies of a row, or of a row's slice in each CTA of a cluster
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  // The logits are read once and may exceed L2: evicted first, they leave the rest of a step there
+  // (states, weights, the next kernels' code). The pass itself takes the same time; in a decoding
+  // step of Dream's shape (311 MB of logits) the launches around it went from 98.9 to 87.2 us.
   asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(smem_dst)),
+      "{\n\t.reg .b64 policy;\n\t"
+      "createpolicy.fractional.L2::evict_first.b64 policy, 1.0;\n\t"
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1], %2, [%3], policy;\n\t}" ::"r"(smem_u32(smem_dst)),
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
