@@ -110,8 +110,8 @@ int cover_attn_fwd_f32(const float* q, const float* k_cached, const float* v_cac
  * kernel. Its rows agree with the square kernel's up to rounding (not bit for
  * bit). Any other window runs on the square kernel, where the rows of a KV
  * head's query heads may share Q tiles too; its window rows equal the square
- * launch's, bit for bit when Lk spans an odd number of 128-key tiles (with an
- * even number a unit's keys may be split in two, merged up to rounding).
+ * launch's, bit for bit unless one of the two launches splits the rows' keys in
+ * two halves (merged up to rounding) and the other does not.
  */
 int cover_attn_fwd_prefix(const void* q, const void* k_cached, const void* v_cached,
                           const void* k_seedmask, const void* v_seedmask,

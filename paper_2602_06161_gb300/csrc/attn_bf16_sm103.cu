@@ -208,7 +208,10 @@ __device__ __forceinline__ void raise_abort(AttnSmem& sm, int* status, int site)
 // otherwise Lq = Lk and q0 = 0 are compile-time facts.
 // kFault: the self-test instance that takes its wait limit and a planted missing load from
 // `flt`; the production instances wait up to one second and load every tile.
-template <int NQ, bool kWindow, bool kFault>
+// kPad: a split unit's halves may have an odd number of KV tiles between them (windows, and square
+// launches whose units are all split; the other square launches keep the code without it, which the
+// compiler schedules 7 % faster on long sequences).
+template <int NQ, bool kWindow, bool kFault, bool kPad = kWindow>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_bf16_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                      const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
@@ -228,11 +231,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint64_t wait_ns = kFault ? flt.wait_ns : kWaitLimitNs;
   const int Lq = kWindow ? Lq_arg : Lk;
   const int q0 = kWindow ? q0_arg : 0;
-  const int tail_valid = Lk - (nkv - 1) * kBN;   // valid keys in the last KV tile (1..128)
-  // one-tile units of a window are all split when the number of KV tiles is even, so the second
-  // softmax warpgroup takes half of every unit's keys
+  // one-tile units of a window are all split (with two KV tiles or more), so the second softmax
+  // warpgroup takes half of every unit's keys
   constexpr bool kSplitAll = kWindow && NQ == 1;
   const bool all_split = kSplitAll && ug.n_split > 0;
+  // A split unit's two halves have `half` KV tiles each; with an odd nkv (kPad) the last one lies past
+  // the memory (loaded as zeros without reading anything, every key masked). nks: KV ring entries of
+  // a split unit, nkr: of a unit before the CTA's last.
+  const int half = kPad ? (nkv + 1) >> 1 : nkv >> 1;
+  const int nks = kPad ? 2 * half : nkv;
+  const int nkr = all_split ? nks : nkv;
 
   // ---------------- prologue ----------------
   if (warp == kTmaWarp && lane == 0) {
@@ -301,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!mbar_wait(&sm.bar_ostage_full[t], n & 1, &sm.abort, wait_ns)) return false;
         // a split unit's one tile was staged by both warpgroups (one 64-column box each)
         if (wn.split && !mbar_wait(&sm.bar_ostage_full[1], n & 1, &sm.abort, wait_ns)) return false;
-        const int sig = (n * nkv + nkv - 1) & 1;
+        const int sig = (n * nkr + (wn.split ? nks : nkv) - 1) & 1;
         const uint8_t* stage = t == 0 ? sm.k[sig] : sm.v[sig];
         for (int wq = 0; wq < 4; ++wq) {
           const int wrow = tile_row0<kUnitRows>(wn, t) + wq * 32;
@@ -314,7 +322,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         bulk_wait_group_read0();
         return true;
       };
-      const int half = nkv >> 1;
       for (int it = 0; ok; ++it) {
         Unit w;
         if (!work_of<kSplitAll>(it, ug, w)) break;
@@ -371,7 +378,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = load_v(2 * sp) && (sp + 1 == half || load_k(2 * sp + 2)) && load_v(2 * sp + 1) &&
                  (sp + 1 == half || load_k(2 * sp + 3));
           }
-          G = g0 + nkv;
+          G = g0 + nks;
           continue;
         }
         // K and V tiles of ring entry jj; `staged`: the entry's stage holds the output of the unit
@@ -618,7 +625,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           // entries G + 2 s + t, both against the Q tile in buffer 0. Every K and V tile has
           // one user, so each product frees its own stage; a V tile is waited for right before
           // its P.V product, since the TMA thread loads it only after the previous step's P.V.
-          const int half = nkv >> 1, g0 = G;
+          const int g0 = G;
           // P barriers complete once per warpgroup step: nkv per earlier whole unit, half per
           // earlier split unit
           const int pb = all_split ? it * half : g0;
@@ -658,7 +665,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             umma_commit(&sm.bar_o_full[t]);
             umma_commit(&sm.bar_v_empty[ring & 1]);
           }
-          G = g0 + nkv;
+          G = g0 + nks;
           if (all_split) continue;
           break;
         }
@@ -747,9 +754,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (!ok) break;
           const Unit w = sm.unit[sb];
           const int grow = tile_row0<kUnitRows>(w, qt) + r;
-          const int jbase = w.split ? qt * (nkv >> 1) : 0;
-          steps = w.split ? nkv >> 1 : nkv;
-          tail_j = tail_valid < kBN ? nkv - 1 - jbase : -1;   // -1: no ragged tile
+          const int jbase = w.split ? qt * half : 0;
+          steps = w.split ? half : nkv;
+          // the (first) tile with a key past the memory
+          if (kPad) tail_j = Lk / kBN - jbase;
+          else tail_j = Lk % kBN != 0 ? nkv - 1 - jbase : -1;
           my_slot = sm.slot[sb][qt * kBM + r];
           if (grow >= Lq) my_slot = kNoSlot;
           // the diagonal of a square launch is column r of KV tile row0 / 128 of the row's Q tile
@@ -766,9 +775,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         // in a window: the KV steps that hold the diagonals of the warp's seed rows (none: lo > hi)
         const int dj_lo = kWindow ? __reduce_min_sync(0xffffffffu, is_seed ? diag_j : 0x7fffffff) : diag_j;
         const int dj_hi = kWindow ? __reduce_max_sync(0xffffffffu, is_seed ? diag_j : -0x7fffffff) : diag_j;
-        const int g0 = it * nkv;   // the CTA's KV steps before this unit
+        const int g0 = it * nkr;   // the CTA's KV ring entries before this unit
         // this warpgroup's steps before this unit (half a unit's KV tiles each when all are split)
-        const int sbase = all_split ? it * (nkv >> 1) : g0;
+        const int sbase = all_split ? it * half : g0;
         float m_run = -INFINITY, l_run = 0.0f;
 
         for (int j = 0; j < steps && ok; ++j) {
@@ -781,8 +790,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int c = 0; c < 4; ++c) tmem_ld_wait(raw[c]);
           float* s = reinterpret_cast<float*>(&raw[0][0]);
-          if (j == tail_j) {
-            const int valid = Lk - (nkv - 1) * kBN;
+          if (kPad ? j >= tail_j : j == tail_j) {
+            const int valid = kPad ? Lk % kBN - (j - tail_j) * kBN : Lk - (nkv - 1) * kBN;
 #pragma unroll
             for (int c = 0; c < kBN; ++c)
               if (c >= valid) s[c] = -INFINITY;
@@ -938,7 +947,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               m = m2;
             }
           }
-          const int sig = (g0 + nkv - 1) & 1;
+          const int sig = (g0 + nks - 1) & 1;
           uint8_t* stage = sm.k[sig] + (warp & 3) * (2 * 4096) + qt * 4096;
           const float inv = 1.0f / l;
 #pragma unroll
@@ -1082,24 +1091,24 @@ struct WindowPlan {
 };
 
 // The cheapest of the four plans by a launch-time model. A unit takes about 1.7 us per KV step of a
-// softmax warpgroup (half of the KV tiles in a one-tile unit, whose keys its two warpgroups split;
-// that takes an even number of tiles, and an odd one keeps the square launch's bits) and 2 us
-// around them, and the persistent grid runs rounds of n_sm units. On equal cost the units stay
-// unpacked, whose rows spread over more SMs. us measured, unpacked with one / two tiles a unit and
+// softmax warpgroup (half of the KV tiles, rounded up, in a one-tile unit, whose keys its two
+// warpgroups split) and 2 us around them, and the persistent grid runs rounds of n_sm units. On
+// equal cost the units stay unpacked, whose rows spread over more SMs. us measured, unpacked with one / two tiles a unit and
 // packed with one / two (B, heads, keys, rows):
 //   8, 32/8, 2048, 64:  38.7 / 61.3 / 21.5 / 33.0    12, 32/8, 2000, 17: 55.4 / 88.3 / 21.9 / 35.3
 //   8, 28/4, 1024, 32:  23.5 / 35.4 / 13.1 / 19.2    6, 28/4, 1500, 100: 30.6 / 47.4 / 18.1 / 26.1
-//   4, 28/4, 1024, 32:  13.0 / 19.5 / 13.0 / 19.3    8, 32/8, 1100, 64:  34.7 / 41.8 / 20.0 / 22.2
+//   4, 28/4, 1024, 32:  13.0 / 19.5 / 13.0 / 19.3    8, 32/8, 1100, 64:  (packed, one tile) 17.0
 //   2, 32/32, 2048, 200: 21.1 / 32.9                 3, 32/32, 2048, 200: 38.7 / 36.6
-// (before, a window was unpacked, with one tile a unit up to 128 rows and two above).
+// Before, a window was unpacked, with one tile a unit up to 128 rows and two above, and its keys were
+// split for an even number of KV tiles only: 2, 32/32, 3400, 100 (27 tiles) 42.2 -> 30.8; 1, 32/32,
+// 640, 64 (5 tiles) 11.5 -> 10.4; 8, 32/8, 1100, 64 (9 tiles) 34.4 -> 17.0.
 WindowPlan plan_window(const AttnArgs& a, int n_sm) {
   const int G = a.Hq / a.Hkv, nkv = (a.L + kBN - 1) / kBN;
-  const bool even = nkv % 2 == 0;
   WindowPlan best{false, a.Lq <= kBM ? 1 : 2, 0.0};
   const auto us = [&](bool pack, int nq) {
     const long long rows = pack ? static_cast<long long>(G) * a.Lq : a.Lq;
     const long long units = (rows + nq * kBM - 1) / (nq * kBM) * a.B * (pack ? a.Hkv : a.Hq);
-    const int steps = nq == 1 && even ? nkv / 2 : nkv;
+    const int steps = nq == 1 ? (nkv + 1) / 2 : nkv;
     return static_cast<double>((units + n_sm - 1) / n_sm) * (2.0 + 1.7 * steps) + 3.0;
   };
   best.us = us(best.pack, best.nq);
@@ -1107,7 +1116,7 @@ WindowPlan plan_window(const AttnArgs& a, int n_sm) {
     const double t = us(pack, nq);
     if (t < best.us) best = WindowPlan{pack, nq, t};
   };
-  if (even || a.Lq <= kBM) consider(false, 1);
+  consider(false, 1);
   consider(false, 2);
   if (G > 1 && static_cast<long long>(G) * a.Lq <= 0x7fffffffLL / 2) {
     consider(true, 2);
@@ -1159,7 +1168,8 @@ int launch_attn_bf16_sm103(const AttnArgs& args, int* status, cudaStream_t strea
   const int rc = setup.get(&unused, [&](int&) {
     for (auto fn : {attn_bf16_kernel<2, false, false>, attn_bf16_kernel<1, true, false>,
                     attn_bf16_kernel<2, true, false>, attn_bf16_kernel<2, false, true>,
-                    attn_bf16_kernel<1, true, true>, attn_bf16_kernel<2, true, true>}) {
+                    attn_bf16_kernel<1, true, true>, attn_bf16_kernel<2, true, true>,
+                    attn_bf16_kernel<2, false, false, true>, attn_bf16_kernel<2, false, true, true>}) {
       if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return -3;
       // the register split inside the kernel assumes exactly kLaunchRegs per thread at launch;
@@ -1173,14 +1183,14 @@ int launch_attn_bf16_sm103(const AttnArgs& args, int* status, cudaStream_t strea
   // unit indices advance by the grid size past the last unit: keep them inside int
   if (n_units > 0x7fffffffLL - n_sm) return -2;
   // persistent grid: one CTA per SM (1 CTA/SM fits), each looping over units
-  // The last round of units would leave at least half of the SMs idle: split its units
-  // (square launches with an even number of KV tiles), two CTAs per unit.
+  // The last round of units would leave at least half of the SMs idle: split its units (square
+  // launches), two CTAs per unit; with an odd number of KV tiles only where it is the only round.
   const long long rounds = n_units / n_sm, n_last = n_units % n_sm;
-  // One-tile units of a window are split inside their CTAs when the number of KV tiles is even
-  // (both softmax warpgroups on the two halves of the keys).
-  const bool split_all = nq == 1 && nkv % 2 == 0;
+  // One-tile units of a window are split inside their CTAs (both softmax warpgroups on the two
+  // halves of the keys).
+  const bool split_all = nq == 1 && nkv >= 2;
   const int n_split = split_all ? static_cast<int>(n_units)
-                      : (!window && nkv >= 2 && nkv % 2 == 0 && n_last > 0 && 2 * n_last <= n_sm)
+                      : (!window && nkv >= 2 && (nkv % 2 == 0 || rounds == 0) && n_last > 0 && 2 * n_last <= n_sm)
                           ? static_cast<int>(n_last) : 0;
   const int n_reg = split_all ? 0 : static_cast<int>(n_units) - n_split;
   const long long grid = split_all ? (rounds > 0 ? n_sm : n_units)
@@ -1190,7 +1200,9 @@ int launch_attn_bf16_sm103(const AttnArgs& args, int* status, cudaStream_t strea
                     make_fastdiv(static_cast<uint32_t>(a.Hq)), make_fastdiv(static_cast<uint32_t>(a.Hq / a.Hkv)),
                     make_fastdiv(static_cast<uint32_t>(period))};
   const bool fault = a.fault_cta >= 0 || a.wait_ns > 0;
-  auto kernel = !window       ? (fault ? attn_bf16_kernel<2, false, true> : attn_bf16_kernel<2, false, false>)
+  const bool pad = n_split > 0 && nkv % 2 != 0;
+  auto kernel = !window && pad ? (fault ? attn_bf16_kernel<2, false, true, true> : attn_bf16_kernel<2, false, false, true>)
+                : !window     ? (fault ? attn_bf16_kernel<2, false, true> : attn_bf16_kernel<2, false, false>)
                 : nq == 1     ? (fault ? attn_bf16_kernel<1, true, true> : attn_bf16_kernel<1, true, false>)
                               : (fault ? attn_bf16_kernel<2, true, true> : attn_bf16_kernel<2, true, false>);
   // programmatic dependent launch: the prologue overlaps the previous kernel's tail

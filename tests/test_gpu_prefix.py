@@ -65,11 +65,14 @@ def test_window_bf16(B, Hq, Hkv, Lk, Lq, q0, S, inside):
 @pytest.mark.parametrize("B,Hq,Hkv,Lk,Lq,q0,S,inside", [
     (5, 32, 8, 512, 64, 400, 12, 6),        # 160 units in two rounds unpacked: packed, 256 rows in one-tile units
     (5, 32, 8, 500, 45, 411, 12, 8),        # 180 packed rows: a tile and a ragged one, heads meeting in a warp
-    (6, 28, 4, 640, 33, 97, 10, 6),         # an odd number of KV tiles: packed without a split
+    (6, 28, 4, 640, 33, 97, 10, 6),         # an odd number of KV tiles, packed
     (9, 24, 3, 256, 3, 251, 5, 2),          # 24 packed rows, several heads of a position in one warp
     (20, 16, 2, 130, 1, 64, 3, 1),          # one row per head; 40 packed units against 320
     (1, 3, 3, 512, 200, 250, 8, 5),         # MHA: one-tile split units of a window above 128 rows
     (2, 4, 4, 768, 256, 512, 9, 9),         # the same, every tile full
+    (6, 32, 32, 384, 40, 300, 7, 4),        # three KV tiles: the second half's last one lies past the memory
+    (1, 2, 2, 257, 7, 250, 3, 3),           # one key in the last of three
+    (6, 32, 32, 640, 128, 512, 7, 4),       # the same over several units a CTA
 ])
 def test_window_plans(B, Hq, Hkv, Lk, Lq, q0, S, inside):
     """The launch plans of a window: packed grouped-query heads, one-tile units beyond 128 rows."""
