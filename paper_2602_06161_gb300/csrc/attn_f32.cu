@@ -20,12 +20,13 @@
 // (76 TFLOP/s at 1.95 GHz) are the floor (tensor cores would round the operands), but an FMA whose
 // three operands all come from the register file takes about 1.4 issue slots instead of 1, packed
 // f32x2 (2.8 for two, measured) or not. The packed form leaves issue slots for the rest of the
-// loop: 122 against 143 us with scalar FMAs on 32 heads x 512 rows x 512 keys, D = 128 (35 TFLOP/s;
+// loop: 118 against 143 us with scalar FMAs on 32 heads x 512 rows x 512 keys, D = 128 (36 TFLOP/s;
 // one warp per row with a shuffle reduction per key took 1140 us). Two other layouts measured the
 // same there: eight warps with half the register tile (125 us), and lanes whose shared-memory reads
 // do not merge (124 us).
 #include <math.h>
 
+#include "cluster.cuh"
 #include "context.cuh"
 #include "kernels.cuh"
 #include "ptx.cuh"
@@ -79,7 +80,23 @@ __device__ __forceinline__ void load_rows(float* dst, const float* __restrict__ 
   }
 }
 
-template <int D, int TM>
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 ld_cluster2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+
+// C > 1: the keys of a row tile are split over the C CTAs of a cluster. Each leaves its (m, l, O) in
+// its own shared memory, and CTA k combines rows k, k + C, ... from all of them.
+template <int D, int TM, int C>
 __global__ void __launch_bounds__(kThreads, 2)
     attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ kc, const float* __restrict__ vc,
                     const float* __restrict__ km, const float* __restrict__ vm, const int32_t* __restrict__ seed_idx,
@@ -98,21 +115,26 @@ __global__ void __launch_bounds__(kThreads, 2)
   // a half-warp's 16-byte shared-memory reads merge into one access when lanes i, i ^ 1 or lanes
   // i, i ^ 2 read the same address: tx comes in adjacent pairs, tyl alternates
   const int tx = (lane >> 1) & 7, tyl = (lane & 1) | (lane >> 4) << 1;
-  const unsigned head = blockIdx.x / static_cast<unsigned>(tiles);        // b * Hq + hq
-  const int row0 = static_cast<int>(blockIdx.x - head * tiles) * T::kBM;  // first query row of the tile
+  const int rank = C > 1 ? static_cast<int>(cluster_ctarank()) : 0;
+  const unsigned unit = blockIdx.x / C;
+  const unsigned head = unit / static_cast<unsigned>(tiles);        // b * Hq + hq
+  const int row0 = static_cast<int>(unit - head * tiles) * T::kBM;  // first query row of the tile
   const int b = static_cast<int>(head / static_cast<unsigned>(Hq)), hq = static_cast<int>(head - b * Hq);
   const size_t kv_head = static_cast<size_t>(b) * Hkv + hq / (Hq / Hkv);
   const float* const k_base = kc + kv_head * L * D;
   const float* const v_base = vc + kv_head * L * D;
   const float scale = 1.0f / sqrtf(static_cast<float>(D));
-  const int n_kv = (L + kBN - 1) / kBN;
+  const int n_all = (L + kBN - 1) / kBN;
+  // this CTA's key tiles (at least one: C <= n_all)
+  const int j0 = C > 1 ? static_cast<int>(static_cast<long long>(rank) * n_all / C) : 0;
+  const int n_kv = C > 1 ? static_cast<int>(static_cast<long long>(rank + 1) * n_all / C) : n_all;
 
   route_clear(slot, T::kBM, threadIdx.x, kThreads);
   griddep_wait();
   load_rows<D, T::kBM, true>(sq, q + (static_cast<size_t>(head) * Lq + row0) * D, Lq - row0, vec);
-  load_rows<D, kBN, true>(sk, k_base, L, vec);
+  load_rows<D, kBN, true>(sk, k_base + static_cast<size_t>(j0) * kBN * D, L - j0 * kBN, vec);
   cp_async_commit();
-  load_rows<D, kBN, false>(sv, v_base, L, vec);
+  load_rows<D, kBN, false>(sv, v_base + static_cast<size_t>(j0) * kBN * D, L - j0 * kBN, vec);
   cp_async_commit();
   __syncthreads();
   route_scan(slot, seed_idx + static_cast<size_t>(b) * n_seeds, n_seeds, q0 + row0, T::kBM, L, threadIdx.x, kThreads);
@@ -129,39 +151,55 @@ __global__ void __launch_bounds__(kThreads, 2)
   }
   int diag[TM];   // key column of a seed row's excluded diagonal term
 
-  for (int j = 0; j < n_kv; ++j) {
+  for (int j = j0; j < n_kv; ++j) {
     cp_async_wait<1>();   // K(j) (and Q) have landed; V(j) may be in flight
     __syncthreads();
-    if (j == 0) {
+    if (j == j0) {
 #pragma unroll
       for (int i = 0; i < TM; ++i) diag[i] = slot[r0 + 4 * i] != kNoSlot ? q0 + row0 + r0 + 4 * i : -1;
     }
-    // ---- scores: partial sums over even and odd d in the two halves of a pair ----
-    uint64_t s2[TM][8];
+    // ---- scores: partial sums over even and odd d in the two halves of a pair, and over kParts
+    // stretches of d where there are registers for it (a dot product's rounding error grows with
+    // its longest chain) ----
+    constexpr int kParts = TM == 1 ? 4 : TM == 2 ? 2 : 1;
+    float dots[TM][8];
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
+    for (int part = 0; part < kParts; ++part) {
+      uint64_t s2[TM][8];
 #pragma unroll
-      for (int jj = 0; jj < 8; ++jj) s2[i][jj] = 0;
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int jj = 0; jj < 8; ++jj) s2[i][jj] = 0;
 #pragma unroll 4
-    for (int c = 0; c < D / 4; ++c) {
-      ulonglong2 qa[TM];
+      for (int c = part * (D / 4 / kParts); c < (part + 1) * (D / 4 / kParts); ++c) {
+        ulonglong2 qa[TM];
 #pragma unroll
-      for (int i = 0; i < TM; ++i) {
-        const int r = r0 + 4 * i;
-        qa[i] = lds2(sq + r * D + 4 * (c ^ (r & 7)));
+        for (int i = 0; i < TM; ++i) {
+          const int r = r0 + 4 * i;
+          qa[i] = lds2(sq + r * D + 4 * (c ^ (r & 7)));
+        }
+        const float* kp = sk + tx * D + 4 * (c ^ tx);
+#pragma unroll
+        for (int jj = 0; jj < 8; ++jj) {
+          const ulonglong2 ka = lds2(kp + 8 * jj * D);
+#pragma unroll
+          for (int i = 0; i < TM; ++i) s2[i][jj] = f2_fma(qa[i].x, ka.x, s2[i][jj]);
+#pragma unroll
+          for (int i = 0; i < TM; ++i) s2[i][jj] = f2_fma(qa[i].y, ka.y, s2[i][jj]);
+        }
       }
-      const float* kp = sk + tx * D + 4 * (c ^ tx);
 #pragma unroll
-      for (int jj = 0; jj < 8; ++jj) {
-        const ulonglong2 ka = lds2(kp + 8 * jj * D);
+      for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int i = 0; i < TM; ++i) s2[i][jj] = f2_fma(qa[i].x, ka.x, s2[i][jj]);
-#pragma unroll
-        for (int i = 0; i < TM; ++i) s2[i][jj] = f2_fma(qa[i].y, ka.y, s2[i][jj]);
-      }
+        for (int jj = 0; jj < 8; ++jj) {
+          float lo, hi;
+          f2_unpack(s2[i][jj], lo, hi);
+          dots[i][jj] = part == 0 ? lo + hi : dots[i][jj] + (lo + hi);
+        }
     }
     __syncthreads();   // every warp is done with K(j)
-    if (j + 1 < n_kv) load_rows<D, kBN, true>(sk, k_base + static_cast<size_t>(j + 1) * kBN * D, L - (j + 1) * kBN, vec);
+    if (j + 1 < n_kv)
+      load_rows<D, kBN, true>(sk, k_base + static_cast<size_t>(j + 1) * kBN * D, L - (j + 1) * kBN, vec);
     cp_async_commit();
     // ---- online softmax of this thread's rows; P to shared memory ----
     const int key0 = j * kBN + tx;
@@ -172,10 +210,8 @@ __global__ void __launch_bounds__(kThreads, 2)
       float s[8], mx = -INFINITY;
 #pragma unroll
       for (int jj = 0; jj < 8; ++jj) {
-        float lo, hi;
-        f2_unpack(s2[i][jj], lo, hi);
         const int key = key0 + 8 * jj;
-        s[jj] = (lo + hi) * scale;
+        s[jj] = dots[i][jj] * scale;
         if (masked && (key >= L || key == diag[i])) s[jj] = -INFINITY;
         mx = fmaxf(mx, s[jj]);
       }
@@ -227,101 +263,197 @@ __global__ void __launch_bounds__(kThreads, 2)
       }
     }
     __syncthreads();   // every warp is done with V(j)
-    if (j + 1 < n_kv) load_rows<D, kBN, false>(sv, v_base + static_cast<size_t>(j + 1) * kBN * D, L - (j + 1) * kBN, vec);
+    if (j + 1 < n_kv)
+      load_rows<D, kBN, false>(sv, v_base + static_cast<size_t>(j + 1) * kBN * D, L - (j + 1) * kBN, vec);
     cp_async_commit();
   }
 
+  if constexpr (C > 1) {
+    // this split's rows to shared memory (every warp is done with K and V): O over the K tile,
+    // (m, l) over the V tile
+    float2* const ml = reinterpret_cast<float2*>(sv);
 #pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    const int r = r0 + 4 * i;
+    for (int i = 0; i < TM; ++i) {
+      const int r = r0 + 4 * i;
 #pragma unroll
-    for (int off = 8; off > 1; off >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
-    const int sl = slot[r];
-    if (__any_sync(0xffffffffu, sl != kNoSlot)) {
-      // merge the masked-input self term (k_i, v_i) of the warp's seed rows
+      for (int off = 8; off > 1; off >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
+#pragma unroll
+      for (int c = 0; c < kC; ++c)
+        *reinterpret_cast<ulonglong2*>(sk + r * D + 32 * c + 4 * tx) = make_ulonglong2(o[i][2 * c], o[i][2 * c + 1]);
+      if (tx == 0) ml[r] = make_float2(m[i], l[i]);
+    }
+    cluster_sync();
+    // D / 4 lanes of a warp take a row, four columns each
+    constexpr int kLanes = D / 4;
+    for (int e = threadIdx.x; e < T::kBM / C * kLanes; e += kThreads) {
+      const int r = e / kLanes * C + rank, c4 = e % kLanes;
+      float2 st[C];
+      float mm = -INFINITY;
+#pragma unroll
+      for (int k = 0; k < C; ++k) {
+        st[k] = ld_cluster2(cluster_map(smem_u32(ml + r), k));
+        mm = fmaxf(mm, st[k].x);
+      }
+      const int sl = slot[r];
       const bool is_seed = sl != kNoSlot;
-      const size_t mrow = (kv_head * n_seeds + (is_seed ? sl : 0)) * D;
+      const size_t mrow = (kv_head * n_seeds + (is_seed ? sl : 0)) * D + 4 * c4;
       float dot = 0.0f;
       if (is_seed) {
-#pragma unroll
-        for (int c = tx; c < D / 4; c += 8) {
-          const float4 qv = *reinterpret_cast<const float4*>(sq + r * D + 4 * (c ^ (r & 7)));
-          const float* kp = km + mrow + 4 * c;
-          dot = fmaf(qv.x, kp[0], fmaf(qv.y, kp[1], fmaf(qv.z, kp[2], fmaf(qv.w, kp[3], dot))));
-        }
+        const float4 qv = *reinterpret_cast<const float4*>(sq + r * D + 4 * (c4 ^ (r & 7)));
+        dot = fmaf(qv.x, km[mrow], fmaf(qv.y, km[mrow + 1], fmaf(qv.z, km[mrow + 2], qv.w * km[mrow + 3])));
       }
 #pragma unroll
-      for (int off = 8; off > 1; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-      if (is_seed) {
-        const float s = dot * scale;
-        const float m_new = fmaxf(m[i], s);
-        const float a = (m[i] == -INFINITY) ? 0.0f : expf(m[i] - m_new);
-        const float p = expf(s - m_new);
-        l[i] = l[i] * a + p;
-        m[i] = m_new;
-        const uint64_t aa = f2_pack(a, a), pp = f2_pack(p, p);
+      for (int off = kLanes / 2; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+      const float s_self = is_seed ? dot * scale : -INFINITY;
+      mm = fmaxf(mm, s_self);
+      const float ref = mm == -INFINITY ? 0.0f : mm;
+      float ll = 0.0f;
+      float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-        for (int c = 0; c < kC; ++c) {
-          const float* vp = vm + mrow + 32 * c + 4 * tx;
-          o[i][2 * c] = f2_fma(pp, f2_pack(vp[0], vp[1]), f2_mul(o[i][2 * c], aa));
-          o[i][2 * c + 1] = f2_fma(pp, f2_pack(vp[2], vp[3]), f2_mul(o[i][2 * c + 1], aa));
+      for (int k = 0; k < C; ++k) {
+        const float w = expf(st[k].x - ref);
+        const float4 x = ld_cluster4(cluster_map(smem_u32(sk + r * D + 4 * c4), k));
+        ll = fmaf(w, st[k].y, ll);
+        acc.x = fmaf(w, x.x, acc.x);
+        acc.y = fmaf(w, x.y, acc.y);
+        acc.z = fmaf(w, x.z, acc.z);
+        acc.w = fmaf(w, x.w, acc.w);
+      }
+      if (is_seed) {
+        // the masked-input self term (k_i, v_i)
+        const float p = expf(s_self - ref);
+        ll += p;
+        acc.x = fmaf(p, vm[mrow], acc.x);
+        acc.y = fmaf(p, vm[mrow + 1], acc.y);
+        acc.z = fmaf(p, vm[mrow + 2], acc.z);
+        acc.w = fmaf(p, vm[mrow + 3], acc.w);
+      }
+      if (row0 + r < Lq) {
+        const float inv = 1.0f / ll;
+        const size_t row = static_cast<size_t>(head) * Lq + row0 + r;
+        float* op = out + row * D + 4 * c4;
+        if (vec) {
+          *reinterpret_cast<float4*>(op) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+        } else {
+          op[0] = acc.x * inv;
+          op[1] = acc.y * inv;
+          op[2] = acc.z * inv;
+          op[3] = acc.w * inv;
         }
+        if (lse != nullptr && c4 == 0) lse[row] = mm + logf(ll);
       }
     }
-    if (row0 + r < Lq) {
-      const float inv = 1.0f / l[i];
-      const size_t row = static_cast<size_t>(head) * Lq + row0 + r;
+    cluster_sync();   // no CTA leaves while another reads its shared memory
+  } else {
 #pragma unroll
-      for (int c = 0; c < kC; ++c) {
-        float x0, x1, x2, x3;
-        f2_unpack(o[i][2 * c], x0, x1);
-        f2_unpack(o[i][2 * c + 1], x2, x3);
-        float* op = out + row * D + 32 * c + 4 * tx;
-        if (vec) {
-          *reinterpret_cast<float4*>(op) = make_float4(x0 * inv, x1 * inv, x2 * inv, x3 * inv);
-        } else {
-          op[0] = x0 * inv;
-          op[1] = x1 * inv;
-          op[2] = x2 * inv;
-          op[3] = x3 * inv;
+    for (int i = 0; i < TM; ++i) {
+      const int r = r0 + 4 * i;
+#pragma unroll
+      for (int off = 8; off > 1; off >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
+      const int sl = slot[r];
+      if (__any_sync(0xffffffffu, sl != kNoSlot)) {
+        // merge the masked-input self term (k_i, v_i) of the warp's seed rows
+        const bool is_seed = sl != kNoSlot;
+        const size_t mrow = (kv_head * n_seeds + (is_seed ? sl : 0)) * D;
+        float dot = 0.0f;
+        if (is_seed) {
+#pragma unroll
+          for (int c = tx; c < D / 4; c += 8) {
+            const float4 qv = *reinterpret_cast<const float4*>(sq + r * D + 4 * (c ^ (r & 7)));
+            const float* kp = km + mrow + 4 * c;
+            dot = fmaf(qv.x, kp[0], fmaf(qv.y, kp[1], fmaf(qv.z, kp[2], fmaf(qv.w, kp[3], dot))));
+          }
+        }
+#pragma unroll
+        for (int off = 8; off > 1; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+        if (is_seed) {
+          const float s = dot * scale;
+          const float m_new = fmaxf(m[i], s);
+          const float a = (m[i] == -INFINITY) ? 0.0f : expf(m[i] - m_new);
+          const float p = expf(s - m_new);
+          l[i] = l[i] * a + p;
+          m[i] = m_new;
+          const uint64_t aa = f2_pack(a, a), pp = f2_pack(p, p);
+#pragma unroll
+          for (int c = 0; c < kC; ++c) {
+            const float* vp = vm + mrow + 32 * c + 4 * tx;
+            o[i][2 * c] = f2_fma(pp, f2_pack(vp[0], vp[1]), f2_mul(o[i][2 * c], aa));
+            o[i][2 * c + 1] = f2_fma(pp, f2_pack(vp[2], vp[3]), f2_mul(o[i][2 * c + 1], aa));
+          }
         }
       }
-      if (lse != nullptr && tx == 0) lse[row] = m[i] + logf(l[i]);
+      if (row0 + r < Lq) {
+        const float inv = 1.0f / l[i];
+        const size_t row = static_cast<size_t>(head) * Lq + row0 + r;
+#pragma unroll
+        for (int c = 0; c < kC; ++c) {
+          float x0, x1, x2, x3;
+          f2_unpack(o[i][2 * c], x0, x1);
+          f2_unpack(o[i][2 * c + 1], x2, x3);
+          float* op = out + row * D + 32 * c + 4 * tx;
+          if (vec) {
+            *reinterpret_cast<float4*>(op) = make_float4(x0 * inv, x1 * inv, x2 * inv, x3 * inv);
+          } else {
+            op[0] = x0 * inv;
+            op[1] = x1 * inv;
+            op[2] = x2 * inv;
+            op[3] = x3 * inv;
+          }
+        }
+        if (lse != nullptr && tx == 0) lse[row] = m[i] + logf(l[i]);
+      }
     }
   }
 }
 
-template <int D, int TM>
+template <int D, int TM, int C = 1>
 int launch_tile(const AttnArgs& a, bool vec, cudaStream_t stream) {
   static ContextCache<int> cache;
   int ready = 0;
   const int rc = cache.get(&ready, [](int& v) {
     v = 1;
-    return cudaFuncSetAttribute(attn_f32_kernel<D, TM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(attn_f32_kernel<D, TM, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 static_cast<int>(F32Tile<D, TM>::kBytes)) == cudaSuccess ? 0 : -3;
   });
   if (rc != 0) return rc;
   const int tiles = (a.Lq + F32Tile<D, TM>::kBM - 1) / F32Tile<D, TM>::kBM;
-  const long long blocks = static_cast<long long>(a.B) * a.Hq * tiles;
+  const long long blocks = static_cast<long long>(a.B) * a.Hq * tiles * C;
   if (blocks > 0x7fffffffLL) return -2;
-  cudaLaunchAttribute attr[1];
-  const cudaLaunchConfig_t cfg =
-      pdl_config(dim3(static_cast<unsigned>(blocks)), dim3(kThreads), F32Tile<D, TM>::kBytes, stream, attr);
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = C;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(blocks));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = F32Tile<D, TM>::kBytes;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = C > 1 ? 2 : 1;
   const cudaError_t err = cudaLaunchKernelEx(
-      &cfg, attn_f32_kernel<D, TM>, static_cast<const float*>(a.q), static_cast<const float*>(a.k_cached),
+      &cfg, attn_f32_kernel<D, TM, C>, static_cast<const float*>(a.q), static_cast<const float*>(a.k_cached),
       static_cast<const float*>(a.v_cached), static_cast<const float*>(a.k_seedmask),
       static_cast<const float*>(a.v_seedmask), a.seed_idx, a.n_seeds, a.Hq, a.Hkv, a.Lq, a.L, a.q0, tiles,
       vec ? 1 : 0, static_cast<float*>(a.out), a.lse);
   return err == cudaSuccess ? 0 : -3;
 }
 
-// Rows per CTA: a launch lasts about as long as the SM with the most CTAs, so the cost of 16 TM
-// rows a CTA is ceil(CTAs / SMs) times a CTA's cost, which the shared K / V work keeps from falling
-// with TM: 32, 43, 75 for TM = 1, 2, 4 (in rows of the FMA pipe's rate; fitted to the first and
-// fourth shape below). us at TM = 1 / 2 / 4 (heads x rows x keys, D): 32 x 512 x 512, 128: 177 / 136
-// / 119; 8 x 512 x 512, 128: 50 / 42 / 69; 4 x 256 x 256, 64: 11.3 / 13.8 / 20.8; 32 x 300 x 300, 128:
-// 63 / 66 / 76; 16 x 700 x 700, 64: 97 / 80 / 87; 32 x 32 x 1024, 128: 66 / 80 / 132. The rule takes
-// the fastest on each.
+// Rows per CTA and key split, by the launch's predicted time. A CTA takes t us a key tile (alone on
+// its SM, or less where an SM has several, which overlap) and 2 us around them; an SM with w CTAs runs
+// them in w turns; combining a split costs 1 us. t as measured at D = 128 (TM = 1, 2, 4: 4.1, 5.0,
+// 8.2 alone, 3.15, 4.25, 7.4 shared), about half of it at D = 64. us measured at the candidates:
+//   heads x rows x keys, D      TM = 1 / 2 / 4 unsplit     TM = 1 split in 2 / 4 / 8   TM = 2 in 2 / 4
+//   32 x 512 x 512, 128         177 / 136 / 119
+//   8 x 512 x 512, 128          50 / 42 / 69
+//   32 x 300 x 300, 128         63 / 66 / 76
+//   8 x 100 x 1000, 128         65 / 80 / 131              36 / 28 / 31                44 / 24
+//   2 x 1000 x 1000, 128        65                         51 / 54 / 61                44 / 39
+//   4 x 256 x 256, 64           10.6 / 13.8 / 20.8         7.5 / 6.8
+//   5 x 20 x 600, 64            22.4                       13.4 / 9.4 / 7.4
+// Unsplit, a few rows over many keys left most SMs idle for the whole chain of key tiles.
 template <int D>
 int launch_rows(const AttnArgs& a, bool vec, cudaStream_t stream) {
   static ContextCache<int> cache;
@@ -332,14 +464,29 @@ int launch_rows(const AttnArgs& a, bool vec, cudaStream_t stream) {
     return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? 0 : -3;
   });
   if (rc != 0) return rc;
-  const auto cost = [&](int rows, int cta_cost) {
-    const long long ctas = static_cast<long long>(a.B) * a.Hq * ((a.Lq + rows - 1) / rows);
-    return (ctas + n_sm - 1) / n_sm * cta_cost;
+  const int n_kv = (a.L + kBN - 1) / kBN;
+  double best = 0.0;
+  int tm = 0, split = 0;
+  const auto consider = [&](int t, int c, double alone, double shared) {
+    if (c > n_kv) return;
+    const long long ctas = static_cast<long long>(a.B) * a.Hq * ((a.Lq + 16 * t - 1) / (16 * t)) * c;
+    const long long w = (ctas + n_sm - 1) / n_sm;
+    const double us = w * (2.0 + (n_kv + c - 1) / c * (w == 1 ? alone : shared) * (D == 64 ? 0.53 : 1.0)) + (c > 1);
+    if (tm == 0 || us < best) best = us, tm = t, split = c;
   };
-  const long long c16 = cost(16, 32), c32 = cost(32, 43), c64 = cost(64, 75);
-  if (c64 <= c32 && c64 <= c16) return launch_tile<D, 4>(a, vec, stream);
-  if (c32 <= c16) return launch_tile<D, 2>(a, vec, stream);
-  return launch_tile<D, 1>(a, vec, stream);
+  consider(4, 1, 8.2, 7.4);
+  for (const int c : {1, 2, 4}) consider(2, c, 5.0, 4.25);
+  for (const int c : {1, 2, 4, 8}) consider(1, c, 4.1, 3.15);
+  switch (100 * tm + split) {
+    case 401: return launch_tile<D, 4>(a, vec, stream);
+    case 201: return launch_tile<D, 2>(a, vec, stream);
+    case 202: return launch_tile<D, 2, 2>(a, vec, stream);
+    case 204: return launch_tile<D, 2, 4>(a, vec, stream);
+    case 102: return launch_tile<D, 1, 2>(a, vec, stream);
+    case 104: return launch_tile<D, 1, 4>(a, vec, stream);
+    case 108: return launch_tile<D, 1, 8>(a, vec, stream);
+    default: return launch_tile<D, 1>(a, vec, stream);
+  }
 }
 
 }  // namespace

@@ -101,6 +101,31 @@ def test_f32_row_tiles(B, Hq, Hkv, L, D, S):
     H.assert_f32_close(out, ref, lse, ref_lse)
 
 
+@pytest.mark.parametrize("Hq,Hkv,Lk,D,Lq,q0,S", [
+    (2, 1, 128, 64, 128, 0, 5),       # 16 rows a CTA, two splits of one key tile
+    (4, 4, 256, 64, 256, 0, 9),       # two splits of two
+    (5, 1, 600, 64, 20, 577, 4),      # eight splits of one or two tiles, the last ragged; seeds in the window
+    (1, 1, 520, 128, 7, 511, 3),      # eight splits of nine tiles; one key in the last
+    (8, 2, 1000, 128, 100, 440, 40),  # 32 rows a CTA, four splits
+    (16, 4, 300, 128, 100, 200, 7),   # 32 rows, two splits of five tiles
+    (3, 3, 65, 128, 1, 64, 1),        # one row, a seed whose diagonal is the only key of the second split
+])
+def test_f32_key_split(Hq, Hkv, Lk, D, Lq, q0, S):
+    """The fp32 kernel's key splits over a cluster (152 SMs choose as noted)."""
+    full = W.make_attn_inputs(2 if Lq < 30 else 1, Hq, Hkv, Lk, D, S, dtype="f32", seed=Lk + Lq, seed_lo=max(0, q0 - 2),
+                              seed_hi=Lk)
+    if Lq == 1:
+        full.seed_idx[:] = q0
+    dev = [H.to_dev(x, "f32") for x in (np.ascontiguousarray(full.q[:, :, q0:q0 + Lq]), full.k_cached, full.v_cached,
+                                        full.k_seedmask, full.v_seedmask)]
+    out, lse = api.cover_attn_fwd_prefix_f32(*dev, H.to_dev(full.seed_idx, "i32"), q0=q0)
+    torch.cuda.synchronize()
+    f = lambda x: x.astype(np.float64)   # noqa: E731
+    ref, ref_lse = oracle.override_attention_window(f(full.q[:, :, q0:q0 + Lq]), f(full.k_cached), f(full.v_cached),
+                                                    f(full.k_seedmask), f(full.v_seedmask), full.seed_idx, q0)
+    H.assert_f32_close(out.cpu().numpy(), ref, lse.cpu().numpy(), ref_lse)
+
+
 @pytest.mark.parametrize("which", range(4))
 def test_f32_unaligned_rows_equal_aligned(which):
     """A tensor that is only 4-byte aligned takes the 4-byte copies: the same bits."""
