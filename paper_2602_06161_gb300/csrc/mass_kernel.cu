@@ -27,18 +27,19 @@
 //
 // A CTA keeps Q_t and K_t of NT tiles of one head resident: they serve as the A operands of both
 // orientations and as the B operands of the products among themselves; the block's other tiles
-// stream through a two-slot ring. Each of the two warpgroups of the math threads takes the products
-// of one tile (NT = 2) or of one orientation (NT = 1) from two tensor-memory buffers, so a product
-// overlaps the previous one's exponentials.
+// stream through a two-slot ring. The math warpgroups take the products of one tile each (NT = 2,
+// two warpgroups a tile, 64 columns each) or of one orientation each (NT = 1) from two tensor-memory
+// buffers, so a product overlaps the previous one's exponentials.
 //
 // Bound: latency and, with many heads, reading Q and K once (8 x 32 heads x 256 rows: 34 MB, 5 us).
 // With NT = 2 a head's 256-row block is one CTA that reads it once, instead of four CTAs (one per
-// tile and orientation) reading three tiles each: 29.1 -> 19.4 us there (both launches), 16.6 ->
-// 10.2 us with 4 x 32 heads. What is left is a CTA's chain (column data, tile loads, four products
-// and their exponentials, about 8 us) in ceil(CTAs / SMs) waves.
+// tile and orientation) reading three tiles each: 29.1 -> 17.9 us there (both launches), 16.6 -> 9.4
+// us with 4 x 32 heads, 53.7 -> 34.7 us with 8 x 28/4 heads and 512 rows. What is left is a CTA's
+// chain in ceil(CTAs / SMs) waves, about 8 us: its tiles and seed keys from DRAM (2 to 4 us, while
+// every SM loads), four products' exponentials (half a microsecond each), 1.2 us until the next CTA.
 //
-// Warps: 0-7 rows / keys of the tiles (thread = tensor-memory lane), 8 issues the TMA loads (lane
-// 0), 9 allocates tensor memory and issues the products (lane 0).
+// Warps: the math warps (thread = tensor-memory lane, a row / key of a tile), then one whose lane 0
+// issues the TMA loads and one that allocates tensor memory and whose lane 0 issues the products.
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -53,10 +54,15 @@ namespace {
 
 constexpr int kD = 128;
 constexpr int kT = 128;                     // rows / keys per tile
-constexpr int kMathThreads = 256;           // two warpgroups
-constexpr int kTmaWarp = 8;
-constexpr int kMmaWarp = 9;
-constexpr int kThreads = 320;
+// Math warps: two warpgroups (one per tile with NT = 2, one per orientation with NT = 1); with NT = 2
+// there are two of each, taking 64 of a product's 128 columns each.
+template <int NT>
+struct MassRoles {
+  static constexpr int kHalves = NT == 2 ? 2 : 1;
+  static constexpr int kMathWarps = 8 * kHalves;
+  static constexpr int kTmaWarp = kMathWarps, kMmaWarp = kMathWarps + 1;
+  static constexpr int kThreads = 32 * (kMathWarps + 2);
+};
 constexpr int kTileBytes = kT * kD * 2;     // 32 KB
 constexpr int kBoxBytes = kTileBytes / 2;   // one 64-column, 128-byte-swizzled box
 constexpr int kMaxPer = kMassMaxPer;        // per-column staging must fit in shared memory
@@ -72,6 +78,7 @@ struct alignas(128) MassCtrl {
   uint32_t tmem_base;
   int abort;
   int slot[2 * kT];                         // seed slot of the resident tiles' positions
+  float half1[2][2][kT];                    // [tile][kind] sums over columns 64 .. 127 (NT = 2)
 };
 
 // Shared memory: NT Q tiles | NT K tiles | kSlots ring slots (when the block has more than NT tiles) |
@@ -83,36 +90,17 @@ size_t mass_smem_bytes(int NT, int n_t) {
          static_cast<size_t>(n_t) * (8 * sizeof(uint32_t) + kT * sizeof(float)) + 1024;
 }
 
-// q . k over the 128 dimensions: q is row r of a 128-byte-swizzled tile in shared memory, k a row
-// in global memory.
-__device__ __forceinline__ float dot_row(const uint8_t* qtile, int r, const __nv_bfloat16* krow) {
-  const uint4* kv = reinterpret_cast<const uint4*>(krow);
-  float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-  for (int ch = 0; ch < 16; ++ch) {
-    const uint4 a = *reinterpret_cast<const uint4*>(qtile + (ch >> 3) * kBoxBytes + r * 128 +
-                                                    (((ch & 7) ^ (r & 7)) << 4));
-    const uint4 b = __ldg(kv + ch);
-    const __nv_bfloat162* ap = reinterpret_cast<const __nv_bfloat162*>(&a);
-    const __nv_bfloat162* bp = reinterpret_cast<const __nv_bfloat162*>(&b);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 af = __bfloat1622float2(ap[e]), bf = __bfloat1622float2(bp[e]);
-      d[e] = fmaf(af.x, bf.x, d[e]);
-      d[e] = fmaf(af.y, bf.y, d[e]);
-    }
-  }
-  return (d[0] + d[1]) + (d[2] + d[3]);
-}
-
 // blockIdx.x = (b * Hq + hq) * n_g + g: tiles NT g .. of head (b, hq).
 template <int NT>
-__global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
+__global__ void __launch_bounds__(MassRoles<NT>::kThreads, NT == 1 ? 2 : 1)
     mass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const __nv_bfloat16* __restrict__ k_seedmask, const int32_t* __restrict__ seed_idx, int n_seeds,
                 const float* __restrict__ lse, int Hq, int Hkv, int L, int pos0, int per, int n_t, int n_g,
                 const int32_t* __restrict__ tok, const uint8_t* __restrict__ flags, int mask_id, float scale_log2,
                 float* __restrict__ part_in, float* __restrict__ part_out, int* status) {
+  using Roles = MassRoles<NT>;
+  constexpr int kTmaWarp = Roles::kTmaWarp, kMmaWarp = Roles::kMmaWarp, kThreads = Roles::kThreads;
+  constexpr int kHalves = Roles::kHalves;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* const base =
       reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -153,7 +141,7 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
       mbar_init(&sm.bar_ring_empty[s], 1);
       for (int u = 0; u < 2; ++u) {
         mbar_init(&sm.bar_s_full[s][u], 1);
-        mbar_init(&sm.bar_s_empty[s][u], 4);
+        mbar_init(&sm.bar_s_empty[s][u], 4 * kHalves);
       }
     }
     mbar_init(&sm.bar_drain, 1);
@@ -202,11 +190,12 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
     }
   }
   // the log2-scaled lse of a math thread's own query (thread = row of its tile)
-  const int g = (warp >> 2) & 1;                       // warpgroup
+  const int g = (warp >> 2) & 1;                       // tile (NT = 2) or orientation (NT = 1) of its products
+  const int half = warp >> 3;                          // and the 64 columns it takes of them (NT = 2)
   const int my = NT == 2 ? g : 0;                      // its resident tile
   const int r = tid & (kT - 1);                        // tensor-memory lane
   const int i = (t0 + my) * kT + r;                    // response index of this thread's query / key
-  const bool valid = warp < kMathThreads / 32 && my < nw && i < per;
+  const bool valid = warp < Roles::kMathWarps && my < nw && i < per;
   const float own = valid ? lse[static_cast<size_t>(bh) * L + pos0 + i] * 1.4426950408889634f : 0.0f;
   tc_fence_before_sync();
   __syncthreads();
@@ -222,6 +211,8 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
   }
   __syncthreads();
   const uint32_t tbase = sm.tmem_base;
+  float sum[2] = {0.0f, 0.0f};   // NT = 2: this thread's sums over its half of the columns
+  bool done = false;             // and whether it adds the other half's and writes them
 
   if (warp == kTmaWarp) {
     if (lane == 0) {
@@ -313,16 +304,62 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
     const uint32_t trow = tbase + (static_cast<uint32_t>((warp & 3) * 32) << 16);
     // the diagonal entry of a seed query uses its masked-input key (leave-one-out view): its score
     // replaces the cached one before the exponentials
-    const int my_slot = valid ? sm.slot[my * kT + r] : kNoSlot;
-    const bool warp_seed = __any_sync(0xffffffffu, my_slot != kNoSlot);
+    // (in the half of the columns that holds the diagonal)
+    const int my_slot = valid && (kHalves == 1 || r / 64 == half) ? sm.slot[my * kT + r] : kNoSlot;
+    uint32_t pending = __ballot_sync(0xffffffffu, my_slot != kNoSlot);
+    const bool warp_seed = pending != 0u;
     float s_self = 0.0f;
     bool ok = true;
     if (warp_seed) {
-      ok = mbar_wait(&sm.bar_q[my], 0, &sm.abort);
-      if (ok && my_slot != kNoSlot)
-        s_self = dot_row(xq + my * kTileBytes, r,
-                         k_seedmask + ((static_cast<size_t>(b) * Hkv + hkv) * n_seeds + my_slot) * kD);
-      ok = __all_sync(0xffffffffu, ok);
+      // four seed rows at a time, eight lanes each (lane l of the eight takes dimensions 16 l .. + 15),
+      // the next four rows' keys on their way; the first ones' are, while the Q tile lands
+      const __nv_bfloat16* km = k_seedmask + (static_cast<size_t>(b) * Hkv + hkv) * n_seeds * kD;
+      const int gl = lane & 7;
+      int src = -1;
+      uint4 kv[2];
+      const auto fetch = [&] {
+        uint32_t p = pending;
+        for (int e = lane >> 3; e > 0; --e) p &= p - 1u;
+        src = p != 0u ? __ffs(p) - 1 : -1;
+        const int sl = __shfl_sync(0xffffffffu, my_slot, src & 31);
+        if (src >= 0) {
+          const uint4* krow = reinterpret_cast<const uint4*>(km + static_cast<size_t>(sl) * kD) + 2 * gl;
+          kv[0] = __ldg(krow);
+          kv[1] = __ldg(krow + 1);
+        }
+      };
+      fetch();
+      ok = __all_sync(0xffffffffu, mbar_wait(&sm.bar_q[my], 0, &sm.abort));
+      const uint8_t* qbox = xq + my * kTileBytes + (gl >> 2) * kBoxBytes;
+#pragma unroll 1
+      while (ok && pending != 0u) {
+        const int from = src;
+        const uint4 k0 = kv[0], k1 = kv[1];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) pending &= pending - 1u;
+        if (pending != 0u) fetch();
+        const int row = (warp & 3) * 32 + (from & 31);
+        float dot = 0.0f;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const uint4 qv = *reinterpret_cast<const uint4*>(qbox + row * 128 + (((2 * (gl & 3) + c) ^ (row & 7)) << 4));
+          const __nv_bfloat162* qp = reinterpret_cast<const __nv_bfloat162*>(&qv);
+          const __nv_bfloat162* kp = reinterpret_cast<const __nv_bfloat162*>(c == 0 ? &k0 : &k1);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float2 qf = __bfloat1622float2(qp[e]), kf = __bfloat1622float2(kp[e]);
+            dot = fmaf(qf.x, kf.x, fmaf(qf.y, kf.y, dot));
+          }
+        }
+#pragma unroll
+        for (int o = 4; o >= 1; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int at = __shfl_sync(0xffffffffu, from, 8 * e);
+          const float v = __shfl_sync(0xffffffffu, dot, 8 * e);
+          if (lane == at) s_self = v;
+        }
+      }
     }
     const uint64_t scale2 = f2_pack(scale_log2, scale_log2), nown2 = f2_pack(-own, -own);
     float acc[2] = {0.0f, 0.0f};   // rows, columns
@@ -339,16 +376,19 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
         tc_fence_after_sync();
         const int diag = my_slot != kNoSlot ? r : -1;   // column of the seed diagonal in tile t0 + my
         uint64_t a2[2] = {0, 0};
-        // a quarter of the tile in registers at a time
+        // a quarter of the tile at a time, in a rolled loop: a CTA runs through its code once or
+        // twice, and what it has to fetch counts
+        constexpr int kQuarters = 4 / kHalves;
+        const int q0 = kHalves == 2 ? 2 * half : 0;
 #pragma unroll 1
-        for (int c32 = 0; c32 < 4; ++c32) {
+        for (int c32 = q0; c32 < q0 + kQuarters; ++c32) {
           const uint32_t word = bits[(kind * n_t + j) * 4 + c32];   // the same for every thread
           uint32_t raw[32];
           if (word != 0u) {
             tmem_ld32(trow + (g * nbuf + buf) * kT + 32 * c32, raw);
             tmem_ld_wait(raw);
           }
-          if (c32 == 3) {
+          if (c32 == q0 + kQuarters - 1) {
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.bar_s_empty[g][buf]);
@@ -400,16 +440,29 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
         report_status(status, kStatusTimeout, 62);
         sm.abort = 1;
       }
+    } else if (kHalves == 2) {
+      if (half == 1) {
+        sm.half1[my][0][r] = acc[0];
+        sm.half1[my][1][r] = acc[1];
+      }
+      sum[0] = acc[0];
+      sum[1] = acc[1];
+      done = valid && half == 0;
     } else if (valid) {
       const size_t o = static_cast<size_t>(bh) * per + i;
-      if (NT == 2 || g == 0) part_out[o] = acc[0];
-      if (NT == 2 || g == 1) part_in[o] = acc[1];
+      if (g == 0) part_out[o] = acc[0];
+      else part_in[o] = acc[1];
     }
   }
 
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
+  if (kHalves == 2 && done) {
+    const size_t o = static_cast<size_t>(bh) * per + i;
+    part_out[o] = sum[0] + sm.half1[my][0][r];
+    part_in[o] = sum[1] + sm.half1[my][1][r];
+  }
   if (warp == kMmaWarp) tmem_dealloc(tbase, tmem_cols);
 }
 
@@ -465,7 +518,8 @@ int launch_tiles(const MassArgs& a, int n_t, const CUtensorMap& tq, const CUtens
   const float scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(kD));
   cudaLaunchAttribute attr[1];
   const cudaLaunchConfig_t cfg =
-      pdl_config(dim3(static_cast<unsigned>(grid)), dim3(kThreads), mass_smem_bytes(NT, n_t), stream, attr);
+      pdl_config(dim3(static_cast<unsigned>(grid)), dim3(MassRoles<NT>::kThreads), mass_smem_bytes(NT, n_t), stream,
+                 attr);
   return cudaLaunchKernelEx(&cfg, mass_kernel<NT>, tq, tk, static_cast<const __nv_bfloat16*>(a.k_seedmask), a.seed_idx,
                             a.n_seeds, a.lse, a.Hq, a.Hkv, a.L, a.pos0, a.per, n_t, n_g, a.tok, a.flags, a.mask_id,
                             scale_log2, part_in, part_out, status) == cudaSuccess ? 0 : -3;
@@ -495,8 +549,9 @@ int launch_attn_mass(const MassArgs& a, int* status, cudaStream_t stream) {
   });
   if (rc != 0) return rc;
   // Tiles per CTA: two while the tiles outnumber the SMs; below that one tile a CTA spreads over
-  // more SMs. us at NT = 1 / 2 (B, heads, rows): 4, 32, 256: 16.8 / 10.9; 1, 32 / 32, 1024: 34.9 /
-  // 23.7; 2, 32 / 8, 256 (128 tiles): 9.5 / 10.2; 1, 28 / 4, 512 (112 tiles): 12.0 / 14.4.
+  // more SMs. us at NT = 1 / 2 when the rule was set (B, heads, rows): 4, 32, 256: 16.8 / 10.9; 1,
+  // 32 / 32, 1024: 34.9 / 23.7; 2, 32 / 8, 256 (128 tiles): 9.5 / 10.2; 1, 28 / 4, 512 (112 tiles):
+  // 12.0 / 14.4.
   const bool pair = n_t > 1 && n_t <= kMaxTilesPair && static_cast<long long>(n_t) * a.Hq * a.B > n_sm;
   rc = pair ? launch_tiles<2>(a, n_t, tq, tk, part_in, part_out, status, stream)
             : launch_tiles<1>(a, n_t, tq, tk, part_in, part_out, status, stream);
