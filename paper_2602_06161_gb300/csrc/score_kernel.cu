@@ -99,14 +99,6 @@ __device__ __forceinline__ void raise_max(RowAcc& a, float new_m, int new_i, int
   a.mref = new_ref;
 }
 
-__device__ __forceinline__ uint4 ld_stream(const uint4* p) {
-  uint4 r;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
-               : "l"(p));
-  return r;
-}
-
 __device__ __forceinline__ float bf16_to_f32(uint16_t h) { return __uint_as_float(static_cast<uint32_t>(h) << 16); }
 
 __device__ __forceinline__ void acc_scalar(RowAcc& a, float x, int idx) {
@@ -160,17 +152,31 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   e = (a - (s - bb)) + (b - bb);
 }
 
-// A thread's recorded batch is re-read from the row in global memory, in up to four vectors
-// kStride elements apart; the loads are issued by the threads that hold their warp's maximum
-// before the block-wide maximum is known, so their latency overlaps the reduction.
+// A thread's recorded batch is re-read, in up to four vectors kStride elements apart, from the ring
+// while it still holds the batch's chunk, else from the row in global memory; the loads are issued
+// by the threads that hold their warp's maximum before the block-wide maximum is known, so their
+// latency overlaps the reduction.
 constexpr int kMaxBatch = 4;
 static_assert(kVecPerThread <= kMaxBatch, "batches hold at most four vectors");
 
+// Where the row kernel's ring holds a row (slice) after its last chunk: element `first` of the row
+// began chunk 0, and chunks from `held` on are there.
+struct Ring {
+  const uint8_t* base;
+  int first, held;
+};
+
 template <int kStride>
-__device__ __forceinline__ void load_batch(const RowAcc& a, const uint16_t* row, uint4 (&w)[kMaxBatch]) {
+__device__ __forceinline__ void load_batch(const RowAcc& a, const uint16_t* row, const Ring& ring,
+                                           uint4 (&w)[kMaxBatch]) {
+  const int at = a.mi - ring.first, c = at / kChunkElems;
+  const uint16_t* src = a.mu != 0 && c >= ring.held
+                            ? reinterpret_cast<const uint16_t*>(ring.base + (c % kRingStages) * kChunkBytes) +
+                                  (at - c * kChunkElems)
+                            : row + a.mi;
 #pragma unroll
   for (int u = 0; u < kMaxBatch; ++u)
-    if (u < a.mu) w[u] = ld_stream(reinterpret_cast<const uint4*>(row + a.mi + u * kStride));
+    if (u < a.mu) w[u] = *reinterpret_cast<const uint4*>(src + u * kStride);
 }
 
 // First index of the value M in the thread's recorded batch w.
@@ -191,7 +197,7 @@ __device__ __forceinline__ int first_index_of(const RowAcc& a, float M, const ui
 }
 
 template <int NW, int kStride>
-__device__ __forceinline__ RowSum row_reduce(const RowAcc& a, const uint16_t* row, float* red_m, int* red_i,
+__device__ __forceinline__ RowSum row_reduce(const RowAcc& a, const uint16_t* row, const Ring& ring, float* red_m, int* red_i,
                                              float2* red_z, float2* red_s) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float m = a.m;
@@ -199,7 +205,7 @@ __device__ __forceinline__ RowSum row_reduce(const RowAcc& a, const uint16_t* ro
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   const bool cand = a.m == m && m != -INFINITY;   // may hold the row maximum
   uint4 w[kMaxBatch];
-  if (cand) load_batch<kStride>(a, row, w);
+  if (cand) load_batch<kStride>(a, row, ring, w);
   if (lane == 0) red_m[warp] = m;
   __syncthreads();
   float M = red_m[0];
@@ -312,23 +318,33 @@ __device__ __forceinline__ RowSum row_combine(const RowSum* part, int lane) {
   return r;
 }
 
+// What a row's scores need beside its sums, read by the producer while the row streams: the current
+// token y, its logit (NaN for a token outside [0, V), which has no probability), d_in and d_out.
+// Read after the sums, they were two more round trips to memory at the end of each row: with the
+// batches read back from the ring (load_batch) 7.27 -> 6.81 us on 32 rows of 126464 logits with all of
+// them given, 19.1 -> 18.4 us on 256 rows, 57.1 -> 55.9 us on 1024 rows of 152064.
+struct RowSide {
+  int y;
+  float xy, din, dout;
+};
+constexpr int kGreedy = 0x7fffffff;   // RowSide::y: no current token
+
+// The logit of the side's current token; takes the token's load as its latency.
+__device__ __forceinline__ void side_logit(RowSide& r, const uint16_t* row, int V) {
+  if (r.y == kGreedy) return;
+  const bool in = r.y >= 0 && r.y < V;
+  r.xy = in ? bf16_to_f32(row[r.y]) : __int_as_float(0x7fc00000);
+}
+
 // Thread 0 writes the row's outputs; returns (to thread 0) whether this CTA is
 // the last of its segment to finish.
-__device__ __forceinline__ bool row_write(const RowOut& r, int n, const uint16_t* row, int V, int per_seq,
-                                          const int32_t* cur_tok, const float* d_in, const float* d_out, int topk,
+__device__ __forceinline__ bool row_write(const RowOut& r, const RowSide& side, int n, int per_seq, int topk,
                                           float* maxprob, float* entropy, int32_t* argmax, float* score,
                                           uint32_t* counters, float* ws_u = nullptr, float* ws_lnz = nullptr) {
   const float Zf = r.Z;
   const float lnZ = logf(Zf);
   const float H = lnZ - 0.6931471805599453f * r.q;
-  const int y = cur_tok != nullptr ? cur_tok[n] : r.yhat;
-  float u = __int_as_float(0x7fc00000);   // a current token outside [0, V) has no probability
-  if (y >= 0 && y < V) {
-    const float xy = (y == r.yhat) ? r.M : bf16_to_f32(row[y]);
-    u = lnZ - (xy - r.M);
-  }
-  const float din = d_in != nullptr ? d_in[n] : 0.0f;
-  const float dout = d_out != nullptr ? d_out[n] : 0.0f;
+  const float u = side.y == kGreedy ? lnZ : lnZ - (side.xy - r.M);
   maxprob[n] = 1.0f / Zf;
   entropy[n] = H;
   argmax[n] = r.yhat;
@@ -338,7 +354,7 @@ __device__ __forceinline__ bool row_write(const RowOut& r, int n, const uint16_t
     ws_lnz[n] = lnZ;
     if (counters == nullptr) return false;   // the decisions have a launch of their own
   } else {
-    score[n] = u * (1.0f + din) / (1.0f + dout);
+    score[n] = u * (1.0f + side.din) / (1.0f + side.dout);
     if (topk <= 0) return false;
   }
   // The counter increment is a release (thread 0 wrote all of the row's results above) and an
@@ -1324,6 +1340,7 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
   __shared__ float2 red_z[kConsumerWarps + 1], red_s[kConsumerWarps + 1];
   __shared__ int s_last, s_abort;
   __shared__ RowSum s_part[C];   // the cluster's slice sums, in its first CTA
+  __shared__ RowSide s_side;
   if (C > 1) cluster_arrive();   // completed before the slice sums are sent: every CTA has started
   // programmatic dependent launch: wait for the stream's previous kernel, let the next one be
   // scheduled
@@ -1369,6 +1386,15 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
   if (warp == kConsumerWarps) {
     // producer: one lane streams the row chunk by chunk
     if (lane == 0) {
+      // the row's side data, on its way while the row streams (its logit once the token is here)
+      RowSide side{kGreedy, 0.0f, 0.0f, 0.0f};
+      if (rank == 0) {
+        const int32_t* tok = P.decide ? P.dec.tok : P.cur_tok;
+        if (tok != nullptr) side.y = tok[n];
+        if (!P.decide && P.d_in != nullptr) side.din = P.d_in[n];
+        if (!P.decide && P.d_out != nullptr) side.dout = P.d_out[n];
+      }
+      if (nchunks <= kRingStages) side_logit(side, row, V);
       for (int c = kRingStages; c < nchunks; ++c) {
         const int st = c % kRingStages;
         if (!mbar_wait(&bar_empty[st], ((c / kRingStages) - 1) & 1, &s_abort)) {
@@ -1380,7 +1406,9 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
         mbar_arrive_expect_tx(&bar_full[st], static_cast<uint32_t>(elems * 2));
         bulk_load(ring + st * kChunkBytes, src_row + static_cast<size_t>(c) * kChunkElems,
                   static_cast<uint32_t>(elems * 2), &bar_full[st]);
+        if (c == kRingStages) side_logit(side, row, V);
       }
+      s_side = side;
       // every copy issued has been consumed once the consumers pass their last
       // full-barrier wait; nothing is left in flight at the final barrier
     } else if (rank == 0 && lane <= 16) {
@@ -1425,7 +1453,8 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
   }
   __syncwarp();
 
-  RowSum r = row_reduce<kConsumerWarps + 1, kConsumerWarps * 32 * 8>(a, row, red_m, red_i, red_z, red_s);
+  const Ring held{ring, first, nchunks - kRingStages};
+  RowSum r = row_reduce<kConsumerWarps + 1, kConsumerWarps * 32 * 8>(a, row, held, red_m, red_i, red_z, red_s);
   if (C > 1) {
     // every CTA sends its slice's sums to the cluster's first, which adds them
     __syncwarp();
@@ -1438,9 +1467,8 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
     if (warp == 0) r = row_combine<C>(s_part, lane);
   }
   if (tid == 0)
-    s_last = row_write(row_finish(r), n, row, V, P.per_seq, P.decide ? P.dec.tok : P.cur_tok, P.d_in, P.d_out, P.topk,
-                       P.maxprob, P.entropy, P.argmax, P.score, P.decide == kDecideApart ? nullptr : P.counters,
-                       P.decide ? P.dec.ws_u : nullptr,
+    s_last = row_write(row_finish(r), s_side, n, P.per_seq, P.topk, P.maxprob, P.entropy, P.argmax, P.score,
+                       P.decide == kDecideApart ? nullptr : P.counters, P.decide ? P.dec.ws_u : nullptr,
                        P.decide ? P.dec.ws_lnz : nullptr);
   __syncthreads();
   if (s_last) {
