@@ -298,7 +298,7 @@ def run_ours(args):
                 "kernel_ms": round(attn_ms, 4)}
 
     score_bytes = si.N * si.V * 2 + si.N * 20 + n_seq * k * 8
-    scoring = {"kernel": "score_kernel", "ms": round(score_ms, 4),
+    scoring = {"kernel": "score_bulk_kernel", "ms": round(score_ms, 4),
                "gbs": round(score_bytes / (score_ms * 1e-3) / 1e9, 1),
                "frac_of_measured_hbm": round(score_bytes / (score_ms * 1e-3) / 1e9 / peaks["hbm_gbs"], 4),
                "frac_of_8tbs_nominal": round(score_bytes / (score_ms * 1e-3) / 1e9 / 8000.0, 4),

@@ -33,10 +33,10 @@
 //
 // Bound: latency and, with many heads, reading Q and K once (8 x 32 heads x 256 rows: 34 MB, 5 us).
 // With NT = 2 a head's 256-row block is one CTA that reads it once, instead of four CTAs (one per
-// tile and orientation) reading three tiles each: 29.1 -> 17.9 us there (both launches), 16.6 -> 9.4
-// us with 4 x 32 heads, 53.7 -> 34.7 us with 8 x 28/4 heads and 512 rows. What is left is a CTA's
-// chain in ceil(CTAs / SMs) waves, about 8 us: its tiles and seed keys from DRAM (2 to 4 us, while
-// every SM loads), four products' exponentials (half a microsecond each), 1.2 us until the next CTA.
+// tile and orientation) reading three tiles each: 29.1 -> 17.9 us there (both launches, 32 seeds a
+// sequence; 31.1 -> 19.4 with 64), 16.6 -> 9.4 us with 4 x 32 heads, 53.7 -> 34.7 us with 8 x 28/4
+// heads and 512 rows. What is left is a CTA's chain in ceil(CTAs / SMs) waves, about 8 us: its tiles
+// and seed keys from DRAM (2 to 4 us, while every SM loads), then four products and their exponentials.
 //
 // Warps: the math warps (thread = tensor-memory lane, a row / key of a tile), then one whose lane 0
 // issues the TMA loads and one that allocates tensor memory and whose lane 0 issues the products.

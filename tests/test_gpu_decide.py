@@ -156,7 +156,7 @@ def test_decide_longest_segment_and_workspace_reuse():
 
 
 def test_decide_register_path_odd_vocab():
-    di = W.make_decide_inputs(48, 3001, 2, seed=29, block_len=8)   # V % 8 != 0: the register-load kernel
+    di = W.make_decide_inputs(48, 3001, 2, seed=29, block_len=8)   # V % 8 != 0: unaligned rows
     p = _params()
     check(di, p, run_decide(di, p), what="odd V")
 
@@ -187,7 +187,7 @@ def test_decide_named_workload_full():
     (288, 1000),    # one row per thread of the bulk-copy kernel (288 threads): the fast path
     (289, 1000),    # one row more than its threads: the general path
     (1153, 1000),   # the general path, four rows per thread and one more
-    (512, 1001),    # the register-load kernel (odd vocabulary, 512 threads): its fast-path limit
+    (512, 1001),    # an odd vocabulary, more rows than the row kernel's threads
     (513, 1001),    # and one row past it
     (2049, 1001),   # a segment of 2049 rows: 48 KB of keys and scores in shared memory
 ])

@@ -100,8 +100,8 @@ def test_window_f32(D, Lk, Lq, q0):
 
 def test_window_rows_equal_square_rows_bit_exactly():
     # a query row's arithmetic does not depend on where its tile starts: the window rows
-    # are bit-identical to the same rows of the square launch (an odd number of KV tiles,
-    # so the square launch does not split any unit's keys over two CTAs). The windows run on the
+    # are bit-identical to the same rows of the square launch (an odd number of KV tiles in one
+    # round of units: both split every unit's keys alike, with a last tile past the memory). The windows run on the
     # square kernel through the fault entry with no planted load: the prefix call itself may take
     # the packed grouped-query kernel, whose rows agree up to rounding (test_gpu_window_gqa.py)
     B, Hq, Hkv, Lk, S = 2, 4, 2, 1100, 20

@@ -108,7 +108,7 @@ def test_score_ties_and_uniform_rows():
     check(inp, r)
 
 
-@pytest.mark.parametrize("V", [40000, 40001])   # bulk-copy kernel (V % 8 == 0), register-load kernel
+@pytest.mark.parametrize("V", [40000, 40001])   # aligned rows (V % 8 == 0), unaligned rows
 def test_score_argmax_ties_across_batches(V):
     """The first index of the row maximum when it occurs several times: in different chunks, in one
     thread's batch (different vectors), in one thread's batches of different chunks, at the row's
@@ -161,13 +161,13 @@ def test_score_named_workloads_full(name):
     (288, 1000, 40),    # one row per thread of the bulk-copy kernel: selection by rank
     (289, 1000, 20),    # the general path, a short list: warp sorts and merges
     (289, 1000, 40),    # the general path, a long list: the bitonic sort
-    (512, 1001, 33),    # the register-load kernel (512 threads): selection by rank
+    (512, 1001, 33),    # an odd vocabulary, more rows than a CTA has threads
     (513, 1001, 32),    # and one row past it: warp sorts and merges
     (4096, 136, 32),    # the largest segment, k = 32
     (600, 300, 9),      # the fewest keys taken by warp sorts
     (600, 300, 8),      # the most taken by rounds of a CTA-wide maximum
     (777, 200, 1),      # k = 1
-    (600, 1001, 5),     # the register-load kernel's general path (16 warps), rounds
+    (600, 1001, 5),     # an odd vocabulary, the general path, rounds
 ])
 def test_score_topk_on_both_sides_of_the_fast_path(per, V, k):
     inp = W.make_score_inputs(2 * per, V, 2, k, seed=per + k, spike_frac=0.1, eligible_frac=0.8)
