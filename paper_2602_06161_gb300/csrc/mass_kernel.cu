@@ -36,7 +36,8 @@
 // tile and orientation) reading three tiles each: 29.1 -> 17.9 us there (both launches, 32 seeds a
 // sequence; 31.1 -> 19.4 with 64), 16.6 -> 9.4 us with 4 x 32 heads, 53.7 -> 34.7 us with 8 x 28/4
 // heads and 512 rows. What is left is a CTA's chain in ceil(CTAs / SMs) waves, about 8 us: its tiles
-// and seed keys from DRAM (2 to 4 us, while every SM loads), then four products and their exponentials.
+// and seed keys (2 to 4 us), then four products and their exponentials. Prefetching the next wave's
+// tiles and seed keys into L2 did not shorten it (19.4 us either way; 5 x 32/8, 384 rows: 23.9 -> 24.4).
 //
 // Warps: the math warps (thread = tensor-memory lane, a row / key of a tile), then one whose lane 0
 // issues the TMA loads and one that allocates tensor memory and whose lane 0 issues the products.
