@@ -198,56 +198,6 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
   return __all_sync(0xffffffffu, ok);
 }
 
-// A seed row's masked self term s_self merged into its running (m, l) as (O + p v) / (l + p),
-// p = 2^(s_self - m): returns p, and in *scale what O has to be multiplied with first (1 unless the
-// self term lies far above the row's other scores, where (m, l, O) is rescaled to it).
-__device__ __forceinline__ float merge_self(float s_self, float& m, float& l, float* scale) {
-  if (m != -INFINITY && s_self <= m + kSelfInPlace) {
-    const float p = ex2_approx(s_self - m);
-    l += p;
-    return p;
-  }
-  const float m2 = fmaxf(m, s_self);
-  *scale = (m == -INFINITY) ? 0.0f : ex2_approx(m - m2);
-  const float p = ex2_approx(s_self - m2);
-  l = l * *scale + p;
-  m = m2;
-  return p;
-}
-
-// x = scale x + p v on 32 columns; v: four 16-byte vectors of bf16.
-__device__ __forceinline__ void add_self(float (&x)[32], float scale, float p, const uint4* v) {
-  if (scale != 1.0f) {
-#pragma unroll
-    for (int e = 0; e < 32; ++e) x[e] *= scale;
-  }
-#pragma unroll
-  for (int ch = 0; ch < 4; ++ch) {
-    const uint4 vv = v[ch];
-    const __nv_bfloat162* vp = reinterpret_cast<const __nv_bfloat162*>(&vv);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 vf = __bfloat1622float2(vp[e]);
-      x[8 * ch + 2 * e] = fmaf(p, vf.x, x[8 * ch + 2 * e]);
-      x[8 * ch + 2 * e + 1] = fmaf(p, vf.y, x[8 * ch + 2 * e + 1]);
-    }
-  }
-}
-
-// Stages 32 columns of a row, normalised, as bf16: 16-byte chunks ch0 .. ch0 + 3 of lane's row of a
-// 128-byte-swizzled box of 64 columns.
-__device__ __forceinline__ void stage_row(uint8_t* box, int lane, int ch0, const float (&x)[32], float inv) {
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    uint4 v;
-    v.x = pack_bf16x2(x[8 * q + 0] * inv, x[8 * q + 1] * inv);
-    v.y = pack_bf16x2(x[8 * q + 2] * inv, x[8 * q + 3] * inv);
-    v.z = pack_bf16x2(x[8 * q + 4] * inv, x[8 * q + 5] * inv);
-    v.w = pack_bf16x2(x[8 * q + 6] * inv, x[8 * q + 7] * inv);
-    *reinterpret_cast<uint4*>(box + lane * 128 + (((ch0 + q) ^ (lane & 7)) << 4)) = v;
-  }
-}
-
 __device__ __forceinline__ void raise_abort(AttnSmem& sm, int* status, int site) {
   report_status(status, kStatusTimeout, site);
   sm.abort = 1;
@@ -944,66 +894,138 @@ __global__ void __launch_bounds__(kThreads, 1)
           const float a1 = (m1 == -INFINITY) ? 0.0f : ex2_approx(m1 - m);
           float l = sm.split_l[0][r] * a0 + sm.split_l[1][r] * a1;
           const int cb = qt * 64;   // this warpgroup's columns
-          const int grow = tile_row0<kUnitRows>(w, 0) + r;
-          float scale = 1.0f, pself = 0.0f;
-          const uint4* vmv = nullptr;
-          if (is_seed) {
-            const int vi = sm.vidx[sb][r];
-            const size_t mrow = ((static_cast<size_t>(w.b) * Hkv + ug.group.div(static_cast<uint32_t>(w.hq))) * n_seeds + my_slot) * kD;
-            vmv = (vi != kNotStaged ? reinterpret_cast<const uint4*>(sm.vstage[sb][vi])
-                                    : reinterpret_cast<const uint4*>(v_seedmask + mrow)) + cb / 8;
-            pself = merge_self(sm.sself[sb][r], m, l, &scale);
-          }
-          const int sig = (g0 + nks - 1) & 1;
-          uint8_t* stage = sm.k[sig] + (warp & 3) * (2 * 4096) + qt * 4096;
-          const float inv = 1.0f / l;
-#pragma unroll 1
+          float oh[64];
+#pragma unroll
           for (int c = 0; c < 2; ++c) {
             uint32_t x0[32], x1[32];
             tmem_ld32(trow + col_o(0) + cb + 32 * c, x0);
             tmem_ld32(trow + col_o(1) + cb + 32 * c, x1);
             tmem_ld_wait(x0);
             tmem_ld_wait(x1);
-            float x[32];
 #pragma unroll
-            for (int e = 0; e < 32; ++e) x[e] = __uint_as_float(x0[e]) * a0 + __uint_as_float(x1[e]) * a1;
-            if (is_seed) add_self(x, scale, pself, vmv + 4 * c);
-            __syncwarp();   // the next chunk's load is warp-wide
-            stage_row(stage, lane, 4 * c, x, inv);
+            for (int e = 0; e < 32; ++e) oh[32 * c + e] = __uint_as_float(x0[e]) * a0 + __uint_as_float(x1[e]) * a1;
           }
+          const int grow = tile_row0<kUnitRows>(w, 0) + r;
+          if (is_seed) {
+            const float s_self = sm.sself[sb][r];
+            const int vi = sm.vidx[sb][r];
+            const size_t mrow = ((static_cast<size_t>(w.b) * Hkv + ug.group.div(static_cast<uint32_t>(w.hq))) * n_seeds + my_slot) * kD;
+            const uint4* vmv = (vi != kNotStaged ? reinterpret_cast<const uint4*>(sm.vstage[sb][vi])
+                                                 : reinterpret_cast<const uint4*>(v_seedmask + mrow)) + cb / 8;
+            if (m != -INFINITY && s_self <= m + kSelfInPlace) {
+              // (O + p v) / (l + p) with p = 2^(s_self - m): one multiply-add per element
+              const float pself = ex2_approx(s_self - m);
+              l += pself;
+#pragma unroll
+              for (int ch = 0; ch < 8; ++ch) {
+                const uint4 vv = vmv[ch];
+                const __nv_bfloat162* vp = reinterpret_cast<const __nv_bfloat162*>(&vv);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  const float2 vf = __bfloat1622float2(vp[e]);
+                  oh[ch * 8 + 2 * e] = fmaf(pself, vf.x, oh[ch * 8 + 2 * e]);
+                  oh[ch * 8 + 2 * e + 1] = fmaf(pself, vf.y, oh[ch * 8 + 2 * e + 1]);
+                }
+              }
+            } else {
+              // a self term far above the row's other scores: rescale (m, l, O) to it
+              const float m2 = fmaxf(m, s_self);
+              const float a = (m == -INFINITY) ? 0.0f : ex2_approx(m - m2);
+              const float pself = ex2_approx(s_self - m2);
+              l = l * a + pself;
+#pragma unroll
+              for (int ch = 0; ch < 8; ++ch) {
+                const uint4 vv = vmv[ch];
+                const __nv_bfloat162* vp = reinterpret_cast<const __nv_bfloat162*>(&vv);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  const float2 vf = __bfloat1622float2(vp[e]);
+                  oh[ch * 8 + 2 * e] = oh[ch * 8 + 2 * e] * a + pself * vf.x;
+                  oh[ch * 8 + 2 * e + 1] = oh[ch * 8 + 2 * e + 1] * a + pself * vf.y;
+                }
+              }
+              m = m2;
+            }
+          }
+          const int sig = (g0 + nks - 1) & 1;
+          uint8_t* stage = sm.k[sig] + (warp & 3) * (2 * 4096) + qt * 4096;
+          const float inv = 1.0f / l;
+#pragma unroll
+          for (int ch = 0; ch < 8; ++ch) {
+            uint4 v;
+            v.x = pack_bf16x2(oh[ch * 8 + 0] * inv, oh[ch * 8 + 1] * inv);
+            v.y = pack_bf16x2(oh[ch * 8 + 2] * inv, oh[ch * 8 + 3] * inv);
+            v.z = pack_bf16x2(oh[ch * 8 + 4] * inv, oh[ch * 8 + 5] * inv);
+            v.w = pack_bf16x2(oh[ch * 8 + 6] * inv, oh[ch * 8 + 7] * inv);
+            *reinterpret_cast<uint4*>(stage + lane * 128 + ((ch ^ (lane & 7)) << 4)) = v;
+          }
+          if (qt == 0 && lse != nullptr && grow < Lq)
+            lse[(static_cast<size_t>(w.b) * Hq + w.hq) * Lq + grow] = (m + log2f(l)) * 0.6931471805599453f;
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
             mbar_arrive(&sm.bar_ostage_full[qt]);
             mbar_arrive(&sm.bar_slot_empty[sb]);
           }
-          if (qt == 0 && lse != nullptr && grow < Lq)
-            lse[(static_cast<size_t>(w.b) * Hq + w.hq) * Lq + grow] = (m + log2f(l)) * 0.6931471805599453f;
           continue;
         }
         // ---------------- epilogue of the unit ----------------
-        // O is read out before this warpgroup's next P is published, so the next unit's first P.V
-        // product cannot overwrite it early. The columns go 32 at a time in a rolled loop, and lse is
-        // stored behind the proxy fence, which would wait for that store: from one unit's last P to
-        // the next one's first took 8300 cycles of a seeded unit (3000 between steps), 2200 to 4000
-        // of them from O read to staged; now 6500. 5 x 32 heads, L = 1150: 111.9 -> 109.0 us; 8 x 32,
-        // L = 2048: 381.8 -> 379.8 us, where the clock is held by the power limit.
+        // O is read into registers before this warpgroup's next P is published, so the
+        // next unit's first P.V product cannot overwrite it early.
         tc_fence_after_sync();
+        uint32_t oraw[4][32];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tmem_ld32(o_addr + 32 * c, oraw[c]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tmem_ld_wait(oraw[c]);
+        float* o = reinterpret_cast<float*>(&oraw[0][0]);
         const int grow = tile_row0<kUnitRows>(w, qt) + r;
         if (warp_seed) {
           ok = warp_wait(&sm.bar_sself_full[sb], (it >> 1) & 1, &sm.abort, wait_ns);
           if (!ok) break;
         }
-        float scale = 1.0f, pself = 0.0f;
-        const uint4* vmv = nullptr;
         if (is_seed) {
-          // merge the masked-input self term (k_i, v_i) of this seed row; generic loads of v_i: shared
-          // memory when warp 11 staged the row, else global memory
+          // merge the masked-input self term (k_i, v_i) of this seed row
+          const float s_self = sm.sself[sb][qt * kBM + r];
           const int vi = sm.vidx[sb][qt * kBM + r];
           const size_t mrow = ((static_cast<size_t>(w.b) * Hkv + ug.group.div(static_cast<uint32_t>(w.hq))) * n_seeds + my_slot) * kD;
-          vmv = vi != kNotStaged ? reinterpret_cast<const uint4*>(sm.vstage[sb][vi])
-                                 : reinterpret_cast<const uint4*>(v_seedmask + mrow);
-          pself = merge_self(sm.sself[sb][qt * kBM + r], m_run, l_run, &scale);
+          // generic loads: shared memory when warp 11 staged the row, else global memory
+          const uint4* vmv = vi != kNotStaged ? reinterpret_cast<const uint4*>(sm.vstage[sb][vi])
+                                              : reinterpret_cast<const uint4*>(v_seedmask + mrow);
+          if (m_run != -INFINITY && s_self <= m_run + kSelfInPlace) {
+            // (O + p v) / (l + p) with p = 2^(s_self - m): one multiply-add per element
+            const float pself = ex2_approx(s_self - m_run);
+            l_run += pself;
+#pragma unroll
+            for (int ch = 0; ch < 16; ++ch) {
+              const uint4 vv = vmv[ch];
+              const __nv_bfloat162* vp = reinterpret_cast<const __nv_bfloat162*>(&vv);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const float2 vf = __bfloat1622float2(vp[e]);
+                o[ch * 8 + 2 * e] = fmaf(pself, vf.x, o[ch * 8 + 2 * e]);
+                o[ch * 8 + 2 * e + 1] = fmaf(pself, vf.y, o[ch * 8 + 2 * e + 1]);
+              }
+            }
+          } else {
+            // a self term far above the row's other scores: rescale (m, l, O) to it
+            const float m2 = fmaxf(m_run, s_self);
+            const float a = (m_run == -INFINITY) ? 0.0f : ex2_approx(m_run - m2);
+            const float pself = ex2_approx(s_self - m2);
+            l_run = l_run * a + pself;
+#pragma unroll
+            for (int ch = 0; ch < 16; ++ch) {
+              const uint4 vv = vmv[ch];
+              const __nv_bfloat162* vp = reinterpret_cast<const __nv_bfloat162*>(&vv);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const float2 vf = __bfloat1622float2(vp[e]);
+                o[ch * 8 + 2 * e] = o[ch * 8 + 2 * e] * a + pself * vf.x;
+                o[ch * 8 + 2 * e + 1] = o[ch * 8 + 2 * e + 1] * a + pself * vf.y;
+              }
+            }
+            m_run = m2;
+          }
         }
         // Output: the warp's 32 rows x 128 columns are staged in the shared-memory stage of
         // the unit's last KV tile (K stage for Q tile 0, V stage for Q tile 1: both finished
@@ -1014,29 +1036,25 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int sig = (g0 + nkv - 1) & 1;
           uint8_t* stage = (qt == 0 ? sm.k[sig] : sm.v[sig]) + (warp & 3) * (2 * 4096);
           const float inv = 1.0f / l_run;
-#pragma unroll 1
-          for (int c = 0; c < 4; ++c) {
-            uint32_t xr[32];
-            tmem_ld32(o_addr + 32 * c, xr);
-            tmem_ld_wait(xr);
-            float x[32];
 #pragma unroll
-            for (int e = 0; e < 32; ++e) x[e] = __uint_as_float(xr[e]);
-            if (is_seed) add_self(x, scale, pself, vmv + 4 * c);
-            __syncwarp();   // the next chunk's load is warp-wide
-            stage_row(stage + (c >> 1) * 4096, lane, 4 * (c & 1), x, inv);
-          }
-          // the staged rows go to the TMA thread, which stores them before it reloads the stage; the
-          // unit's routing and self scores are consumed
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) {
-            mbar_arrive(&sm.bar_ostage_full[qt]);
-            mbar_arrive(&sm.bar_slot_empty[sb]);
+          for (int ch = 0; ch < 16; ++ch) {
+            uint4 v;
+            v.x = pack_bf16x2(o[ch * 8 + 0] * inv, o[ch * 8 + 1] * inv);
+            v.y = pack_bf16x2(o[ch * 8 + 2] * inv, o[ch * 8 + 3] * inv);
+            v.z = pack_bf16x2(o[ch * 8 + 4] * inv, o[ch * 8 + 5] * inv);
+            v.w = pack_bf16x2(o[ch * 8 + 6] * inv, o[ch * 8 + 7] * inv);
+            *reinterpret_cast<uint4*>(stage + (ch >> 3) * 4096 + lane * 128 + (((ch & 7) ^ (lane & 7)) << 4)) = v;
           }
           if (lse != nullptr && grow < Lq)
             lse[(static_cast<size_t>(w.b) * Hq + w.hq) * Lq + grow] = (m_run + log2f(l_run)) * 0.6931471805599453f;
+          // the staged rows go to the TMA thread, which stores them before it reloads the stage
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sm.bar_ostage_full[qt]);
         }
+        // the unit's routing and self scores are consumed
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.bar_slot_empty[sb]);
       }
       if (!ok && !sm.abort) raise_abort(sm, status, 30 + qt);
     }
