@@ -208,9 +208,10 @@ __device__ __forceinline__ void raise_abort(AttnSmem& sm, int* status, int site)
 // otherwise Lq = Lk and q0 = 0 are compile-time facts.
 // kFault: the self-test instance that takes its wait limit and a planted missing load from
 // `flt`; the production instances wait up to one second and load every tile.
-// kPad: a split unit's halves may have an odd number of KV tiles between them (windows, and square
-// launches whose units are all split; the other square launches keep the code without it, which the
-// compiler schedules 7 % faster on long sequences).
+// kPad: a split unit's halves may have an odd number of KV tiles between them, and a window's rows may be
+// packed heads. Without it are square launches whose units are not all split, which the compiler then
+// schedules 7 % faster on long sequences, and one-tile windows of unpacked heads over an even number of
+// KV tiles (8 x 32 heads, 64 rows over 2048 keys: 49.7 -> 49.5 us; 32 heads, 32 rows over 512: 7.98 -> 7.90).
 template <int NQ, bool kWindow, bool kFault, bool kPad = kWindow>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_bf16_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
@@ -234,6 +235,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // one-tile units of a window are all split (with two KV tiles or more), so the second softmax
   // warpgroup takes half of every unit's keys
   constexpr bool kSplitAll = kWindow && NQ == 1;
+  constexpr bool kWrap = kWindow && kPad;   // packed heads: rows may wrap past the window's end
   const bool all_split = kSplitAll && ug.n_split > 0;
   // A split unit's two halves have `half` KV tiles each; with an odd nkv (kPad) the last one lies past
   // the memory (loaded as zeros without reading anything, every key masked). nks: KV ring entries of
@@ -469,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int32_t* seeds_b = seed_idx + static_cast<size_t>(w.b) * n_seeds;
       route_clear(sm.slot[sb], rows, lane, 32);
       __syncwarp();
-      if (kWindow) {
+      if (kWrap) {
         // the rows at a seed's position, one per packed head
         const int period = static_cast<int>(ug.period.d), end = min(row0 + rows, Lq);
         for (int sd = lane; sd < n_seeds; sd += 32) {
@@ -479,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (P >= row0) atomicMin(sm.slot[sb] + (P - row0), sd);
         }
       } else {
-        route_scan(sm.slot[sb], seeds_b, n_seeds, row0, rows, Lk, lane, 32);
+        route_scan(sm.slot[sb], seeds_b, n_seeds, q0 + row0, rows, Lk, lane, 32);
       }
       if (w.split) {
         // both warpgroups of a split unit work on the same rows
@@ -763,18 +765,23 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (grow >= Lq) my_slot = kNoSlot;
           // the diagonal of a square launch is column r of KV tile row0 / 128 of the row's Q tile
           int pos = 0;
-          if (kWindow) {
+          if (kWrap) {
             const uint32_t P = static_cast<uint32_t>(grow);
             pos = q0 + static_cast<int>(P - ug.period.div(P) * ug.period.d);
+          } else if (kWindow) {
+            pos = q0 + grow;
           }
           diag_j = (kWindow ? pos / kBN : tile_row0<kUnitRows>(w, qt) / kBN) - jbase;
           diag_c = kWindow ? pos % kBN : r;
         }
         const bool is_seed = my_slot != kNoSlot;
         const bool warp_seed = __any_sync(0xffffffffu, is_seed);
-        // in a window: the KV steps that hold the diagonals of the warp's seed rows (none: lo > hi)
-        const int dj_lo = kWindow ? __reduce_min_sync(0xffffffffu, is_seed ? diag_j : 0x7fffffff) : diag_j;
-        const int dj_hi = kWindow ? __reduce_max_sync(0xffffffffu, is_seed ? diag_j : -0x7fffffff) : diag_j;
+        // in a window: the KV steps that hold the diagonals of the warp's seed rows (none: lo > hi); 32
+        // consecutive rows that do not wrap meet theirs in at most two KV tiles
+        const int dj_lo = kWrap ? __reduce_min_sync(0xffffffffu, is_seed ? diag_j : 0x7fffffff)
+                          : kWindow ? __shfl_sync(0xffffffffu, diag_j, 0) : diag_j;
+        const int dj_hi = kWrap ? __reduce_max_sync(0xffffffffu, is_seed ? diag_j : -0x7fffffff)
+                          : kWindow ? __shfl_sync(0xffffffffu, diag_j, 31) : diag_j;
         const int g0 = it * nkr;   // the CTA's KV ring entries before this unit
         // this warpgroup's steps before this unit (half a unit's KV tiles each when all are split)
         const int sbase = all_split ? it * half : g0;
@@ -796,7 +803,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int c = 0; c < kBN; ++c)
               if (c >= valid) s[c] = -INFINITY;
           }
-          if (kWindow ? j >= dj_lo && j <= dj_hi : warp_seed && j == diag_j) {
+          if (kWrap ? j >= dj_lo && j <= dj_hi : warp_seed && (j == dj_lo || j == dj_hi)) {
             // exclusion of the cached diagonal term of a seed row
             const bool here = is_seed && j == diag_j;
             if (!kWindow) {
@@ -1142,10 +1149,12 @@ int launch_attn_bf16_sm103(const AttnArgs& args, int* status, cudaStream_t strea
   const bool window = a.Lq != a.L || a.q0 != 0;
   const int period = a.Lq;
   int nq = kNQ;
+  bool pack = false;
   if (window) {
     const WindowPlan plan = plan_window(a, n_sm);
     nq = plan.nq;
-    if (plan.pack) {
+    pack = plan.pack;
+    if (pack) {
       // the query heads of a KV head as the rows of one head
       a.Lq *= a.Hq / a.Hkv;
       a.Hq = a.Hkv;
@@ -1169,7 +1178,8 @@ int launch_attn_bf16_sm103(const AttnArgs& args, int* status, cudaStream_t strea
     for (auto fn : {attn_bf16_kernel<2, false, false>, attn_bf16_kernel<1, true, false>,
                     attn_bf16_kernel<2, true, false>, attn_bf16_kernel<2, false, true>,
                     attn_bf16_kernel<1, true, true>, attn_bf16_kernel<2, true, true>,
-                    attn_bf16_kernel<2, false, false, true>, attn_bf16_kernel<2, false, true, true>}) {
+                    attn_bf16_kernel<2, false, false, true>, attn_bf16_kernel<2, false, true, true>,
+                    attn_bf16_kernel<1, true, false, false>, attn_bf16_kernel<1, true, true, false>}) {
       if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return -3;
       // the register split inside the kernel assumes exactly kLaunchRegs per thread at launch;
@@ -1203,6 +1213,8 @@ int launch_attn_bf16_sm103(const AttnArgs& args, int* status, cudaStream_t strea
   const bool pad = n_split > 0 && nkv % 2 != 0;
   auto kernel = !window && pad ? (fault ? attn_bf16_kernel<2, false, true, true> : attn_bf16_kernel<2, false, false, true>)
                 : !window     ? (fault ? attn_bf16_kernel<2, false, true> : attn_bf16_kernel<2, false, false>)
+                : nq == 1 && nkv % 2 == 0 && !pack
+                    ? (fault ? attn_bf16_kernel<1, true, true, false> : attn_bf16_kernel<1, true, false, false>)
                 : nq == 1     ? (fault ? attn_bf16_kernel<1, true, true> : attn_bf16_kernel<1, true, false>)
                               : (fault ? attn_bf16_kernel<2, true, true> : attn_bf16_kernel<2, true, false>);
   // programmatic dependent launch: the prologue overlaps the previous kernel's tail

@@ -118,6 +118,23 @@ def test_window_rows_equal_square_rows_bit_exactly():
     assert api.cover_device_status() == 0
 
 
+@pytest.mark.parametrize("B,Hq,Lk,Lq,q0,S,inside", [
+    (1, 3, 129, 2, 127, 3, 2),              # one key in the last of two KV tiles, a diagonal in each
+    (1, 3, 1024, 129, 895, 9, 9),           # a full tile and one row, at the memory's end
+    (7, 32, 250, 40, 110, 6, 5),            # several units a CTA, a ragged last tile, diagonals in both tiles
+    (7, 32, 1000, 1, 999, 4, 1),            # one row, the memory's last
+])
+def test_window_unpacked_even_tiles(B, Hq, Lk, Lq, q0, S, inside):
+    """Unpacked heads over an even number of KV tiles: the one-tile instance without padding."""
+    q, kc, vc, km, vm, seeds = _case(B, Hq, Hq, Lk, 128, S, q0, Lq, "bf16", Lk + Lq, inside)
+    out, lse = run_window(q, kc, vc, km, vm, seeds, q0, Lq, "bf16")
+    f = W.bf16_bits_to_f64
+    ref, ref_lse = oracle.override_attention_window(f(q[:, :, q0:q0 + Lq]), f(kc), f(vc), f(km), f(vm), seeds, q0)
+    d = np.abs(out - ref)
+    assert d.max() <= H.TOL_BF16_MAX and d.mean() <= H.TOL_BF16_MEAN, (d.max(), d.mean())
+    assert np.abs(lse - ref_lse).max() <= H.TOL_LSE
+
+
 def test_window_rows_match_split_square_rows():
     # with an even number of KV tiles and few units the square launch splits every unit's keys
     # over two CTAs (merged in the epilogue); the window rows then agree up to rounding
