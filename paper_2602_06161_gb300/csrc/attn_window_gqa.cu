@@ -645,7 +645,7 @@ int win_setup(WinSetup* out, size_t smem) {
 
 // Predicted microseconds of one call, fitted to calls measured back to back on
 // GB300 (Dream-shaped windows of 16 to 128 rows over 1024 keys, batches of 1 to 8, memories of
-// 2048 to 8192 keys; up to 19 % high, and the square kernel's up to 20 % low, over 22 shapes, on
+// 2048 to 8192 keys; up to 19 % high, and the square kernel's up to 21 % low, over 22 shapes, on
 // all of which the faster kernel was taken): a packed CTA takes about 7 us plus
 // 1.5 us per KV step, and the clusters beyond those resident at once run in further waves (the
 // square kernel's prediction: window_square_us).
