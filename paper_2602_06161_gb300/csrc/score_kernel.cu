@@ -318,22 +318,22 @@ __device__ __forceinline__ RowSum row_combine(const RowSum* part, int lane) {
   return r;
 }
 
-// What a row's scores need beside its sums, read by the producer while the row streams: the current
-// token y, its logit (NaN for a token outside [0, V), which has no probability), d_in and d_out.
+// What a row's scores need beside its sums, read by the producer while the row streams: the logit of
+// the current token y (NaN for a token outside [0, V), which has no probability), d_in and d_out.
 // Read after the sums, they were two more round trips to memory at the end of each row: with the
 // batches read back from the ring (load_batch) 7.27 -> 6.81 us on 32 rows of 126464 logits with all of
 // them given, 19.1 -> 18.4 us on 256 rows, 57.1 -> 55.9 us on 1024 rows of 152064.
+// Whether a token is given is a flag of its own: every 32-bit value may come as a token.
 struct RowSide {
-  int y;
+  bool greedy;   // no current token: y is the row's greedy token
   float xy, din, dout;
 };
-constexpr int kGreedy = 0x7fffffff;   // RowSide::y: no current token
 
-// The logit of the side's current token; takes the token's load as its latency.
-__device__ __forceinline__ void side_logit(RowSide& r, const uint16_t* row, int V) {
-  if (r.y == kGreedy) return;
-  const bool in = r.y >= 0 && r.y < V;
-  r.xy = in ? bf16_to_f32(row[r.y]) : __int_as_float(0x7fc00000);
+// The logit of the given current token y; takes the token's load as its latency.
+__device__ __forceinline__ void side_logit(RowSide& r, int y, const uint16_t* row, int V) {
+  if (r.greedy) return;
+  const bool in = y >= 0 && y < V;
+  r.xy = in ? bf16_to_f32(row[y]) : __int_as_float(0x7fc00000);
 }
 
 // Thread 0 writes the row's outputs; returns (to thread 0) whether this CTA is
@@ -344,7 +344,7 @@ __device__ __forceinline__ bool row_write(const RowOut& r, const RowSide& side, 
   const float Zf = r.Z;
   const float lnZ = logf(Zf);
   const float H = lnZ - 0.6931471805599453f * r.q;
-  const float u = side.y == kGreedy ? lnZ : lnZ - (side.xy - r.M);
+  const float u = side.greedy ? lnZ : lnZ - (side.xy - r.M);
   maxprob[n] = 1.0f / Zf;
   entropy[n] = H;
   argmax[n] = r.yhat;
@@ -1387,14 +1387,16 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
     // producer: one lane streams the row chunk by chunk
     if (lane == 0) {
       // the row's side data, on its way while the row streams (its logit once the token is here)
-      RowSide side{kGreedy, 0.0f, 0.0f, 0.0f};
+      RowSide side{true, 0.0f, 0.0f, 0.0f};
+      int y = 0;
       if (rank == 0) {
         const int32_t* tok = P.decide ? P.dec.tok : P.cur_tok;
-        if (tok != nullptr) side.y = tok[n];
+        side.greedy = tok == nullptr;
+        if (tok != nullptr) y = tok[n];
         if (!P.decide && P.d_in != nullptr) side.din = P.d_in[n];
         if (!P.decide && P.d_out != nullptr) side.dout = P.d_out[n];
       }
-      if (nchunks <= kRingStages) side_logit(side, row, V);
+      if (nchunks <= kRingStages) side_logit(side, y, row, V);
       for (int c = kRingStages; c < nchunks; ++c) {
         const int st = c % kRingStages;
         if (!mbar_wait(&bar_empty[st], ((c / kRingStages) - 1) & 1, &s_abort)) {
@@ -1406,7 +1408,7 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
         mbar_arrive_expect_tx(&bar_full[st], static_cast<uint32_t>(elems * 2));
         bulk_load(ring + st * kChunkBytes, src_row + static_cast<size_t>(c) * kChunkElems,
                   static_cast<uint32_t>(elems * 2), &bar_full[st]);
-        if (c == kRingStages) side_logit(side, row, V);
+        if (c == kRingStages) side_logit(side, y, row, V);
       }
       s_side = side;
       // every copy issued has been consumed once the consumers pass their last

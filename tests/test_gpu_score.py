@@ -77,6 +77,26 @@ def test_score_side_inputs_and_eligibility():
     check(inp, run_score(inp))
 
 
+@pytest.mark.parametrize("N,V", [(6, 20001), (400, 5000)])   # rows split over a cluster, and not
+def test_score_token_outside_the_vocabulary(N, V):
+    """Every value outside [0, V) has no probability, the largest and smallest of the type too: u and score are NaN."""
+    x = H.to_dev(W.make_score_inputs(N, V, 1, 1, seed=V).logits, "bf16")
+    outside = [-1, V, 2**31 - 1, -2**31]
+    tok = torch.zeros(N, dtype=torch.int32, device="cuda")
+    tok[:4] = torch.tensor(outside)
+    r = api.cover_score_fwd(x, 1, 0, cur_tok=tok)
+    ref = api.cover_score_fwd(x, 1, 0, cur_tok=torch.zeros_like(tok))
+    assert r["score"][:4].isnan().all() and torch.equal(r["score"][4:], ref["score"][4:])
+    assert torch.equal(r["maxprob"], ref["maxprob"])
+    # in the decision step such a row has no score: neither counted in n_t nor chosen
+    t, flags = tok.clone(), torch.zeros(N, dtype=torch.uint8, device="cuda")
+    d = api.cover_score_decide_fwd(x, 1, t, flags, flags.clone(), tau_draft=0.9, draft_budget=1, remask_budget=3, mask_id=3,
+                                   max_seeds=N)
+    assert d["score"][:4].isneginf().all() and int(d["stats"][0, 4]) == N - 4
+    assert int(flags[:4].sum()) == 0 and t[:4].tolist() == outside
+    assert api.cover_device_status() == 0
+
+
 @pytest.mark.parametrize("per,k,frac", [(1000, 32, 0.012), (300, 20, 0.012), (1000, 6, 0.003)])
 def test_score_topk_fewer_eligible_than_k(per, k, frac):
     """General path with fewer eligible rows than k: the list ends in -1 / -inf."""
