@@ -344,7 +344,8 @@ __device__ __forceinline__ bool row_write(const RowOut& r, const RowSide& side, 
   const float Zf = r.Z;
   const float lnZ = logf(Zf);
   const float H = lnZ - 0.6931471805599453f * r.q;
-  const float u = side.greedy ? lnZ : lnZ - (side.xy - r.M);
+  // a row without a greedy token (no logit above -inf) has no uncertainty of it either
+  const float u = !side.greedy ? lnZ - (side.xy - r.M) : r.M != -INFINITY ? lnZ : __int_as_float(0x7fc00000);
   maxprob[n] = 1.0f / Zf;
   entropy[n] = H;
   argmax[n] = r.yhat;

@@ -97,6 +97,18 @@ def test_score_token_outside_the_vocabulary(N, V):
     assert api.cover_device_status() == 0
 
 
+@pytest.mark.parametrize("N,V", [(6, 20001), (400, 5000)])   # rows split over a cluster, and not
+def test_score_rows_without_a_greedy_token(N, V):
+    """A row of -inf has no greedy token: its score is NaN, not -inf, beside rows that it leaves as they are."""
+    x = H.to_dev(W.make_score_inputs(N, V, 1, 1, seed=V).logits, "bf16")
+    ref = api.cover_score_fwd(x, 1, 0)
+    x[1] = -float("inf")
+    r = api.cover_score_fwd(x, 1, 0)
+    others = torch.arange(N, device="cuda") != 1
+    assert r["score"][1].isnan() and torch.equal(r["score"][others], ref["score"][others])
+    assert api.cover_device_status() == 0
+
+
 @pytest.mark.parametrize("per,k,frac", [(1000, 32, 0.012), (300, 20, 0.012), (1000, 6, 0.003)])
 def test_score_topk_fewer_eligible_than_k(per, k, frac):
     """General path with fewer eligible rows than k: the list ends in -1 / -inf."""
