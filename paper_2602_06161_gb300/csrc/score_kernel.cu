@@ -80,9 +80,15 @@ __device__ __forceinline__ void kahan_add(float& sum, float& c, float x) {
   sum = t;
 }
 
+// t of the maximum itself is the rounding of its reference, up to half a unit in the last place: below
+// this reference 2^t can overflow. A masked logit is often the type's lowest value, and it may be the
+// maximum of a lane's or a slice's every element: references stop here, where what lies lower has 2^t = 0.
+// (A row of nothing else has no finite sums.)
+constexpr float kLowestRef = -2147483648.0f;   // -2^31
+
 // Move the exponent reference to a larger maximum new_m.
 __device__ __forceinline__ void raise_max(RowAcc& a, float new_m, int new_i, int new_u) {
-  const float new_ref = new_m * kLog2e;
+  const float new_ref = fmaxf(new_m * kLog2e, kLowestRef);
   if (a.m != -INFINITY) {
     const float d = a.mref - new_ref;  // <= 0
     const float f = ex2_approx(d);
@@ -284,7 +290,9 @@ __device__ __forceinline__ RowSum row_combine(const RowSum* part, int lane) {
 #pragma unroll
   for (int o = C / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
   int y = r.M == M ? r.yhat : 0x7fffffff;
-  if (r.M != -INFINITY) {
+  if (r.M < M && r.M * kLog2e < kLowestRef) {
+    r.zh = r.zl = r.sh = r.sl = 0.0f;   // a slice of masked logits (two such bf16 maxima differ by 2^23 at least)
+  } else if (r.M != -INFINITY) {
     // d + dl = (r.M - M) log2 e to twice the precision: its rounding would shift the whole slice
     const float d = __fmul_rn(r.M - M, kLog2e);   // <= 0
     const float dl = fmaf(r.M - M, kLog2e, -d);

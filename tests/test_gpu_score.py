@@ -109,6 +109,29 @@ def test_score_rows_without_a_greedy_token(N, V):
     assert api.cover_device_status() == 0
 
 
+LOWEST = float(torch.finfo(torch.bfloat16).min)
+
+
+@pytest.mark.parametrize("low", [LOWEST, -1e38, -1e35, -1e30, -1e10, -1e9])
+@pytest.mark.parametrize("N,V", [(4, 20001), (4, 126464), (400, 20001), (400, 5000)])   # split rows and not
+def test_score_masked_logits(N, V, low):
+    """Masked logits: in the elements past the aligned vectors, in whole batches of a lane, in whole slices of
+    a row, at its start and between. They have no weight. (t 2^t of the lowest value is -inf times 0: no entropy.)"""
+    inp = W.make_score_inputs(N, V, 1, 1, seed=V)
+    x = H.to_dev(inp.logits, "bf16")
+    spans = [(V - 1, V), (V - 5, V), (V - 40, V), (2 * V // 3, V), (V // 2, V), (0, 1), (0, V // 3), (V // 4, V // 2),
+             (1, V), (0, V - 1)]
+    for lo, hi in spans:
+        y = x.clone()
+        y[:, lo:hi] = low
+        r = {k: v.cpu().numpy() for k, v in api.cover_score_fwd(y, 1, 0).items()}
+        ref = oracle.score_rows(y[:3].double().cpu().numpy())
+        assert np.array_equal(r["argmax"][:3], ref["argmax"]), (lo, hi)
+        for k in ("maxprob", "score") + (("entropy",) if low > LOWEST else ()):
+            assert np.abs(r[k][:3] - ref[k]).max() <= TOL, (lo, hi, k, r[k][:3], ref[k])
+    assert api.cover_device_status() == 0
+
+
 @pytest.mark.parametrize("per,k,frac", [(1000, 32, 0.012), (300, 20, 0.012), (1000, 6, 0.003)])
 def test_score_topk_fewer_eligible_than_k(per, k, frac):
     """General path with fewer eligible rows than k: the list ends in -1 / -inf."""
