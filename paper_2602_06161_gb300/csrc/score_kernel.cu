@@ -228,6 +228,8 @@ __device__ __forceinline__ RowSum row_reduce(const RowAcc& a, const uint16_t* ro
     const float ss = a.s - a.sc;
     z = f * zz;
     sv = f * fmaf(d, zz, ss);
+  } else {
+    z = a.z - a.zc;   // 0, or NaN if a lane without a maximum has seen one
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -277,7 +279,7 @@ __device__ __forceinline__ RowSum row_reduce(const RowAcc& a, const uint16_t* ro
 __device__ __forceinline__ RowOut row_finish(const RowSum& r) {
   const float q0 = r.sh / r.zh;
   const float res = fmaf(-q0, r.zh, r.sh) + (r.sl - q0 * r.zl);
-  return {r.M, r.yhat, r.zh + r.zl, q0 + res / r.zh};
+  return {r.M, r.yhat, r.M != -INFINITY ? r.zh + r.zl : 0.0f, q0 + res / r.zh};
 }
 
 // The sum of the row slices in part[0 .. C), on the lanes of one warp: every lane returns it.

@@ -132,6 +132,21 @@ def test_score_masked_logits(N, V, low):
     assert api.cover_device_status() == 0
 
 
+@pytest.mark.parametrize("N,V", [(4, 20001), (4, 126464), (400, 20001), (400, 5000)])   # split rows and not
+def test_score_nan_logits_show(N, V):
+    """One NaN logit anywhere, or a slice of them, leaves its row NaN and the other rows as they are."""
+    x = H.to_dev(W.make_score_inputs(N, V, 1, 1, seed=V).logits, "bf16")
+    ref = api.cover_score_fwd(x, 1, 0)
+    for lo, hi in [(V - 1, V), (0, 1), (V // 2, V // 2 + 1), (V // 3, V), (V - 3, V)]:
+        y = x.clone()
+        y[1, lo:hi] = float("nan")
+        r = api.cover_score_fwd(y, 1, 0)
+        others = torch.arange(N, device="cuda") != 1
+        for k in ("maxprob", "entropy", "score"):
+            assert r[k][1].isnan() and torch.equal(r[k][others], ref[k][others]), (lo, hi, k)
+    assert api.cover_device_status() == 0
+
+
 @pytest.mark.parametrize("per,k,frac", [(1000, 32, 0.012), (300, 20, 0.012), (1000, 6, 0.003)])
 def test_score_topk_fewer_eligible_than_k(per, k, frac):
     """General path with fewer eligible rows than k: the list ends in -1 / -inf."""
