@@ -94,6 +94,57 @@ __device__ __forceinline__ float2 ld_cluster2(uint32_t addr) {
   return v;
 }
 
+// A whole warp writes row `row` of head `head` again, its keys one by one and the excluded one left out.
+// The tiled loop gives that key p = 0, which drops its term only if its cached value row is finite; a
+// seed row whose result is not comes here, after the rest. (32 heads x 512 x 512, D = 128: 118.4 against
+// 117.0 us without the check, the tiled loop being scheduled otherwise; leaving the term out in that loop
+// took 124.8, going through the keys again before the epilogue 122.5.)
+template <int D>
+__device__ __noinline__ void redo_seed_row(const float* __restrict__ q, const float* __restrict__ kc,
+                                           const float* __restrict__ vc, const float* __restrict__ km,
+                                           const float* __restrict__ vm, int n_seeds, int Hq, int Hkv, int Lq, int L,
+                                           int q0, unsigned head, int row, int slot, float* __restrict__ out,
+                                           float* __restrict__ lse) {
+  constexpr int E = D / 32;
+  const int lane = threadIdx.x & 31;
+  const size_t kv_head = static_cast<size_t>(head / static_cast<unsigned>(Hq)) * Hkv +
+                         static_cast<int>(head % static_cast<unsigned>(Hq)) / (Hq / Hkv);
+  const size_t at = (static_cast<size_t>(head) * Lq + row) * D + lane;
+  const float scale = 1.0f / sqrtf(static_cast<float>(D));
+  float qr[E], acc[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    qr[e] = q[at + 32 * e];
+    acc[e] = 0.0f;
+  }
+  float m = -INFINITY, l = 0.0f;
+#pragma unroll 1
+  for (int j = 0; j <= L; ++j) {   // j == L: the masked-input pair
+    if (j == q0 + row) continue;
+    const bool self = j == L;
+    const size_t src = (self ? kv_head * n_seeds + slot : kv_head * L + j) * D + lane;
+    const float* const kr = (self ? km : kc) + src;
+    const float* const vr = (self ? vm : vc) + src;
+    float dot = 0.0f;
+#pragma unroll
+    for (int e = 0; e < E; ++e) dot = fmaf(qr[e], kr[32 * e], dot);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+    const float s = dot * scale;
+    const float m_new = fmaxf(m, s);
+    const float a = m == -INFINITY ? 0.0f : expf(m - m_new);
+    const float p = expf(s - m_new);
+    l = l * a + p;
+#pragma unroll
+    for (int e = 0; e < E; ++e) acc[e] = acc[e] * a + p * vr[32 * e];
+    m = m_new;
+  }
+  const float inv = 1.0f / l;
+#pragma unroll
+  for (int e = 0; e < E; ++e) out[at + 32 * e] = acc[e] * inv;
+  if (lse != nullptr && lane == 0) lse[static_cast<size_t>(head) * Lq + row] = m + logf(l);
+}
+
 // C > 1: the keys of a row tile are split over the C CTAs of a cluster. Each leaves its (m, l, O) in
 // its own shared memory, and CTA k combines rows k, k + C, ... from all of them.
 template <int D, int TM, int C>
@@ -268,6 +319,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     cp_async_commit();
   }
 
+  bool bad = false;   // a seed row of this thread came out not finite
   if constexpr (C > 1) {
     // this split's rows to shared memory (every warp is done with K and V): O over the K tile,
     // (m, l) over the V tile
@@ -328,8 +380,10 @@ __global__ void __launch_bounds__(kThreads, 2)
         acc.z = fmaf(p, vm[mrow + 2], acc.z);
         acc.w = fmaf(p, vm[mrow + 3], acc.w);
       }
+      bool redo = false;
       if (row0 + r < Lq) {
         const float inv = 1.0f / ll;
+        redo = is_seed && !(isfinite(acc.x * inv) && isfinite(acc.y * inv) && isfinite(acc.z * inv) && isfinite(acc.w * inv));
         const size_t row = static_cast<size_t>(head) * Lq + row0 + r;
         float* op = out + row * D + 4 * c4;
         if (vec) {
@@ -342,6 +396,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
         if (lse != nullptr && c4 == 0) lse[row] = mm + logf(ll);
       }
+      bad |= redo;
     }
     cluster_sync();   // no CTA leaves while another reads its shared memory
   } else {
@@ -351,7 +406,8 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
       for (int off = 8; off > 1; off >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
       const int sl = slot[r];
-      if (__any_sync(0xffffffffu, sl != kNoSlot)) {
+      const bool warp_seed = __any_sync(0xffffffffu, sl != kNoSlot);
+      if (warp_seed) {
         // merge the masked-input self term (k_i, v_i) of the warp's seed rows
         const bool is_seed = sl != kNoSlot;
         const size_t mrow = (kv_head * n_seeds + (is_seed ? sl : 0)) * D;
@@ -402,7 +458,24 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
         if (lse != nullptr && tx == 0) lse[row] = m[i] + logf(l[i]);
       }
+      if (warp_seed) {
+        float probe = 0.0f;   // NaN if one of this thread's sums is not finite
+#pragma unroll
+        for (int c = 0; c < 2 * kC; ++c) {
+          float x, y;
+          f2_unpack(o[i][c], x, y);
+          probe = fmaf(x, 0.0f, fmaf(y, 0.0f, probe));
+        }
+        const bool redo = sl != kNoSlot && row0 + r < Lq && probe != 0.0f;
+        bad |= redo;
+      }
     }
+  }
+  if (__syncthreads_or(bad)) {
+#pragma unroll 1
+    for (int r = C > 1 ? rank + C * warp : warp; r < T::kBM && row0 + r < Lq; r += C * (kThreads / 32))
+      if (slot[r] != kNoSlot)
+        redo_seed_row<D>(q, kc, vc, km, vm, n_seeds, Hq, Hkv, Lq, L, q0, head, row0 + r, slot[r], out, lse);
   }
 }
 

@@ -126,6 +126,27 @@ def test_f32_key_split(Hq, Hkv, Lk, D, Lq, q0, S):
     H.assert_f32_close(out.cpu().numpy(), ref, lse.cpu().numpy(), ref_lse)
 
 
+@pytest.mark.parametrize("Hq,L,D", [(2, 70, 64), (50, 96, 128), (38, 130, 64), (2, 300, 128)])   # row tiles and splits
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_f32_seed_rows_do_not_read_their_own_cached_row(Hq, L, D, bad):
+    """A seed row's view has the masked-input pair in the place of its cached one, whatever that holds; the
+    other rows of its tile, which do attend to it, are not finite."""
+    inp = W.make_attn_inputs(1, Hq, Hq, L, D, 1, dtype="f32", seed=L)
+    dev = [H.to_dev(x, "f32") for x in (inp.q, inp.k_cached, inp.v_cached, inp.k_seedmask, inp.v_seedmask)]
+    at = int(inp.seed_idx[0, 0])
+    seeds = H.to_dev(inp.seed_idx, "i32")
+    ref, ref_lse = api.cover_attn_fwd_f32(*dev, seeds)
+    dev[2][:, :, at, ::3] = bad
+    out, lse = api.cover_attn_fwd_f32(*dev, seeds)
+    # the same sums in another order: as far apart as the kernel may be from the oracle, twice
+    close = lambda a, b: float((a - b).abs().max()) <= 2 * H.TOL_F32   # noqa: E731
+    assert close(out[:, :, at], ref[:, :, at]) and close(lse, ref_lse)
+    dev[1][:, :, at] = bad   # nor its key
+    out, lse = api.cover_attn_fwd_f32(*dev, seeds)
+    assert close(out[:, :, at], ref[:, :, at]) and close(lse[:, :, at], ref_lse[:, :, at])
+    assert not out[:, :, :at, ::3].isfinite().any() and api.cover_device_status() == 0
+
+
 @pytest.mark.parametrize("which", range(4))
 def test_f32_unaligned_rows_equal_aligned(which):
     """A tensor that is only 4-byte aligned takes the 4-byte copies: the same bits."""
