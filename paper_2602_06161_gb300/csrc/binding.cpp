@@ -88,6 +88,13 @@ double real(PyObject* o) {
   return PyFloat_AS_DOUBLE(o);
 }
 
+// An object whose truth value raises goes to the caller's own path, which raises it before anything is launched.
+bool truth(PyObject* o) {
+  const int t = PyObject_IsTrue(o);
+  need(t >= 0);
+  return t != 0;
+}
+
 void* stream_of(PyObject* o) {
   need(none(o));
   return c10::cuda::getCurrentCUDAStream().stream();
@@ -190,7 +197,7 @@ PyObject* attn(PyObject*, PyObject* const* a, Py_ssize_t n) {
     float* lse = nullptr;
     if (!none(a[9])) {
       lse = ptr<float>(tensor(a[9], at::kFloat, 3));
-    } else if (PyObject_IsTrue(a[10]) == 1) {
+    } else if (truth(a[10])) {
       lse = ptr<float>(new_lse = empty(q.sizes().slice(0, 3), at::kFloat, q));
     }
     const void *pq = ptr<void>(q), *pk = ptr<void>(k), *pv = ptr<void>(v);
@@ -251,7 +258,7 @@ PyObject* decide(PyObject*, PyObject* const* a, Py_ssize_t n) {
     uint8_t *flags = ptr<uint8_t>(tensor(a[3], at::kByte, 1)), *cnt = ptr<uint8_t>(tensor(a[4], at::kByte, 1));
     const float tau = static_cast<float>(real(a[5]));
     const int budget = integer(a[6]), remask = integer(a[7]), mask_id = integer(a[8]);
-    const int min_one = PyObject_IsTrue(a[9]) == 1 ? 1 : 0;
+    const int min_one = truth(a[9]) ? 1 : 0;
     const int pos0 = integer(a[10]), max_seeds = integer(a[11]), phase = integer(a[12]);
     const float *d_in = ptr_or_null<float>(a[13], at::kFloat, 1), *d_out = ptr_or_null<float>(a[14], at::kFloat, 1);
     const uint8_t* draft_ok = ptr_or_null<uint8_t>(a[15], at::kByte, 1);

@@ -107,3 +107,22 @@ def test_errors_are_those_of_the_python_path():
     assert e.value.code == -1
     with pytest.raises(TypeError, match="logits must be torch.bfloat16"):
         api.cover_score_fwd(q.float()[0, 0], 1, 1, workspace=api.score_workspace(1))
+
+
+class _NoTruth:
+    def __bool__(self):
+        raise ArithmeticError("no truth value")
+
+
+def test_a_flag_without_a_truth_value_raises_before_anything_is_launched():
+    q, k = _r(1, 2, 64, 128), _r(1, 2, 64, 128, seed=9)
+    out = torch.zeros_like(q)
+    with pytest.raises(ArithmeticError, match="no truth value"):
+        api.cover_attn_fwd(q, k, k, out=out, want_lse=_NoTruth())
+    x = _r(12, 1003, seed=5)
+    tok, flags = torch.full((12,), 1000, device="cuda", dtype=torch.int32), torch.zeros(12, device="cuda", dtype=torch.uint8)
+    with pytest.raises(ArithmeticError, match="no truth value"):
+        api.cover_score_decide_fwd(x, 2, tok, flags, flags.clone(), tau_draft=0.0, draft_budget=2, remask_budget=3,
+                                   mask_id=1000, min_one=_NoTruth(), workspace=api.decide_workspace(12, 2))
+    torch.cuda.synchronize()
+    assert not out.any() and (tok == 1000).all() and not flags.any()
