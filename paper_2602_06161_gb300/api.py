@@ -95,10 +95,11 @@ def _attn(fn_name, dtype, q, k_cached, v_cached, k_seedmask, v_seedmask, seed_id
 def cover_attn_fwd(q, k_cached, v_cached, k_seedmask=None, v_seedmask=None, seed_idx=None, *,
                    out=None, lse=None, want_lse=True, stream=None):
     """Two-view override attention (bf16). Returns (out [B,Hq,L,D] bf16, lse [B,Hq,L] f32 or None)."""
-    r = (_nat or _native()).attn(0, q, k_cached, v_cached, k_seedmask, v_seedmask, seed_idx, 0, out, lse, want_lse,
-                                 stream)
-    if r is not None:
-        return _done("cover_attn_fwd", r)
+    if stream is None:
+        r = (_nat or _native()).attn(0, q, k_cached, v_cached, k_seedmask, v_seedmask, seed_idx, 0, out, lse,
+                                     want_lse, None)
+        if r is not None:
+            return _done("cover_attn_fwd", r)
     return _attn("cover_attn_fwd", torch.bfloat16, q, k_cached, v_cached, k_seedmask, v_seedmask, seed_idx,
                  out, lse, want_lse, stream)
 
@@ -106,10 +107,11 @@ def cover_attn_fwd(q, k_cached, v_cached, k_seedmask=None, v_seedmask=None, seed
 def cover_attn_fwd_f32(q, k_cached, v_cached, k_seedmask=None, v_seedmask=None, seed_idx=None, *,
                        out=None, lse=None, want_lse=True, stream=None):
     """Two-view override attention in fp32 (CUDA cores)."""
-    r = (_nat or _native()).attn(1, q, k_cached, v_cached, k_seedmask, v_seedmask, seed_idx, 0, out, lse, want_lse,
-                                 stream)
-    if r is not None:
-        return _done("cover_attn_fwd_f32", r)
+    if stream is None:
+        r = (_nat or _native()).attn(1, q, k_cached, v_cached, k_seedmask, v_seedmask, seed_idx, 0, out, lse,
+                                     want_lse, None)
+        if r is not None:
+            return _done("cover_attn_fwd_f32", r)
     return _attn("cover_attn_fwd_f32", torch.float32, q, k_cached, v_cached, k_seedmask, v_seedmask, seed_idx,
                  out, lse, want_lse, stream)
 
@@ -152,10 +154,11 @@ def _attn_prefix(fn_name, dtype, q, k_cached, v_cached, k_seedmask, v_seedmask, 
 def cover_attn_fwd_prefix(q, k_cached, v_cached, k_seedmask=None, v_seedmask=None, seed_idx=None, *, q0: int,
                           out=None, lse=None, want_lse=True, stream=None):
     """Two-view attention for a window of Lq query rows at memory positions q0 .. q0+Lq-1 (bf16)."""
-    r = (_nat or _native()).attn(2, q, k_cached, v_cached, k_seedmask, v_seedmask, seed_idx, q0, out, lse, want_lse,
-                                 stream)
-    if r is not None:
-        return _done("cover_attn_fwd_prefix", r)
+    if stream is None:
+        r = (_nat or _native()).attn(2, q, k_cached, v_cached, k_seedmask, v_seedmask, seed_idx, q0, out, lse,
+                                     want_lse, None)
+        if r is not None:
+            return _done("cover_attn_fwd_prefix", r)
     return _attn_prefix("cover_attn_fwd_prefix", torch.bfloat16, q, k_cached, v_cached, k_seedmask, v_seedmask,
                         seed_idx, q0, out, lse, want_lse, stream)
 
@@ -163,10 +166,11 @@ def cover_attn_fwd_prefix(q, k_cached, v_cached, k_seedmask=None, v_seedmask=Non
 def cover_attn_fwd_prefix_f32(q, k_cached, v_cached, k_seedmask=None, v_seedmask=None, seed_idx=None, *, q0: int,
                               out=None, lse=None, want_lse=True, stream=None):
     """The prefix-window attention in fp32 (CUDA cores)."""
-    r = (_nat or _native()).attn(3, q, k_cached, v_cached, k_seedmask, v_seedmask, seed_idx, q0, out, lse, want_lse,
-                                 stream)
-    if r is not None:
-        return _done("cover_attn_fwd_prefix_f32", r)
+    if stream is None:
+        r = (_nat or _native()).attn(3, q, k_cached, v_cached, k_seedmask, v_seedmask, seed_idx, q0, out, lse,
+                                     want_lse, None)
+        if r is not None:
+            return _done("cover_attn_fwd_prefix_f32", r)
     return _attn_prefix("cover_attn_fwd_prefix_f32", torch.float32, q, k_cached, v_cached, k_seedmask, v_seedmask,
                         seed_idx, q0, out, lse, want_lse, stream)
 
@@ -213,9 +217,10 @@ def cover_score_fwd(logits, n_seq: int, topk: int, *, cur_tok=None, d_in=None, d
     Returns a dict of CUDA tensors: maxprob, entropy, argmax, score [N];
     topk_idx [n_seq, topk] int32 and topk_score [n_seq, topk] f32.
     """
-    r = (_nat or _native()).score(logits, n_seq, topk, cur_tok, d_in, d_out, eligible, workspace, out, stream)
-    if r is not None:
-        return _done("cover_score_fwd", r)
+    if stream is None and out is None and (workspace is not None or topk == 0):
+        r = (_nat or _native()).score(logits, n_seq, topk, cur_tok, d_in, d_out, eligible, workspace, None, None)
+        if r is not None:
+            return _done("cover_score_fwd", r)
     _need(logits, "logits", torch.bfloat16, 2)
     N, V = logits.shape
     dev = logits.device
@@ -282,9 +287,10 @@ def cover_score_fwd_noalloc(logits, n_seq: int, topk: int, *, cur_tok=None, d_in
 
 
 def _seed_kv(fn_name, k, v, seed_idx, k_cache, v_cache, stream):
-    r = (_nat or _native()).kv(int(fn_name == "cover_seed_kv_override"), k, v, seed_idx, k_cache, v_cache, stream)
-    if r is not None:
-        return _done(fn_name, r)
+    if stream is None and seed_idx is not None:
+        r = (_nat or _native()).kv(int(fn_name == "cover_seed_kv_override"), k, v, seed_idx, k_cache, v_cache, None)
+        if r is not None:
+            return _done(fn_name, r)
     if k.dtype not in (torch.bfloat16, torch.float32):
         raise TypeError("k must be bfloat16 or float32")
     _need(k, "k", k.dtype, 4)
@@ -351,10 +357,12 @@ def cover_score_decide_fwd(logits, n_seq: int, tok, flags, remask_cnt, *, tau_dr
     run (score, seed_idx and n_seeds are left as they are); cover_attn_mass_fwd
     and cover_seed_select_fwd on the same workspace complete the step.
     """
-    r = (_nat or _native()).decide(logits, n_seq, tok, flags, remask_cnt, tau_draft, draft_budget, remask_budget, mask_id,
-                                   min_one, pos0, max_seeds, phase, d_in, d_out, draft_ok, workspace, out, stream)
-    if r is not None:
-        return _done("cover_score_decide_fwd", r)
+    if stream is None and out is None and workspace is not None and type(tau_draft) is float:
+        r = (_nat or _native()).decide(logits, n_seq, tok, flags, remask_cnt, tau_draft, draft_budget, remask_budget,
+                                       mask_id, min_one, pos0, max_seeds, phase, d_in, d_out, draft_ok, workspace, None,
+                                       None)
+        if r is not None:
+            return _done("cover_score_decide_fwd", r)
     _need(logits, "logits", torch.bfloat16, 2)
     N, V = logits.shape
     dev = logits.device
@@ -429,10 +437,11 @@ def cover_attn_mass_fwd(q, k_cached, lse, tok, flags, *, mask_id: int, pos0: int
     cover_attn_fwd wrote it), tok int32 / flags uint8 [B * per] (the state
     after a COVER_DECIDE_UPDATE call). Returns (d_in, d_out), float32 [B * per].
     """
-    r = (_nat or _native()).mass(q, k_cached, lse, tok, flags, mask_id, pos0, per, k_seedmask, seed_idx, workspace, d_in,
-                                 d_out, stream)
-    if r is not None:
-        return _done("cover_attn_mass_fwd", r)
+    if stream is None and workspace is not None:
+        r = (_nat or _native()).mass(q, k_cached, lse, tok, flags, mask_id, pos0, per, k_seedmask, seed_idx, workspace,
+                                     d_in, d_out, None)
+        if r is not None:
+            return _done("cover_attn_mass_fwd", r)
     _need(q, "q", torch.bfloat16, 4)
     _need(k_cached, "k_cached", torch.bfloat16, 4)
     _need(lse, "lse", torch.float32, 3)

@@ -38,30 +38,6 @@ decltype(&cover_attn_mass_fwd) f_mass;
 decltype(&cover_seed_kv_gather) f_gather;
 decltype(&cover_seed_kv_override) f_override;
 
-// Thrown for a call that the caller's own path has to take.
-struct Other {};
-
-void need(bool ok) {
-  if (!ok) throw Other();
-}
-
-void need_plain() {
-  need(!c10::impl::TorchDispatchModeTLS::any_modes_set() && at::impl::PythonTorchFunctionTLS::stack_len() == 0 &&
-       !at::globalContext().deterministicAlgorithms());
-}
-
-const Tensor& any_tensor(PyObject* o) {
-  need(THPVariable_CheckExact(o));
-  return THPVariable_Unpack(o);
-}
-
-const Tensor& tensor(PyObject* o, at::ScalarType dtype, int dims) {
-  const Tensor& t = any_tensor(o);
-  need(t.scalar_type() == dtype && t.is_cuda() && t.dim() == dims && t.is_contiguous());
-  for (const int64_t n : t.sizes()) need(n <= INT_MAX);
-  return t;
-}
-
 bool none(PyObject* o) { return o == Py_None; }
 
 int dim(const Tensor& t, int i) { return static_cast<int>(t.size(i)); }
@@ -70,35 +46,67 @@ template <typename T>
 T* ptr(const Tensor& t) {
   return static_cast<T*>(t.data_ptr());
 }
-template <typename T>
-T* ptr_or_null(PyObject* o, at::ScalarType dtype, int dims) {
-  return none(o) ? nullptr : ptr<T>(tensor(o, dtype, dims));
-}
 
-int integer(PyObject* o) {
-  need(PyLong_CheckExact(o));
-  int over = 0;
-  const long v = PyLong_AsLongAndOverflow(o, &over);
-  need(over == 0 && v >= INT_MIN && v <= INT_MAX);
-  return static_cast<int>(v);
-}
+// Reads a call's arguments. The first one that is not of the plain form ends it: ok is false from then on,
+// what is returned is without meaning, and the call goes to the caller's own path. (No exception
+// says so: throwing and catching one took 6 to 10 us of a call that is then marshalled in Python.)
+struct Args {
+  bool ok = !c10::impl::TorchDispatchModeTLS::any_modes_set() && at::impl::PythonTorchFunctionTLS::stack_len() == 0 &&
+            !at::globalContext().deterministicAlgorithms();
 
-double real(PyObject* o) {
-  need(PyFloat_CheckExact(o));
-  return PyFloat_AS_DOUBLE(o);
-}
+  void need(bool cond) { ok = ok && cond; }
 
-// An object whose truth value raises goes to the caller's own path, which raises it before anything is launched.
-bool truth(PyObject* o) {
-  const int t = PyObject_IsTrue(o);
-  need(t >= 0);
-  return t != 0;
-}
+  const Tensor& any_tensor(PyObject* o) {
+    static const Tensor nothing;
+    need(THPVariable_CheckExact(o));
+    return ok ? THPVariable_Unpack(o) : nothing;
+  }
 
-void* stream_of(PyObject* o) {
-  need(none(o));
-  return c10::cuda::getCurrentCUDAStream().stream();
-}
+  const Tensor& tensor(PyObject* o, at::ScalarType dtype, int dims) {
+    const Tensor& t = any_tensor(o);
+    if (!ok) return t;
+    need(t.scalar_type() == dtype && t.is_cuda() && t.dim() == dims && t.is_contiguous());
+    for (const int64_t n : t.sizes()) need(n <= INT_MAX);
+    return t;
+  }
+
+  template <typename T>
+  T* pointer(PyObject* o, at::ScalarType dtype, int dims) {
+    const Tensor& t = tensor(o, dtype, dims);
+    return ok ? ptr<T>(t) : nullptr;
+  }
+  template <typename T>
+  T* pointer_or_null(PyObject* o, at::ScalarType dtype, int dims) {
+    return none(o) ? nullptr : pointer<T>(o, dtype, dims);
+  }
+
+  int integer(PyObject* o) {
+    need(PyLong_CheckExact(o));
+    if (!ok) return 0;
+    int over = 0;
+    const long v = PyLong_AsLongAndOverflow(o, &over);
+    need(over == 0 && v >= INT_MIN && v <= INT_MAX);
+    return static_cast<int>(v);
+  }
+
+  double real(PyObject* o) {
+    need(PyFloat_CheckExact(o));
+    return ok ? PyFloat_AS_DOUBLE(o) : 0.0;
+  }
+
+  // An object whose truth value raises goes to the caller's own path, which raises it before anything is launched.
+  bool truth(PyObject* o) {
+    if (!ok) return false;
+    const int t = PyObject_IsTrue(o);
+    need(t >= 0);
+    return t > 0;
+  }
+
+  void* stream(PyObject* o) {
+    need(none(o));
+    return ok ? c10::cuda::getCurrentCUDAStream().stream() : nullptr;
+  }
+};
 
 Tensor empty(at::IntArrayRef sizes, at::ScalarType dtype, const Tensor& like) {
   return at::detail::empty_cuda(sizes, dtype, like.device(), std::nullopt);
@@ -143,8 +151,8 @@ PyObject* dict_of(Item (&items)[N]) {
   return d;
 }
 
-// Runs f(launched); a call of another form, or one that an exception ended before its entry point
-// was called, is None.
+// Runs f(args, launched), which returns null for a call of another form; such a call, or one that an
+// exception ended before its entry point was called, is None.
 template <typename F>
 PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F&& f) {
   if (n != want) {
@@ -152,10 +160,10 @@ PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F&& f) {
     return nullptr;
   }
   bool launched = false;
+  Args args;
   try {
-    need_plain();
-    return f(launched);
-  } catch (const Other&) {
+    PyObject* r = args.ok ? f(args, launched) : nullptr;
+    if (r != nullptr || launched) return r;
   } catch (const std::exception& e) {
     if (launched) {
       if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what());
@@ -169,37 +177,38 @@ PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F&& f) {
 // attn(kind, q, k, v, km, vm, seed_idx, q0, out, lse, want_lse, stream); kind: 0 bf16, 1 f32 (whole
 // sequence), 2 bf16, 3 f32 (window at q0)
 PyObject* attn(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  return guarded(n, 12, [&](bool& launched) -> PyObject* {
-    const int kind = integer(a[0]);
+  return guarded(n, 12, [&](Args& in, bool& launched) -> PyObject* {
+    const int kind = in.integer(a[0]);
     const bool window = kind >= 2;
     const at::ScalarType dt = (kind & 1) != 0 ? at::kFloat : at::kBFloat16;
-    const Tensor &q = tensor(a[1], dt, 4), &k = tensor(a[2], dt, 4), &v = tensor(a[3], dt, 4);
+    const Tensor &q = in.tensor(a[1], dt, 4), &k = in.tensor(a[2], dt, 4), &v = in.tensor(a[3], dt, 4);
+    if (!in.ok) return nullptr;
     const int B = dim(q, 0), Hq = dim(q, 1), Lq = dim(q, 2), D = dim(q, 3), Hkv = dim(k, 1), L = dim(k, 2);
-    need(dim(k, 0) == B && dim(k, 3) == D && (window || L == Lq) && v.sizes() == k.sizes());
+    in.need(dim(k, 0) == B && dim(k, 3) == D && (window || L == Lq) && v.sizes() == k.sizes());
     int S = 0;
     const void *km = nullptr, *vm = nullptr;
     const int32_t* idx = nullptr;
     if (!none(a[6])) {
-      const Tensor& seeds = any_tensor(a[6]);
-      need(seeds.dim() == 2);
+      const Tensor& seeds = in.any_tensor(a[6]);
+      if (!in.ok || seeds.dim() != 2) return nullptr;
       if (seeds.size(1) > 0) {
-        const Tensor &si = tensor(a[6], at::kInt, 2), &tk = tensor(a[4], dt, 4), &tv = tensor(a[5], dt, 4);
+        const Tensor &si = in.tensor(a[6], at::kInt, 2), &tk = in.tensor(a[4], dt, 4), &tv = in.tensor(a[5], dt, 4);
+        if (!in.ok) return nullptr;
         S = dim(si, 1);
-        need(dim(si, 0) == B && dim(tk, 0) == B && dim(tk, 1) == Hkv && dim(tk, 2) == S && dim(tk, 3) == D &&
+        in.need(dim(si, 0) == B && dim(tk, 0) == B && dim(tk, 1) == Hkv && dim(tk, 2) == S && dim(tk, 3) == D &&
              tv.sizes() == tk.sizes());
         km = ptr<void>(tk), vm = ptr<void>(tv), idx = ptr<int32_t>(si);
       }
     }
-    const int q0 = window ? integer(a[7]) : 0;
-    void* stream = stream_of(a[11]);
+    const int q0 = window ? in.integer(a[7]) : 0;
+    void* stream = in.stream(a[11]);
+    void* out = in.pointer_or_null<void>(a[8], dt, 4);
+    float* lse = in.pointer_or_null<float>(a[9], at::kFloat, 3);
+    const bool make_lse = none(a[9]) && in.truth(a[10]);
+    if (!in.ok) return nullptr;
     Tensor new_out, new_lse;
-    void* out = none(a[8]) ? ptr<void>(new_out = empty(q.sizes(), dt, q)) : ptr<void>(tensor(a[8], dt, 4));
-    float* lse = nullptr;
-    if (!none(a[9])) {
-      lse = ptr<float>(tensor(a[9], at::kFloat, 3));
-    } else if (truth(a[10])) {
-      lse = ptr<float>(new_lse = empty(q.sizes().slice(0, 3), at::kFloat, q));
-    }
+    if (none(a[8])) out = ptr<void>(new_out = empty(q.sizes(), dt, q));
+    if (make_lse) lse = ptr<float>(new_lse = empty(q.sizes().slice(0, 3), at::kFloat, q));
     const void *pq = ptr<void>(q), *pk = ptr<void>(k), *pv = ptr<void>(v);
     const auto f = [](const void* p) { return static_cast<const float*>(p); };
     const int rc = call(launched, [&] {
@@ -221,16 +230,19 @@ PyObject* attn(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 // score(logits, n_seq, topk, cur_tok, d_in, d_out, eligible, workspace, out, stream)
 PyObject* score(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  return guarded(n, 10, [&](bool& launched) -> PyObject* {
-    const Tensor& x = tensor(a[0], at::kBFloat16, 2);
-    const int N = dim(x, 0), V = dim(x, 1), n_seq = integer(a[1]), topk = integer(a[2]);
-    need(n_seq >= 1 && topk >= 0 && none(a[8]));
-    const int32_t* cur = ptr_or_null<int32_t>(a[3], at::kInt, 1);
-    const float *d_in = ptr_or_null<float>(a[4], at::kFloat, 1), *d_out = ptr_or_null<float>(a[5], at::kFloat, 1);
-    const uint8_t* eligible = ptr_or_null<uint8_t>(a[6], at::kByte, 1);
-    need(topk == 0 || !none(a[7]));   // the caller allocates a missing workspace
-    void* ws = none(a[7]) ? nullptr : ptr<void>(any_tensor(a[7]));
-    void* stream = stream_of(a[9]);
+  return guarded(n, 10, [&](Args& in, bool& launched) -> PyObject* {
+    const Tensor& x = in.tensor(a[0], at::kBFloat16, 2);
+    if (!in.ok) return nullptr;
+    const int N = dim(x, 0), V = dim(x, 1), n_seq = in.integer(a[1]), topk = in.integer(a[2]);
+    in.need(n_seq >= 1 && topk >= 0 && none(a[8]));
+    const int32_t* cur = in.pointer_or_null<int32_t>(a[3], at::kInt, 1);
+    const float *d_in = in.pointer_or_null<float>(a[4], at::kFloat, 1), *d_out = in.pointer_or_null<float>(a[5], at::kFloat, 1);
+    const uint8_t* eligible = in.pointer_or_null<uint8_t>(a[6], at::kByte, 1);
+    in.need(topk == 0 || !none(a[7]));   // the caller allocates a missing workspace
+    void* stream = in.stream(a[9]);
+    const Tensor& work = none(a[7]) ? x : in.any_tensor(a[7]);
+    if (!in.ok) return nullptr;
+    void* ws = none(a[7]) ? nullptr : ptr<void>(work);
     Item r[] = {{"maxprob", empty({N}, at::kFloat, x)},
                 {"entropy", empty({N}, at::kFloat, x)},
                 {"argmax", empty({N}, at::kInt, x)},
@@ -251,20 +263,23 @@ PyObject* score(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // decide(logits, n_seq, tok, flags, remask_cnt, tau_draft, draft_budget, remask_budget, mask_id,
 // min_one, pos0, max_seeds, phase, d_in, d_out, draft_ok, workspace, out, stream)
 PyObject* decide(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  return guarded(n, 19, [&](bool& launched) -> PyObject* {
-    const Tensor& x = tensor(a[0], at::kBFloat16, 2);
-    const int N = dim(x, 0), V = dim(x, 1), n_seq = integer(a[1]);
-    int32_t* tok = ptr<int32_t>(tensor(a[2], at::kInt, 1));
-    uint8_t *flags = ptr<uint8_t>(tensor(a[3], at::kByte, 1)), *cnt = ptr<uint8_t>(tensor(a[4], at::kByte, 1));
-    const float tau = static_cast<float>(real(a[5]));
-    const int budget = integer(a[6]), remask = integer(a[7]), mask_id = integer(a[8]);
-    const int min_one = truth(a[9]) ? 1 : 0;
-    const int pos0 = integer(a[10]), max_seeds = integer(a[11]), phase = integer(a[12]);
-    const float *d_in = ptr_or_null<float>(a[13], at::kFloat, 1), *d_out = ptr_or_null<float>(a[14], at::kFloat, 1);
-    const uint8_t* draft_ok = ptr_or_null<uint8_t>(a[15], at::kByte, 1);
-    need(n_seq >= 1 && max_seeds >= 0 && none(a[17]));
-    void* ws = ptr<void>(any_tensor(a[16]));
-    void* stream = stream_of(a[18]);
+  return guarded(n, 19, [&](Args& in, bool& launched) -> PyObject* {
+    const Tensor& x = in.tensor(a[0], at::kBFloat16, 2);
+    if (!in.ok) return nullptr;
+    const int N = dim(x, 0), V = dim(x, 1), n_seq = in.integer(a[1]);
+    int32_t* tok = in.pointer<int32_t>(a[2], at::kInt, 1);
+    uint8_t *flags = in.pointer<uint8_t>(a[3], at::kByte, 1), *cnt = in.pointer<uint8_t>(a[4], at::kByte, 1);
+    const float tau = static_cast<float>(in.real(a[5]));
+    const int budget = in.integer(a[6]), remask = in.integer(a[7]), mask_id = in.integer(a[8]);
+    const int min_one = in.truth(a[9]) ? 1 : 0;
+    const int pos0 = in.integer(a[10]), max_seeds = in.integer(a[11]), phase = in.integer(a[12]);
+    const float *d_in = in.pointer_or_null<float>(a[13], at::kFloat, 1), *d_out = in.pointer_or_null<float>(a[14], at::kFloat, 1);
+    const uint8_t* draft_ok = in.pointer_or_null<uint8_t>(a[15], at::kByte, 1);
+    in.need(n_seq >= 1 && max_seeds >= 0 && none(a[17]));
+    void* stream = in.stream(a[18]);
+    const Tensor& work = in.any_tensor(a[16]);
+    if (!in.ok) return nullptr;
+    void* ws = ptr<void>(work);
     Item r[] = {{"maxprob", empty({N}, at::kFloat, x)},
                 {"entropy", empty({N}, at::kFloat, x)},
                 {"argmax", empty({N}, at::kInt, x)},
@@ -285,30 +300,34 @@ PyObject* decide(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 // mass(q, k, lse, tok, flags, mask_id, pos0, per, k_seedmask, seed_idx, workspace, d_in, d_out, stream)
 PyObject* mass(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  return guarded(n, 14, [&](bool& launched) -> PyObject* {
-    const Tensor &q = tensor(a[0], at::kBFloat16, 4), &k = tensor(a[1], at::kBFloat16, 4);
-    const Tensor &lse = tensor(a[2], at::kFloat, 3), &tok = tensor(a[3], at::kInt, 1), &flags = tensor(a[4], at::kByte, 1);
+  return guarded(n, 14, [&](Args& in, bool& launched) -> PyObject* {
+    const Tensor &q = in.tensor(a[0], at::kBFloat16, 4), &k = in.tensor(a[1], at::kBFloat16, 4);
+    const Tensor &lse = in.tensor(a[2], at::kFloat, 3), &tok = in.tensor(a[3], at::kInt, 1), &flags = in.tensor(a[4], at::kByte, 1);
+    if (!in.ok) return nullptr;
     const int B = dim(q, 0), Hq = dim(q, 1), L = dim(q, 2), D = dim(q, 3), Hkv = dim(k, 1);
-    const int mask_id = integer(a[5]), pos0 = integer(a[6]), per = integer(a[7]);
+    const int mask_id = in.integer(a[5]), pos0 = in.integer(a[6]), per = in.integer(a[7]);
     const int64_t rows = static_cast<int64_t>(B) * per;
-    need(per >= 1 && tok.size(0) == rows && flags.size(0) == rows);
+    in.need(per >= 1 && tok.size(0) == rows && flags.size(0) == rows);
     int S = 0;
     const void* km = nullptr;
     const int32_t* idx = nullptr;
     if (!none(a[9])) {
-      const Tensor& seeds = any_tensor(a[9]);
-      need(seeds.dim() == 2);
+      const Tensor& seeds = in.any_tensor(a[9]);
+      if (!in.ok || seeds.dim() != 2) return nullptr;
       if (seeds.size(1) > 0) {
-        idx = ptr<int32_t>(tensor(a[9], at::kInt, 2));
-        km = ptr<void>(tensor(a[8], at::kBFloat16, 4));
+        idx = in.pointer<int32_t>(a[9], at::kInt, 2);
+        km = in.pointer<void>(a[8], at::kBFloat16, 4);
         S = dim(seeds, 1);
       }
     }
-    void* ws = ptr<void>(any_tensor(a[10]));
-    void* stream = stream_of(a[13]);
+    void* stream = in.stream(a[13]);
+    const Tensor &work = in.any_tensor(a[10]), &given_in = none(a[11]) ? q : in.any_tensor(a[11]),
+                 &given_out = none(a[12]) ? q : in.any_tensor(a[12]);
+    if (!in.ok) return nullptr;
+    void* ws = ptr<void>(work);
     Tensor new_in, new_out;
-    float* d_in = ptr<float>(none(a[11]) ? (new_in = empty({rows}, at::kFloat, q)) : any_tensor(a[11]));
-    float* d_out = ptr<float>(none(a[12]) ? (new_out = empty({rows}, at::kFloat, q)) : any_tensor(a[12]));
+    float* d_in = ptr<float>(none(a[11]) ? (new_in = empty({rows}, at::kFloat, q)) : given_in);
+    float* d_out = ptr<float>(none(a[12]) ? (new_out = empty({rows}, at::kFloat, q)) : given_out);
     const void *pq = ptr<void>(q), *pk = ptr<void>(k);
     const float* pl = ptr<float>(lse);
     const int32_t* pt = ptr<int32_t>(tok);
@@ -323,18 +342,23 @@ PyObject* mass(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 // kv(swap, k, v, seed_idx, k_cache, v_cache, stream)
 PyObject* kv(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  return guarded(n, 7, [&](bool& launched) -> PyObject* {
-    const bool swap = integer(a[0]) != 0;
-    const at::ScalarType dt = any_tensor(a[1]).scalar_type();
-    need(dt == at::kBFloat16 || dt == at::kFloat);
-    const Tensor &k = tensor(a[1], dt, 4), &v = tensor(a[2], dt, 4), &seeds = tensor(a[3], at::kInt, 2);
+  return guarded(n, 7, [&](Args& in, bool& launched) -> PyObject* {
+    const bool swap = in.integer(a[0]) != 0;
+    const Tensor& any_k = in.any_tensor(a[1]);
+    if (!in.ok) return nullptr;
+    const at::ScalarType dt = any_k.scalar_type();
+    in.need(dt == at::kBFloat16 || dt == at::kFloat);
+    const Tensor &k = in.tensor(a[1], dt, 4), &v = in.tensor(a[2], dt, 4), &seeds = in.tensor(a[3], at::kInt, 2);
+    if (!in.ok) return nullptr;
     const int B = dim(k, 0), Hkv = dim(k, 1), L = dim(k, 2), D = dim(k, 3), S = dim(seeds, 1);
-    need(v.sizes() == k.sizes() && S > 0 && dim(seeds, 0) == B && none(a[4]) == none(a[5]) && (!swap || !none(a[4])));
-    void* stream = stream_of(a[6]);
+    in.need(v.sizes() == k.sizes() && S > 0 && dim(seeds, 0) == B && none(a[4]) == none(a[5]) && (!swap || !none(a[4])));
+    void* stream = in.stream(a[6]);
+    if (!in.ok) return nullptr;
     Tensor new_k, new_v;
-    const Tensor& kc = none(a[4]) ? (new_k = empty({B, Hkv, S, D}, dt, k)) : tensor(a[4], dt, 4);
-    const Tensor& vc = none(a[5]) ? (new_v = empty({B, Hkv, S, D}, dt, k)) : tensor(a[5], dt, 4);
-    need(dim(kc, 0) == B && dim(kc, 1) == Hkv && dim(kc, 2) == S && dim(kc, 3) == D && vc.sizes() == kc.sizes());
+    const Tensor& kc = none(a[4]) ? (new_k = empty({B, Hkv, S, D}, dt, k)) : in.tensor(a[4], dt, 4);
+    const Tensor& vc = none(a[5]) ? (new_v = empty({B, Hkv, S, D}, dt, k)) : in.tensor(a[5], dt, 4);
+    if (!in.ok || dim(kc, 0) != B || dim(kc, 1) != Hkv || dim(kc, 2) != S || dim(kc, 3) != D || vc.sizes() != kc.sizes())
+      return nullptr;
     void *pk = ptr<void>(k), *pv = ptr<void>(v), *pkc = ptr<void>(kc), *pvc = ptr<void>(vc);
     const int32_t* idx = ptr<int32_t>(seeds);
     const int elem = static_cast<int>(k.element_size());

@@ -41,3 +41,28 @@ def test_wrong_number_of_arguments():
 def test_not_a_tensor():
     with pytest.raises(TypeError, match="q must be a torch.Tensor"):
         api.cover_attn_fwd([1.0], None, None)
+
+
+def test_forms_that_the_native_path_does_not_take_are_not_offered_to_it(monkeypatch):
+    """A stream, given outputs, a missing workspace: such calls pay for one marshalling, not for two."""
+    class Native:
+        def __getattr__(self, name):
+            raise AssertionError(name + " was offered the call")
+
+    monkeypatch.setattr(api, "_nat", Native())
+    q, k, v = _qkv()
+    x, t, u = torch.zeros(4, 8, dtype=torch.bfloat16), torch.zeros(4, dtype=torch.int32), torch.zeros(4, dtype=torch.uint8)
+    f32, ws = torch.zeros(1, 2, 16), torch.zeros(64, dtype=torch.int32)
+    dec = dict(draft_budget=1, remask_budget=1, mask_id=0)
+    calls = [lambda: api.cover_attn_fwd(q, k, v, stream=0), lambda: api.cover_attn_fwd_prefix(q, k, v, q0=0, stream=0),
+             lambda: api.cover_score_fwd(x, 1, 1), lambda: api.cover_score_fwd(x, 1, 1, workspace=ws, out={}),
+             lambda: api.cover_score_fwd(x, 1, 0, stream=0), lambda: api.cover_seed_kv_gather(q, q, t[None], stream=0),
+             lambda: api.cover_score_decide_fwd(x, 1, t, u, u, tau_draft=0.5, **dec),
+             lambda: api.cover_score_decide_fwd(x, 1, t, u, u, tau_draft=0.5, workspace=ws, out={}, **dec),
+             lambda: api.cover_score_decide_fwd(x, 1, t, u, u, tau_draft=1, workspace=ws, **dec),
+             lambda: api.cover_attn_mass_fwd(q, k, f32, t, u, mask_id=0, pos0=0, per=4)]
+    for call in calls:
+        with pytest.raises(ValueError, match="must be a CUDA tensor"):
+            call()
+    with pytest.raises(AssertionError, match="attn was offered"):
+        api.cover_attn_fwd(q, k, v)
