@@ -8,6 +8,7 @@ from __future__ import annotations
 import ctypes
 import os
 import threading
+import warnings
 
 from . import build as _build
 
@@ -83,12 +84,29 @@ def load(build_if_needed: bool = True):
         return lib
 
 
+class _Declines:
+    """In the place of the native argument marshalling where it is not there: hands every call back."""
+
+    @staticmethod
+    def attn(*args):
+        return None
+
+    score = decide = mass = kv = attn
+
+
 def native():
     """The native argument marshalling, bound to the loaded library's entry points."""
     global _native
     if _native is None:
         lib = load()
-        from . import _binding
+        try:
+            if _build._binding_stale():
+                raise ImportError("_binding.so was not compiled for this PyTorch and interpreter")
+            from . import _binding
+        except ImportError as e:
+            warnings.warn(f"calls are marshalled in Python: {e}")
+            _native = _Declines
+            return _native
         _binding.bind([ctypes.cast(getattr(lib, name), _P).value for name in _BOUND])
         _native = _binding
     return _native

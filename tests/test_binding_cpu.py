@@ -1,5 +1,7 @@
 """The native argument marshalling takes only calls of plain CUDA tensors: any other form is handed
 back (None) with nothing launched, and the Python path raises its errors as it always did."""
+import sys
+
 import pytest
 import torch
 
@@ -66,3 +68,41 @@ def test_forms_that_the_native_path_does_not_take_are_not_offered_to_it(monkeypa
             call()
     with pytest.raises(AssertionError, match="attn was offered"):
         api.cover_attn_fwd(q, k, v)
+
+
+def test_the_binding_is_made_again_for_another_torch_or_interpreter(monkeypatch, tmp_path):
+    """The object reads PyTorch's and the interpreter's structures: it serves the ones it was compiled for only."""
+    from paper_2602_06161_gb300 import build
+
+    build.build()
+    assert not build._binding_stale()
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    assert build._binding_stale()
+    monkeypatch.undo()
+    monkeypatch.setattr(sys, "version", "9.9.9 (other)")
+    assert build._binding_stale()
+    monkeypatch.undo()
+    # a failure leaves no object behind, is not tried again for the same pair, and does not touch the library
+    monkeypatch.setattr(build, "BINDING", str(tmp_path / "_binding.so"))
+    monkeypatch.setattr(build, "BINDING_TAG", str(tmp_path / "binding.tag"))
+    (tmp_path / "_binding.so").write_text("of another torch")
+    monkeypatch.setenv("CXX", "no-such-compiler")
+    with pytest.warns(UserWarning, match="marshalled in Python"):
+        assert build.build() == build.LIB
+    assert not (tmp_path / "_binding.so").exists() and not build._binding_stale() and not build._stale()
+    # nor is one used that belongs to another pair and cannot be replaced
+    monkeypatch.setattr(build, "BINDING_TAG", str(tmp_path / "no" / "such" / "folder"))
+    monkeypatch.setattr(_lib, "_native", None)
+    with pytest.warns(UserWarning, match="marshalled in Python"):
+        assert _lib.native() is _lib._Declines
+
+
+def test_calls_work_without_the_binding(monkeypatch):
+    monkeypatch.setitem(sys.modules, "paper_2602_06161_gb300._binding", None)   # its import fails
+    monkeypatch.delattr("paper_2602_06161_gb300._binding", raising=False)
+    monkeypatch.setattr(_lib, "_native", None)
+    monkeypatch.setattr(api, "_nat", None)
+    with pytest.warns(UserWarning, match="marshalled in Python"):
+        with pytest.raises(ValueError, match="q must be a CUDA tensor"):   # the Python path's own check
+            api.cover_attn_fwd(*_qkv())
+    assert _lib.native().kv() is None
