@@ -397,6 +397,7 @@ struct ScoreParams {
   uint32_t* counters;
   int decide;          // kDecideFused: the last CTA of a segment decides; kDecideApart: decide_kernel does
   DecideArgs dec;
+  bool evict_first;    // the logits do not fit in L2
 };
 
 // Descending bitonic sort of n (a power of two) 64-bit keys in shared memory;
@@ -1318,16 +1319,26 @@ __device__ __forceinline__ void acc_batch(RowAcc& a, const uint4 (&w)[U], int i0
 // ---------------------------------------------------------------------------
 // row kernel: bulk copies of a row, or of a row's slice in each CTA of a cluster
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  // The logits are read once and may exceed L2: evicted first, they leave the rest of a step there
-  // (states, weights, the next kernels' code). The pass itself takes the same time; in a decoding
-  // step of Dream's shape (311 MB of logits) the launches around it went from 98.9 to 87.2 us.
+// L2 policy of the copies. Logits larger than L2 are gone before they could be read again: evicted
+// first, they leave the rest of a step there (states, weights, the next kernels' code). The pass itself
+// takes the same time; in a decoding step of Dream's shape (311 MB of logits) the launches around it
+// went from 98.9 to 87.2 us. Smaller ones stay where they are, for whoever reads them next: evicted first,
+// a second pass over 1024 rows of 32000 logits took 16.8 instead of 13.9 us, over 1024 of 50000 22.3 instead
+// of 20.2, over 300 of 126464 15.8 instead of 14.2.
+__device__ __forceinline__ uint64_t stream_policy(bool evict_first) {
+  uint64_t p;
+  if (evict_first)
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+  else
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+__device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar,
+                                          uint64_t policy) {
   asm volatile(
-      "{\n\t.reg .b64 policy;\n\t"
-      "createpolicy.fractional.L2::evict_first.b64 policy, 1.0;\n\t"
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1], %2, [%3], policy;\n\t}" ::"r"(smem_u32(smem_dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      " [%0], [%1], %2, [%3], %4;" ::"r"(smem_u32(smem_dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
       : "memory");
 }
 
@@ -1374,6 +1385,7 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
   const int nchunks = (elems_all + kChunkElems - 1) / kChunkElems;
   const uint16_t* src_row = row + first;
   uint8_t* ring = dsmem;
+  const uint64_t policy = stream_policy(P.evict_first);
 
   if (warp == kConsumerWarps && lane == 0) {
     // the producer initialises the ring and issues its first chunks at once, so their latency
@@ -1388,7 +1400,7 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
       const int elems = min(kChunkElems, elems_all - c * kChunkElems);
       mbar_arrive_expect_tx(&bar_full[c], static_cast<uint32_t>(elems * 2));
       bulk_load(ring + c * kChunkBytes, src_row + static_cast<size_t>(c) * kChunkElems,
-                static_cast<uint32_t>(elems * 2), &bar_full[c]);
+                static_cast<uint32_t>(elems * 2), &bar_full[c], policy);
     }
   }
   __syncthreads();
@@ -1418,7 +1430,7 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
         const int elems = min(kChunkElems, elems_all - c * kChunkElems);
         mbar_arrive_expect_tx(&bar_full[st], static_cast<uint32_t>(elems * 2));
         bulk_load(ring + st * kChunkBytes, src_row + static_cast<size_t>(c) * kChunkElems,
-                  static_cast<uint32_t>(elems * 2), &bar_full[st]);
+                  static_cast<uint32_t>(elems * 2), &bar_full[st], policy);
         if (c == kRingStages) side_logit(side, y, row, V);
       }
       s_side = side;
@@ -1586,20 +1598,26 @@ int row_split(int N, int V, int n_sm) {
 }
 
 int launch_score_impl(const ScoreArgs& a, const DecideArgs* d, int* status, cudaStream_t stream) {
-  static ContextCache<int> sms;
-  int n_sm = 0;
-  const int rc = sms.get(&n_sm, [](int& v) {
+  struct Device {
+    int n_sm, l2_bytes;
+  };
+  static ContextCache<Device> devices;
+  Device gpu{};
+  const int rc = devices.get(&gpu, [](Device& v) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return -3;
-    return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? 0 : -3;
+    return cudaDeviceGetAttribute(&v.n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+                   cudaDeviceGetAttribute(&v.l2_bytes, cudaDevAttrL2CacheSize, dev) == cudaSuccess ? 0 : -3;
   });
   if (rc != 0) return rc;
+  const int n_sm = gpu.n_sm;
   const int per = a.N / a.n_seq;
   int sort_n = 1;
   while (sort_n < per) sort_n <<= 1;
   ScoreParams P{static_cast<const uint16_t*>(a.logits), a.V, per, a.cur_tok, a.d_in, a.d_out, a.eligible,
                 a.topk, sort_n, a.maxprob, a.entropy, a.argmax, a.score, a.topk_idx, a.topk_score, a.counters,
-                d == nullptr ? 0 : per > kBulkThreads ? kDecideApart : kDecideFused, d != nullptr ? *d : DecideArgs{}};
+                d == nullptr ? 0 : per > kBulkThreads ? kDecideApart : kDecideFused, d != nullptr ? *d : DecideArgs{},
+                2LL * a.N * a.V > gpu.l2_bytes};
   // top-k keys (at most 4096 x 8 bytes) reuse the ring; so does the decision step, which keeps a
   // float score per row behind them (4096 x 12 bytes, exactly the ring)
   static_assert((sizeof(uint64_t) + sizeof(float)) * kMaxPerSeq <= kRingStages * kChunkBytes, "keys fit the ring");
