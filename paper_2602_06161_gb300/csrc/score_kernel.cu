@@ -57,6 +57,7 @@ constexpr int kMaxPerSeq = 4096;            // rows per segment (the entry point
 constexpr int kRowLoads = 4;                // rows whose state a thread loads at once (general paths)
 constexpr int kRoundsMax = 32;              // selections up to this size by rounds or warp sorts (top_select)
 constexpr int kRoundsFew = 8;               // selections up to this size by per-warp rounds (top_rounds)
+constexpr int kFusedTopk = 2;               // longest list that the row kernel finds in segments longer than its CTAs
 constexpr int kMaxWarps = 32;               // the selection kernels run up to 1024 threads
 constexpr int kMaxThreads = 32 * kMaxWarps;
 constexpr int kRankWarps = 16;              // top_small ranks the published keys of up to this many warps
@@ -939,33 +940,41 @@ __device__ __forceinline__ int rank_below(const uint64_t* keys, int n, uint64_t 
 }
 
 
+// The 32 largest of the CTA's keys, descending, on the lanes of warp 0: the warps' sorted lists merged
+// pairwise (log2(warps) barriers). `sorted` is this lane's key of its warp's list; the merged list of the
+// last merge a warp took part in is returned. All threads of the CTA call it; cand holds blockDim.x keys.
+__device__ __forceinline__ uint64_t top_merged(uint64_t sorted, uint64_t* cand) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  cand[threadIdx.x] = sorted;
+  for (int n = blockDim.x >> 5; n > 1;) {
+    // the upper half's lists go into the lower half's
+    const int half = (n + 1) >> 1;
+    __syncthreads();
+    if (warp + half < n) {
+      uint64_t mine[1] = {sorted};
+      const uint64_t other[1] = {cand[(warp + half) * 32 + lane]};
+      warp_merge_desc<1>(mine, other, lane);
+      sorted = mine[0];
+      cand[threadIdx.x] = sorted;
+    }
+    n = half;
+  }
+  return sorted;
+}
+
 // The k largest (k <= 32) of the CTA's keys, one per thread (distinct, 0 = none). Each warp sorts
 // its keys and publishes its k largest in cand[warp * k ..]; a key can be among the CTA's k
 // largest only if it is among its warp's, and the number of larger published keys is its rank,
 // exact while below k (a warp publishes at most k). With many warps the
-// sorted lists are merged pairwise instead (log2(warps) barriers), since ranking against every
-// published key would cost warps * k reads a thread. Returns, for the key this lane then holds
+// sorted lists are merged instead, since ranking against every published key would cost warps * k
+// reads a thread. Returns, for the key this lane then holds
 // (*held), its slot 0 .. k-1 among the CTA's k largest, else -1. All threads of the CTA call it;
 // cand holds blockDim.x keys.
 __device__ __forceinline__ int top_small(uint64_t key, int k, uint64_t* cand, uint64_t* held) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   uint64_t sorted = warp_sort_desc(key, lane);
   if (nw > kRankWarps) {
-    cand[threadIdx.x] = sorted;
-    for (int n = nw; n > 1;) {
-      // the upper half's lists go into the lower half's
-      const int half = (n + 1) >> 1;
-      __syncthreads();
-      if (warp + half < n) {
-        uint64_t mine[1] = {sorted};
-        const uint64_t other[1] = {cand[(warp + half) * 32 + lane]};
-        warp_merge_desc<1>(mine, other, lane);
-        sorted = mine[0];
-        cand[threadIdx.x] = sorted;
-      }
-      n = half;
-    }
-    *held = sorted;
+    *held = sorted = top_merged(sorted, cand);
     return warp == 0 && lane < k && sorted != 0 ? lane : -1;
   }
   if (lane < k) cand[warp * k + lane] = sorted;
@@ -1206,36 +1215,37 @@ __device__ void segment_decide(uint64_t* keys, int seg, int per_seq, int sort_n,
   }
 }
 
-// The last CTA of a segment: top-k by (score desc, index asc) over eligible rows.
-__device__ __forceinline__ void segment_topk(uint64_t* keys, int seg, int per_seq, int sort_n, int topk,
-                                             const float* score, const uint8_t* eligible, int32_t* topk_idx,
-                                             float* topk_score) {
+// Top-k of a segment by (score desc, index asc) over its eligible rows, one row per thread: every
+// eligible row is ranked against the others (see decide_fast). All threads of the CTA call it.
+__device__ __forceinline__ void topk_rank(uint64_t* keys, int seg, int per_seq, int topk, const float* score,
+                                          const uint8_t* eligible, int32_t* topk_idx, float* topk_score) {
   const int tid = threadIdx.x, nt = blockDim.x;
   const int base = seg * per_seq;
-  if (per_seq <= nt) {
-    // one row per thread: rank every eligible row against the others (see decide_fast)
-    uint64_t key = 0;
-    float sc = 0.0f;
-    if (tid < per_seq) {
-      // both loads issued together: the score is read whether or not the row is eligible
-      sc = __ldcg(score + base + tid);
-      if (eligible == nullptr || eligible[base + tid] != 0) key = rank_key(sc, tid);
-    }
-    if (tid < per_seq) keys[tid] = key;
-    const int n_elig = __syncthreads_count(key != 0);
-    {
-      const int r = rank_below(keys, per_seq, key, topk);
-      if (key != 0 && r < topk) {
-        topk_idx[static_cast<size_t>(seg) * topk + r] = tid;
-        if (topk_score != nullptr) topk_score[static_cast<size_t>(seg) * topk + r] = sc;
-      }
-    }
-    for (int t = min(n_elig, topk) + tid; t < topk; t += nt) {
-      topk_idx[static_cast<size_t>(seg) * topk + t] = -1;
-      if (topk_score != nullptr) topk_score[static_cast<size_t>(seg) * topk + t] = -INFINITY;
-    }
-    return;
+  uint64_t key = 0;
+  float sc = 0.0f;
+  if (tid < per_seq) {
+    // both loads issued together: the score is read whether or not the row is eligible
+    sc = __ldcg(score + base + tid);
+    if (eligible == nullptr || eligible[base + tid] != 0) key = rank_key(sc, tid);
   }
+  if (tid < per_seq) keys[tid] = key;
+  const int n_elig = __syncthreads_count(key != 0);
+  const int r = rank_below(keys, per_seq, key, topk);
+  if (key != 0 && r < topk) {
+    topk_idx[static_cast<size_t>(seg) * topk + r] = tid;
+    if (topk_score != nullptr) topk_score[static_cast<size_t>(seg) * topk + r] = sc;
+  }
+  for (int t = min(n_elig, topk) + tid; t < topk; t += nt) {
+    topk_idx[static_cast<size_t>(seg) * topk + t] = -1;
+    if (topk_score != nullptr) topk_score[static_cast<size_t>(seg) * topk + t] = -INFINITY;
+  }
+}
+
+// The keys of a segment of any length in keys[0 .. sort_n).
+__device__ __forceinline__ void topk_keys(uint64_t* keys, int seg, int per_seq, int sort_n, const float* score,
+                                          const uint8_t* eligible) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int base = seg * per_seq;
   // the scores and flags of kLoads rows per thread are loaded before any key is stored, so the
   // loads of a thread overlap instead of waiting one after the other
   constexpr int kLoads = 4;
@@ -1256,24 +1266,25 @@ __device__ __forceinline__ void segment_topk(uint64_t* keys, int seg, int per_se
     }
   }
   __syncthreads();
-  // a short list by warp sorts and merges, a long one by sorting
-  __shared__ uint64_t s_sel[kRoundsMax];
-  const uint64_t* best = keys;
-  if (topk <= kRoundsMax) {
-    top_select(keys, sort_n, topk, s_sel);
-    best = s_sel;
-  } else {
-    bitonic_sort_desc(keys, sort_n);
+}
+
+// Slot `slot` of the lists: the row and score of a key, none for key 0.
+__device__ __forceinline__ void topk_put(uint64_t key, size_t slot, int32_t* topk_idx, float* topk_score) {
+  topk_idx[slot] = key != 0 ? rank_key_row(key) : -1;
+  if (topk_score != nullptr) topk_score[slot] = key != 0 ? order_key_inv(static_cast<uint32_t>(key >> 32)) : -INFINITY;
+}
+
+// The last CTA of a segment in the row kernel: ranks where every row has a thread, else a list of one or two.
+__device__ __forceinline__ void segment_topk(uint64_t* keys, int seg, const ScoreParams& P) {
+  if (P.per_seq <= static_cast<int>(blockDim.x)) {
+    topk_rank(keys, seg, P.per_seq, P.topk, P.score, P.eligible, P.topk_idx, P.topk_score);
+    return;
   }
-  for (int t = tid; t < topk; t += nt) {
-    const uint64_t key = best[t];
-    const bool valid = key != 0;
-    topk_idx[static_cast<size_t>(seg) * topk + t] =
-        valid ? static_cast<int32_t>(0xffffffffu - static_cast<uint32_t>(key)) : -1;
-    if (topk_score != nullptr)
-      topk_score[static_cast<size_t>(seg) * topk + t] =
-          valid ? order_key_inv(static_cast<uint32_t>(key >> 32)) : -INFINITY;
-  }
+  __shared__ uint64_t s_few[kFusedTopk];
+  topk_keys(keys, seg, P.per_seq, P.sort_n, P.score, P.eligible);
+  top_rounds(keys, P.sort_n, P.topk, s_few);
+  if (static_cast<int>(threadIdx.x) < P.topk)
+    topk_put(s_few[threadIdx.x], static_cast<size_t>(seg) * P.topk + threadIdx.x, P.topk_idx, P.topk_score);
 }
 
 // Accumulate U vectors of 8 values; the first index of vector u is i0 + u * istride, istride
@@ -1500,8 +1511,7 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
     if (P.decide)
       segment_decide(reinterpret_cast<uint64_t*>(ring), n / P.per_seq, P.per_seq, P.sort_n, P);
     else
-      segment_topk(reinterpret_cast<uint64_t*>(ring), n / P.per_seq, P.per_seq, P.sort_n, P.topk, P.score,
-                   P.eligible, P.topk_idx, P.topk_score);
+      segment_topk(reinterpret_cast<uint64_t*>(ring), n / P.per_seq, P);
   }
 }
 
@@ -1516,6 +1526,56 @@ __global__ void __launch_bounds__(kMaxThreads) decide_kernel(const ScoreParams P
   griddep_wait();
   griddep_launch_dependents();
   segment_decide(dec_keys, blockIdx.x, P.per_seq, P.sort_n, P);
+}
+
+// The top-k of such segments, likewise (for lists of more than kFusedTopk: one or two rows are found in
+// the row kernel's last CTA before this launch would start). How, by the rows and the list, with the us
+// that the launch adds behind rows of 1001 logits:
+//   rows           list       merged lists   ranks   rounds / warp sorts, 288 / 512 / 1024 threads   sort, 512 / 1024
+//   289            <= 32      2.6            3.9     k = 8: 4.2 / 4.1; k = 32: 6.1 / 6.9             9.4 / 10.2
+//   289, 400, 512  33 .. 200                 3.9, 5.4, 6.3                                           9.4, 9.6, 9.5 / 10.2, 9.8, 10.5
+//   640, 768, 1024 33 .. 200                 9.3, 13.0, 21.7                                         17.3, 17.5, 17.8 / 14.1, 14.3, 14.4
+//   1024           <= 32      3.6            21.7    k = 8: 4.9 / 4.9 / 6.1; k = 32: 6.1 / 8.4 / 16.1
+//   2048           <= 32                             k = 8: 6.0 / 5.5 / 6.7; k = 32: 8.6 / 8.1 / 16.2
+//   4096           <= 32                             k = 8: 8.4 / 7.3 / 8.4; k = 32: 14.2 / 12.0 / 16.5
+// In the row kernel's last CTA of 288 threads, lists of more than 32 rows were sorted: 1 x 512 rows of 20001
+// logits, k = 64: 20.7 us; a row kernel of 512 threads ranked them: 16.4; now 13.3 (1024 rows: 39.3, 35.2, 25.3).
+constexpr int kRankRows = 768;        // segments up to this size are ranked, for lists of more than kRoundsMax
+constexpr int kTopkWarpThreads = 512; // threads for a short list of more rows than a CTA can have threads
+int topk_threads(int per, int topk) {
+  const bool list = topk <= kRoundsMax;
+  if (per > kMaxThreads) return list ? kTopkWarpThreads : kMaxThreads;
+  return list || per <= kRankRows ? (per + 31) / 32 * 32 : kMaxThreads;
+}
+__global__ void __launch_bounds__(kMaxThreads) topk_kernel(const ScoreParams P) {
+  extern __shared__ __align__(16) uint64_t topk_smem[];
+  __shared__ uint64_t s_sel[kRoundsMax];
+  griddep_wait();
+  griddep_launch_dependents();
+  const int tid = threadIdx.x, nt = blockDim.x, seg = blockIdx.x;
+  const size_t list = static_cast<size_t>(seg) * P.topk;
+  if (P.per_seq <= nt && P.topk <= kRoundsMax) {
+    uint64_t key = 0;
+    if (tid < P.per_seq) {
+      const int n = seg * P.per_seq + tid;
+      const float sc = P.score[n];
+      if (P.eligible == nullptr || P.eligible[n] != 0) key = rank_key(sc, tid);
+    }
+    const uint64_t held = top_merged(warp_sort_desc(key, tid & 31), topk_smem);
+    if (tid < P.topk) topk_put(held, list + tid, P.topk_idx, P.topk_score);
+  } else if (P.per_seq <= nt && P.per_seq <= kRankRows) {
+    topk_rank(topk_smem, seg, P.per_seq, P.topk, P.score, P.eligible, P.topk_idx, P.topk_score);
+  } else {
+    const uint64_t* best = topk_smem;
+    topk_keys(topk_smem, seg, P.per_seq, P.sort_n, P.score, P.eligible);
+    if (P.topk <= kRoundsMax) {
+      top_select(topk_smem, P.sort_n, P.topk, s_sel);
+      best = s_sel;
+    } else {
+      bitonic_sort_desc(topk_smem, P.sort_n);
+    }
+    for (int t = tid; t < P.topk; t += nt) topk_put(best[t], list + t, P.topk_idx, P.topk_score);
+  }
 }
 
 // Section 5.3 selection as its own launch (one CTA per segment), after the
@@ -1622,16 +1682,19 @@ int launch_score_impl(const ScoreArgs& a, const DecideArgs* d, int* status, cuda
   // float score per row behind them (4096 x 12 bytes, exactly the ring)
   static_assert((sizeof(uint64_t) + sizeof(float)) * kMaxPerSeq <= kRingStages * kChunkBytes, "keys fit the ring");
   const size_t smem = static_cast<size_t>(kRingStages) * kChunkBytes;
+  const bool long_topk = d == nullptr && a.topk > kFusedTopk && per > kBulkThreads;
+  ScoreParams rows = P;
+  if (long_topk) rows.topk = 0;
   int rl = 0;
   switch (row_split(a.N, a.V, n_sm)) {
-    case 8: rl = launch_rows<8>(P, a.N, smem, status, stream); break;
-    case 4: rl = launch_rows<4>(P, a.N, smem, status, stream); break;
-    case 2: rl = launch_rows<2>(P, a.N, smem, status, stream); break;
-    default: rl = launch_rows<1>(P, a.N, smem, status, stream);
+    case 8: rl = launch_rows<8>(rows, a.N, smem, status, stream); break;
+    case 4: rl = launch_rows<4>(rows, a.N, smem, status, stream); break;
+    case 2: rl = launch_rows<2>(rows, a.N, smem, status, stream); break;
+    default: rl = launch_rows<1>(rows, a.N, smem, status, stream);
   }
-  if (rl != 0 || P.decide != kDecideApart) return rl;
-  const int threads = std::min((per + 31) / 32 * 32, kMaxThreads);
-  const size_t keys = (sizeof(uint64_t) + sizeof(float)) * static_cast<size_t>(std::max(sort_n, threads));
+  if (rl != 0 || (!long_topk && P.decide != kDecideApart)) return rl;
+  const int threads = long_topk ? topk_threads(per, a.topk) : std::min((per + 31) / 32 * 32, kMaxThreads);
+  const size_t keys = (sizeof(uint64_t) + (long_topk ? 0 : sizeof(float))) * static_cast<size_t>(std::max(sort_n, threads));
   static ContextCache<int> setup;
   int unused = 0;
   const int rc2 = setup.get(&unused, [](int&) {
@@ -1642,7 +1705,7 @@ int launch_score_impl(const ScoreArgs& a, const DecideArgs* d, int* status, cuda
   if (rc2 != 0) return rc2;
   cudaLaunchAttribute attr[1];
   const cudaLaunchConfig_t cfg = pdl_config(dim3(static_cast<unsigned>(a.n_seq)), dim3(threads), keys, stream, attr);
-  return cudaLaunchKernelEx(&cfg, decide_kernel, P) == cudaSuccess ? 0 : -3;
+  return cudaLaunchKernelEx(&cfg, long_topk ? topk_kernel : decide_kernel, P) == cudaSuccess ? 0 : -3;
 }
 
 }  // namespace

@@ -159,6 +159,21 @@ def test_score_topk_fewer_eligible_than_k(per, k, frac):
         assert (r["topk_idx"][g, n_elig[g]:] == -1).all() and (r["topk_idx"][g, :n_elig[g]] >= 0).all()
 
 
+@pytest.mark.parametrize("per,k", [
+    (289, 2), (1025, 2),                            # found in the row kernel
+    (289, 3), (512, 32), (513, 32), (1024, 32),     # the lists of 10 to 32 warps, merged
+    (289, 33), (300, 300), (768, 33), (768, 700),   # ranks
+    (769, 33), (1024, 1024), (1025, 33),            # sorts
+    (1025, 3), (1025, 32), (4096, 9),               # rounds, warp sorts on 512 threads
+])
+@pytest.mark.parametrize("frac", [1.0, 0.6, 0.005])
+def test_score_topk_of_long_segments(per, k, frac):
+    """Segments longer than the row kernel's CTAs: lists in a launch of their own, also with fewer eligible rows."""
+    inp = W.make_score_inputs(2 * per, 203, 2, k, seed=per + k, eligible_frac=frac)
+    inp.logits[5] = inp.logits[7] = inp.logits[per + 3] = inp.logits[2]   # equal scores: the lower row first
+    check(inp, run_score(inp, workspace=api.score_workspace(2)), f"per {per} k {k}")
+
+
 def test_score_no_eligible_rows():
     inp = W.make_score_inputs(32, 512, 2, 4, seed=8, eligible_frac=0.0)
     r = run_score(inp)
