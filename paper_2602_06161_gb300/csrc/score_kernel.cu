@@ -970,10 +970,12 @@ __device__ __forceinline__ uint64_t top_merged(uint64_t sorted, uint64_t* cand) 
 // reads a thread. Returns, for the key this lane then holds
 // (*held), its slot 0 .. k-1 among the CTA's k largest, else -1. All threads of the CTA call it;
 // cand holds blockDim.x keys.
+// kMerge: the CTA may have more than kRankWarps warps.
+template <bool kMerge>
 __device__ __forceinline__ int top_small(uint64_t key, int k, uint64_t* cand, uint64_t* held) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   uint64_t sorted = warp_sort_desc(key, lane);
-  if (nw > kRankWarps) {
+  if (kMerge && nw > kRankWarps) {
     *held = sorted = top_merged(sorted, cand);
     return warp == 0 && lane < k && sorted != 0 ? lane : -1;
   }
@@ -993,6 +995,7 @@ __device__ __forceinline__ int top_small(uint64_t key, int k, uint64_t* cand, ui
 // general path): seed score, n_t and the mean, n_t pi_t = #{n_t s_j > sum s}, and
 // the selection of ceil(sqrt(n_t pi_t)) rows by rank. Writes score, flags and the
 // segment's seed list, count and stats[4..5].
+template <bool kMerge>
 __device__ void select_fast(uint64_t* keys, int seg, int per_seq, const DecideArgs& d, bool in, int tok,
                             uint32_t& fl, uint32_t rc, float u, float din, float dout, float* score) {
   __shared__ long long s_fx[32];
@@ -1051,7 +1054,7 @@ __device__ void select_fast(uint64_t* keys, int seg, int per_seq, const DecideAr
     // key writes its slot and marks the row for its owner thread
     uint64_t held;
     if (in) s_mark[tid] = 0;
-    const int slot = top_small(key, k, keys, &held);
+    const int slot = top_small<kMerge>(key, k, keys, &held);
     if (slot >= 0) {
       const int row = rank_key_row(held);
       d.seed_idx[static_cast<size_t>(seg) * d.max_seeds + slot] = d.pos0 + row;
@@ -1083,6 +1086,7 @@ __device__ void select_fast(uint64_t* keys, int seg, int per_seq, const DecideAr
 
 // One segment's decision step, one row per thread (see segment_update and
 // segment_select for the general path).
+template <bool kMerge>
 __device__ void decide_fast(uint64_t* keys, int seg, int per_seq, const ScoreParams& P) {
   __shared__ unsigned long long s_fallback;
   __shared__ int s_cnt[3];
@@ -1141,7 +1145,7 @@ __device__ void decide_fast(uint64_t* keys, int seg, int per_seq, const ScorePar
     if (d.budget <= 32) {
       if (in) s_draft[tid] = 0;
       uint64_t held;
-      const int slot = top_small(ck, d.budget, keys, &held);
+      const int slot = top_small<kMerge>(ck, d.budget, keys, &held);
       if (slot >= 0) s_draft[rank_key_row(held)] = 1;
       __syncthreads();
       drafted = in && s_draft[tid] != 0;
@@ -1184,7 +1188,7 @@ __device__ void decide_fast(uint64_t* keys, int seg, int per_seq, const ScorePar
     if (br) atomicAdd(&s_cnt[1], __popc(br));
     if (bm) atomicAdd(&s_cnt[2], __popc(bm));
   }
-  if (select) select_fast(keys, seg, per_seq, d, in, tok, fl, rc, u, din, dout, P.score);
+  if (select) select_fast<kMerge>(keys, seg, per_seq, d, in, tok, fl, rc, u, din, dout, P.score);
   else __syncthreads();
   if (in) {
     d.tok[n] = tok;
@@ -1201,11 +1205,11 @@ __device__ void decide_fast(uint64_t* keys, int seg, int per_seq, const ScorePar
   }
 }
 
-// The last CTA of a segment in decision mode: the update, then (unless only the
-// update was asked for) the selection with the caller's d_in / d_out.
+// A segment of any length: the update, then (unless only the update was asked
+// for) the selection with the caller's d_in / d_out.
 __device__ void segment_decide(uint64_t* keys, int seg, int per_seq, int sort_n, const ScoreParams& P) {
   if (per_seq <= static_cast<int>(blockDim.x)) {
-    decide_fast(keys, seg, per_seq, P);
+    decide_fast<true>(keys, seg, per_seq, P);
     return;
   }
   segment_update(keys, seg, per_seq, sort_n, P);
@@ -1509,7 +1513,7 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
   __syncthreads();
   if (s_last) {
     if (P.decide)
-      segment_decide(reinterpret_cast<uint64_t*>(ring), n / P.per_seq, P.per_seq, P.sort_n, P);
+      decide_fast<false>(reinterpret_cast<uint64_t*>(ring), n / P.per_seq, P.per_seq, P);
     else
       segment_topk(reinterpret_cast<uint64_t*>(ring), n / P.per_seq, P);
   }
@@ -1607,7 +1611,7 @@ __global__ void __launch_bounds__(kSelectThreads) seed_select_kernel(const Decid
       din = d_in != nullptr ? d_in[n] : 0.0f;
       dout = d_out != nullptr ? d_out[n] : 0.0f;
     }
-    select_fast(sel_keys, blockIdx.x, per_seq, d, in, tok, fl, rc, u, din, dout, score);
+    select_fast<false>(sel_keys, blockIdx.x, per_seq, d, in, tok, fl, rc, u, din, dout, score);
     if (in) d.flags[n] = static_cast<uint8_t>(fl);
     return;
   }
