@@ -398,7 +398,7 @@ struct ScoreParams {
   uint32_t* counters;
   int decide;          // kDecideFused: the last CTA of a segment decides; kDecideApart: decide_kernel does
   DecideArgs dec;
-  bool evict_first;    // the logits do not fit in L2
+  bool evict_first;    // see stream_policy
 };
 
 // Descending bitonic sort of n (a power of two) 64-bit keys in shared memory;
@@ -1334,12 +1334,12 @@ __device__ __forceinline__ void acc_batch(RowAcc& a, const uint4 (&w)[U], int i0
 // ---------------------------------------------------------------------------
 // row kernel: bulk copies of a row, or of a row's slice in each CTA of a cluster
 // ---------------------------------------------------------------------------
-// L2 policy of the copies. Logits larger than L2 are gone before they could be read again: evicted
-// first, they leave the rest of a step there (states, weights, the next kernels' code). The pass itself
-// takes the same time; in a decoding step of Dream's shape (311 MB of logits) the launches around it
-// went from 98.9 to 87.2 us. Smaller ones stay where they are, for whoever reads them next: evicted first,
-// a second pass over 1024 rows of 32000 logits took 16.8 instead of 13.9 us, over 1024 of 50000 22.3 instead
-// of 20.2, over 300 of 126464 15.8 instead of 14.2.
+// L2 policy of the copies: evicted first where the logits are not read again, which leaves the rest of a
+// step there (states, weights, the next kernels' code). That is a decision step's, whose launches went from
+// 98.9 to 87.2 us in Dream's shape (311 MB of logits) and from 39.5 to 33.8 with 28 / 4 heads, 243 rows (74
+// MB), and plain scoring of more than L2 holds. Other plain scoring leaves the logits there: evicted first,
+// a second call on 1024 rows of 32000 logits took 16.9 instead of 13.9 us, of 50000 22.3 instead of 20.2, and
+// calls on three 21 MB sets in turn 10.1 instead of 8.9. The pass itself takes the same time either way.
 __device__ __forceinline__ uint64_t stream_policy(bool evict_first) {
   uint64_t p;
   if (evict_first)
@@ -1681,7 +1681,7 @@ int launch_score_impl(const ScoreArgs& a, const DecideArgs* d, int* status, cuda
   ScoreParams P{static_cast<const uint16_t*>(a.logits), a.V, per, a.cur_tok, a.d_in, a.d_out, a.eligible,
                 a.topk, sort_n, a.maxprob, a.entropy, a.argmax, a.score, a.topk_idx, a.topk_score, a.counters,
                 d == nullptr ? 0 : per > kBulkThreads ? kDecideApart : kDecideFused, d != nullptr ? *d : DecideArgs{},
-                2LL * a.N * a.V > gpu.l2_bytes};
+                d != nullptr || 2LL * a.N * a.V > gpu.l2_bytes};
   // top-k keys (at most 4096 x 8 bytes) reuse the ring; so does the decision step, which keeps a
   // float score per row behind them (4096 x 12 bytes, exactly the ring)
   static_assert((sizeof(uint64_t) + sizeof(float)) * kMaxPerSeq <= kRingStages * kChunkBytes, "keys fit the ring");
