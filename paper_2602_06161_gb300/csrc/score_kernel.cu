@@ -30,9 +30,10 @@
 // 16-byte vectors into a 3-stage shared-memory ring (mbarrier full / empty), 8 consumer warps
 // reduce from shared memory; bytes in flight do not cost registers, and 4 CTAs share an SM. The
 // up to 14 elements outside the aligned vectors (V or the row's offset not a multiple of 8) are
-// read by the producer warp's other lanes, so every V takes this path: a kernel of 16-byte register
-// loads for such rows took 57.9 us on 1024 rows of V = 126465 against 50.1 us. With few
-// rows each is split over the CTAs of a cluster (row_split), whose slice sums its first CTA adds.
+// read by the producer warp's other lanes. With few rows each is split over the CTAs of a cluster
+// (row_split), whose slice sums its first CTA adds. Unaligned rows of which an SM has one or two go
+// through a kernel of 16-byte register loads where that is ahead (loads_to_registers); with more
+// rows it falls behind: 1024 rows of V = 126465 57.9 against 50.1 us.
 #include <math.h>
 #include <stdint.h>
 
@@ -51,6 +52,8 @@ constexpr int kBulkThreads = (kConsumerWarps + 1) * 32;
 constexpr int kChunkElems = 8192;          // 16 KB of bf16 per bulk copy
 constexpr int kChunkBytes = kChunkElems * 2;
 constexpr int kRingStages = 3;
+constexpr int kRegThreads = 512;           // register-load kernel
+constexpr int kRegUnroll = 4;
 constexpr int kVecPerThread = kChunkElems / 8 / (kConsumerWarps * 32);   // 4
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kMaxPerSeq = 4096;            // rows per segment (the entry points refuse more)
@@ -104,6 +107,14 @@ __device__ __forceinline__ void raise_max(RowAcc& a, float new_m, int new_i, int
   a.mi = new_i;
   a.mu = new_u;
   a.mref = new_ref;
+}
+
+__device__ __forceinline__ uint4 ld_stream(const uint4* p) {
+  uint4 r;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+               : "l"(p));
+  return r;
 }
 
 __device__ __forceinline__ float bf16_to_f32(uint16_t h) { return __uint_as_float(static_cast<uint32_t>(h) << 16); }
@@ -164,7 +175,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // by the threads that hold their warp's maximum before the block-wide maximum is known, so their
 // latency overlaps the reduction.
 constexpr int kMaxBatch = 4;
-static_assert(kVecPerThread <= kMaxBatch, "batches hold at most four vectors");
+static_assert(kVecPerThread <= kMaxBatch && kRegUnroll <= kMaxBatch, "batches hold at most four vectors");
 
 // Where the row kernel's ring holds a row (slice) after its last chunk: element `first` of the row
 // began chunk 0, and chunks from `held` on are there.
@@ -1519,6 +1530,65 @@ __global__ void __launch_bounds__(kBulkThreads, 4) score_bulk_kernel(const Score
   }
 }
 
+// Rows that do not start on 16-byte boundaries (V % 8 != 0), a few of them per SM: a CTA's 16 warps load
+// the row's aligned vectors into registers, and the elements before and after them.
+__global__ void __launch_bounds__(kRegThreads, 2) score_reg_kernel(const ScoreParams P) {
+  extern __shared__ __align__(16) uint64_t reg_keys[];
+  constexpr int kWarps = kRegThreads / 32;
+  __shared__ float red_m[kWarps];
+  __shared__ int red_i[kWarps];
+  __shared__ float2 red_z[kWarps], red_s[kWarps];
+  __shared__ int s_last;
+  griddep_wait();
+  griddep_launch_dependents();
+
+  const int n = blockIdx.x, tid = threadIdx.x, V = P.V;
+  const size_t row_off = static_cast<size_t>(n) * V;
+  const uint16_t* row = P.logits + row_off;
+  // the row's side data, on its way while the row streams; the token's logit once the row is read
+  RowSide side{true, 0.0f, 0.0f, 0.0f};
+  int y = 0;
+  if (tid == 0) {
+    const int32_t* tok = P.decide ? P.dec.tok : P.cur_tok;
+    side.greedy = tok == nullptr;
+    if (tok != nullptr) y = tok[n];
+    if (!P.decide && P.d_in != nullptr) side.din = P.d_in[n];
+    if (!P.decide && P.d_out != nullptr) side.dout = P.d_out[n];
+  }
+  RowAcc a{-INFINITY, 0x7fffffff, 0, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  const int head = min(static_cast<int>((8 - (row_off & 7)) & 7), V);
+  const int nvec = (V - head) / 8, tail0 = head + nvec * 8;
+  if (tid < head) acc_scalar(a, bf16_to_f32(row[tid]), tid);
+  const uint4* vrow = reinterpret_cast<const uint4*>(row + head);
+  int v = tid;
+  for (; v + (kRegUnroll - 1) * kRegThreads < nvec; v += kRegUnroll * kRegThreads) {
+    uint4 w[kRegUnroll];
+#pragma unroll
+    for (int u = 0; u < kRegUnroll; ++u) w[u] = ld_stream(vrow + v + u * kRegThreads);
+    acc_batch<kRegUnroll>(a, w, head + v * 8);
+  }
+  for (; v < nvec; v += kRegThreads) {
+    uint4 w[1] = {ld_stream(vrow + v)};
+    acc_batch<1>(a, w, head + v * 8);
+  }
+  if (tail0 + tid < V) acc_scalar(a, bf16_to_f32(row[tail0 + tid]), tail0 + tid);
+  if (tid == 0) side_logit(side, y, row, V);
+
+  const Ring none{nullptr, 0, 0x7fffffff};
+  const RowSum r = row_reduce<kWarps, kRegThreads * 8>(a, row, none, red_m, red_i, red_z, red_s);
+  if (tid == 0)
+    s_last = row_write(row_finish(r), side, n, P.per_seq, P.topk, P.maxprob, P.entropy, P.argmax, P.score,
+                       P.decide == kDecideApart ? nullptr : P.counters, P.decide ? P.dec.ws_u : nullptr,
+                       P.decide ? P.dec.ws_lnz : nullptr);
+  __syncthreads();
+  if (s_last) {
+    if (P.decide)
+      decide_fast<false>(reg_keys, n / P.per_seq, P.per_seq, P);
+    else
+      topk_rank(reg_keys, n / P.per_seq, P.per_seq, P.topk, P.score, P.eligible, P.topk_idx, P.topk_score);
+  }
+}
+
 // One step's decisions as their own launch (one CTA per segment) behind the row kernel, for segments
 // of more rows than that kernel's CTAs have threads: up to 1024 rows then have a thread each, where
 // the last CTA of a segment made five passes over its rows. Segments of up to kBulkThreads rows
@@ -1661,6 +1731,21 @@ int row_split(int N, int V, int n_sm) {
   return c;
 }
 
+// Whether unaligned rows go through the register-load kernel: with one or two unsplit rows per SM its 16
+// warps are ahead of the ring's 8, if a row is little more than whole batches of its CTA (16384 elements; the
+// rest goes a vector at a time) or long. us through the ring / registers:
+//   rows   V = 20001    26001        30001        36355        50257        80001          108602         152065
+//   77     4.3 / 3.9    4.7 / 4.5    4.9 / 5.1    5.4 / 4.6    6.6 / 6.3    (split)
+//   152    4.5 / 4.3    5.4 / 6.0    6.0 / 7.3    6.6 / 6.0    7.5 / 7.1    (split)
+//   153    5.0 / 5.2    5.8 / 6.5    6.6 / 7.8    7.3 / 6.7    8.6 / 7.8    11.1 / 10.9    13.3 / 12.7    16.8 / 15.6
+//   250    6.3 / 6.0    7.0 / 7.3    7.5 / 8.4    8.0 / 7.2    9.2 / 8.7    11.8 / 11.9    14.1 / 13.7    17.8 / 16.9
+//   320    8.2 / 8.9    9.2 / 11.2   10.0 / 13.0  10.9 / 10.8  12.8 / 12.9  17.4 / 18.3    21.4 / 21.8    27.8 / 27.0
+// and 4.0 / 4.1 at 153 rows of 8001, 4.4 / 4.9 of 16385.
+bool loads_to_registers(int N, int V, int split, int n_sm) {
+  constexpr int kBatch = kRegThreads * kRegUnroll * 8;
+  return V % 8 != 0 && split == 1 && N <= 2 * n_sm && V >= kBatch / 8 * 9 && (V % kBatch <= kBatch / 4 || V >= 6 * kBatch);
+}
+
 int launch_score_impl(const ScoreArgs& a, const DecideArgs* d, int* status, cudaStream_t stream) {
   struct Device {
     int n_sm, l2_bytes;
@@ -1690,11 +1775,19 @@ int launch_score_impl(const ScoreArgs& a, const DecideArgs* d, int* status, cuda
   ScoreParams rows = P;
   if (long_topk) rows.topk = 0;
   int rl = 0;
-  switch (row_split(a.N, a.V, n_sm)) {
-    case 8: rl = launch_rows<8>(rows, a.N, smem, status, stream); break;
-    case 4: rl = launch_rows<4>(rows, a.N, smem, status, stream); break;
-    case 2: rl = launch_rows<2>(rows, a.N, smem, status, stream); break;
-    default: rl = launch_rows<1>(rows, a.N, smem, status, stream);
+  const int split = row_split(a.N, a.V, n_sm);
+  if (loads_to_registers(a.N, a.V, split, n_sm)) {
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg =
+        pdl_config(dim3(static_cast<unsigned>(a.N)), dim3(kRegThreads), sizeof(uint64_t) * kRegThreads, stream, attr);
+    rl = cudaLaunchKernelEx(&cfg, score_reg_kernel, rows) == cudaSuccess ? 0 : -3;
+  } else {
+    switch (split) {
+      case 8: rl = launch_rows<8>(rows, a.N, smem, status, stream); break;
+      case 4: rl = launch_rows<4>(rows, a.N, smem, status, stream); break;
+      case 2: rl = launch_rows<2>(rows, a.N, smem, status, stream); break;
+      default: rl = launch_rows<1>(rows, a.N, smem, status, stream);
+    }
   }
   if (rl != 0 || (!long_topk && P.decide != kDecideApart)) return rl;
   const int threads = long_topk ? topk_threads(per, a.topk) : std::min((per + 31) / 32 * 32, kMaxThreads);

@@ -61,6 +61,8 @@ def test_score_shapes(N, V, n_seq, k):
     (39, 20001), (76, 8193),      # four
     (77, 65544), (152, 65537),    # two
     (153, 65544),                 # one
+    (100, 20001), (153, 36355), (304, 18435), (160, 98305),   # loaded to registers
+    (305, 20001), (100, 20481), (100, 18427),                 # and on the other side of that rule
 ])
 def test_score_split_rows(N, V):
     """Rows split over a cluster: sums and, with the maximum in several slices, its first index."""
@@ -77,7 +79,7 @@ def test_score_side_inputs_and_eligibility():
     check(inp, run_score(inp))
 
 
-@pytest.mark.parametrize("N,V", [(6, 20001), (400, 5000)])   # rows split over a cluster, and not
+@pytest.mark.parametrize("N,V", [(6, 20001), (400, 5000), (100, 20001)])   # rows split or not, to registers
 def test_score_token_outside_the_vocabulary(N, V):
     """Every value outside [0, V) has no probability, the largest and smallest of the type too: u and score are NaN."""
     x = H.to_dev(W.make_score_inputs(N, V, 1, 1, seed=V).logits, "bf16")
@@ -97,7 +99,7 @@ def test_score_token_outside_the_vocabulary(N, V):
     assert api.cover_device_status() == 0
 
 
-@pytest.mark.parametrize("N,V", [(6, 20001), (400, 5000)])   # rows split over a cluster, and not
+@pytest.mark.parametrize("N,V", [(6, 20001), (400, 5000), (100, 20001)])   # rows split or not, to registers
 def test_score_rows_without_a_greedy_token(N, V):
     """A row of -inf has no greedy token: its score is NaN, not -inf, beside rows that it leaves as they are."""
     x = H.to_dev(W.make_score_inputs(N, V, 1, 1, seed=V).logits, "bf16")
@@ -113,7 +115,7 @@ LOWEST = float(torch.finfo(torch.bfloat16).min)
 
 
 @pytest.mark.parametrize("low", [LOWEST, -1e38, -1e35, -1e30, -1e10, -1e9])
-@pytest.mark.parametrize("N,V", [(4, 20001), (4, 126464), (400, 20001), (400, 5000)])   # split rows and not
+@pytest.mark.parametrize("N,V", [(4, 20001), (4, 126464), (400, 20001), (400, 5000), (100, 20001)])   # split or not, to registers
 def test_score_masked_logits(N, V, low):
     """Masked logits: in the elements past the aligned vectors, in whole batches of a lane, in whole slices of
     a row, at its start and between. They have no weight. (t 2^t of the lowest value is -inf times 0: no entropy.)"""
@@ -132,7 +134,7 @@ def test_score_masked_logits(N, V, low):
     assert api.cover_device_status() == 0
 
 
-@pytest.mark.parametrize("N,V", [(4, 20001), (4, 126464), (400, 20001), (400, 5000)])   # split rows and not
+@pytest.mark.parametrize("N,V", [(4, 20001), (4, 126464), (400, 20001), (400, 5000), (100, 20001)])   # split or not, to registers
 def test_score_nan_logits_show(N, V):
     """One NaN logit anywhere, or a slice of them, leaves its row NaN and the other rows as they are."""
     x = H.to_dev(W.make_score_inputs(N, V, 1, 1, seed=V).logits, "bf16")
