@@ -147,10 +147,16 @@ def test_f32_seed_rows_do_not_read_their_own_cached_row(Hq, L, D, bad):
     assert not out[:, :, :at, ::3].isfinite().any() and api.cover_device_status() == 0
 
 
+@pytest.mark.parametrize("Hq,L,D", [
+    (2, 70, 64), (2, 300, 128),                   # keys split over a cluster
+    (1, 64, 64), (2, 16, 128),                    # unsplit, 16 rows a CTA
+    (50, 90, 64), (50, 96, 128),                  # 32
+    (38, 130, 64), (76, 127, 128),                # 64
+])
 @pytest.mark.parametrize("which", range(4))
-def test_f32_unaligned_rows_equal_aligned(which):
+def test_f32_unaligned_rows_equal_aligned(which, Hq, L, D):
     """A tensor that is only 4-byte aligned takes the 4-byte copies: the same bits."""
-    inp = W.make_attn_inputs(1, 2, 1, 70, 64, 5, dtype="f32", seed=4)
+    inp = W.make_attn_inputs(1, Hq, max(1, Hq // 2), L, D, 5, dtype="f32", seed=4)
     t = [H.to_dev(x, "f32") for x in (inp.q, inp.k_cached, inp.v_cached, inp.k_seedmask, inp.v_seedmask)]
     seeds = H.to_dev(inp.seed_idx, "i32")
     out = torch.empty_like(t[0])

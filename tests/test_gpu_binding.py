@@ -29,14 +29,15 @@ def _calls():
         calls["prefix" + name] = lambda fn=fw, a=(qw, k, v, km, vm, sd), **kw: fn(*a, q0=20, **kw)
     x = _r(12, 1003, seed=5)
     tok = torch.randint(0, 1003, (12,), device="cuda", dtype=torch.int32)
-    d = torch.rand(12, device="cuda")
+    d, e = torch.rand(12, device="cuda"), torch.rand(12, device="cuda") + 1
     ok = (torch.rand(12, device="cuda") < 0.6).to(torch.uint8)
     calls["score"] = lambda **kw: api.cover_score_fwd(x, 2, 3, workspace=api.score_workspace(2), **kw)
-    calls["score_side"] = lambda **kw: api.cover_score_fwd(x, 2, 3, cur_tok=tok, d_in=d, d_out=d, eligible=ok, **kw)
+    calls["score_side"] = lambda **kw: api.cover_score_fwd(x, 2, 3, cur_tok=tok, d_in=d, d_out=e, eligible=ok,
+                                                           workspace=api.score_workspace(2), **kw)
     calls["score_k0"] = lambda **kw: api.cover_score_fwd(x, 2, 0, **kw)
     calls["decide"] = lambda **kw: api.cover_score_decide_fwd(
         x, 2, tok.clone(), ok.clone(), ok.clone(), tau_draft=0.01, draft_budget=2, remask_budget=3, mask_id=1000, pos0=5,
-        max_seeds=4, d_in=d, d_out=d, workspace=api.decide_workspace(12, 2), **kw)
+        max_seeds=4, d_in=d, d_out=e, draft_ok=1 - ok, workspace=api.decide_workspace(12, 2), **kw)
     q, k, sd = _r(2, 4, 70, 128, seed=4), _r(2, 2, 70, 128), _seeds(2, 3, 70)
     lse, km = _r(2, 4, 70, dtype=torch.float32, seed=6) + 5, _r(2, 2, 3, 128, seed=2)
     t2, f2 = torch.randint(0, 9, (80,), device="cuda", dtype=torch.int32), torch.full((80,), 2, device="cuda", dtype=torch.uint8)
@@ -60,11 +61,30 @@ def _flat(r):
     return [x for _, x in sorted(r.items())] if isinstance(r, dict) else list(r)
 
 
+class _Counting:
+    """The native marshalling, counting the calls that it took."""
+
+    def __init__(self, native):
+        self.native, self.took = native, 0
+
+    def __getattr__(self, name):
+        def call(*args):
+            r = getattr(self.native, name)(*args)
+            self.took += r is not None
+            return r
+        return call
+
+
 @pytest.mark.parametrize("name", NAMES)
-def test_native_call_equals_the_python_path(name):
+def test_native_call_equals_the_python_path(name, monkeypatch):
     torch.manual_seed(0)
     call = _calls()[name]
-    a, b = call(), call(stream=torch.cuda.current_stream())
+    counting = _Counting(api._native())
+    monkeypatch.setattr(api, "_nat", counting)
+    a = call()
+    assert counting.took == 1
+    b = call(stream=torch.cuda.current_stream())
+    assert counting.took == 1
     torch.cuda.synchronize()
     assert type(a) is type(b) and (not isinstance(a, dict) or list(a) == list(b))
     for x, y in zip(_flat(a), _flat(b)):

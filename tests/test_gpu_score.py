@@ -14,6 +14,9 @@ TOL = 1e-5   # fp32 outputs, max |d|
 
 
 def run_score(inp: W.ScoreInputs, workspace=None):
+    # with a workspace the call takes the native marshalling, as a decoding program's does
+    if workspace is None and inp.topk > 0:
+        workspace = api.score_workspace(inp.n_seq)
     logits = H.to_dev(inp.logits, "bf16")
     kw = {}
     if inp.cur_tok is not None:
