@@ -80,8 +80,8 @@ struct ScoreArgs {
 
 int launch_score(const ScoreArgs& a, int* status, cudaStream_t stream);
 
-// One decoding step's decisions, run by the last CTA of each segment after the
-// per-row scoring (a.topk, a.eligible, a.cur_tok, a.topk_idx and a.topk_score
+// One decoding step's decisions, one CTA per segment after the per-row scoring
+// of the segment, in the same launch or behind it (a.topk, a.eligible, a.cur_tok, a.topk_idx and a.topk_score
 // are unused; a.score receives the seed scores of the updated state).
 struct DecideArgs {
   const uint8_t* draft_ok;   // [N] or null (every masked row may be drafted)

@@ -550,9 +550,10 @@ int launch_attn_mass(const MassArgs& a, int* status, cudaStream_t stream) {
   });
   if (rc != 0) return rc;
   // Tiles per CTA: two while the tiles outnumber the SMs; below that one tile a CTA spreads over
-  // more SMs. us at NT = 1 / 2 when the rule was set (B, heads, rows): 4, 32, 256: 16.8 / 10.9; 1,
-  // 32 / 32, 1024: 34.9 / 23.7; 2, 32 / 8, 256 (128 tiles): 9.5 / 10.2; 1, 28 / 4, 512 (112 tiles):
-  // 12.0 / 14.4.
+  // more SMs. us at NT = 1 / 2, 32 seeds (B, heads, rows: tiles), both launches: 1, 32, 256: 64 8.1 / 8.6;
+  // 1, 28/4, 512: 112 11.2 / 12.3; 2, 28/4, 256: 112 9.2 / 8.9; 2, 32/8, 256: 128 8.4 / 9.0; 1, 32/8, 512: 128
+  // 10.5 / 11.9; 2, 38, 256: 152 9.5 / 9.4; 1, 32, 640: 160 21.1 / 13.8; 3, 28/4, 256: 168 14.3 / 9.5; 4, 32,
+  // 256: 256 14.6 / 9.5; 1, 32, 1024: 256 30.1 / 18.5.
   const bool pair = n_t > 1 && n_t <= kMaxTilesPair && static_cast<long long>(n_t) * a.Hq * a.B > n_sm;
   rc = pair ? launch_tiles<2>(a, n_t, tq, tk, part_in, part_out, status, stream)
             : launch_tiles<1>(a, n_t, tq, tk, part_in, part_out, status, stream);

@@ -12,19 +12,21 @@
 // the warp and then across the warps in fp32 with error-free TwoSum pairs.
 // Then c = 1/Z, H = ln Z - ln(2) S / Z, u = ln Z - (x_y - m).
 //
-// Top-k (Section 5.3): the last CTA to finish a segment (sequence) - found
+// Top-k (Section 5.3): a segment's (sequence's) k best eligible rows by (score
+// descending, index ascending) on 64-bit keys. Up to 288 rows (one per thread of
+// the row kernel's CTA) the last CTA to finish a segment ranks them; it is found
 // with a self-resetting counter per segment, incremented with acquire-release
-// semantics - takes the segment's k best eligible rows by (score descending,
-// index ascending) on 64-bit keys: by rank when every row has its own thread,
-// else by warp sorts and merges (k <= 32) or a bitonic sort in shared memory.
+// semantics. Longer segments' lists come from a launch of their own behind the
+// rows (topk_kernel), lists of one or two rows excepted.
 //
 // Decision step (cover_score_decide_fwd, Sections 5.2, 3 and 5.3): the row
 // pass keeps u of the current token and ln Z (= u of the greedy token) in a
-// workspace; the last CTA of a segment then drafts the most confident masked
-// rows above the threshold (at most B), applies Keep / Replace / ReMask to the
-// previous seeds, scores the updated state, counts the scores above their mean
-// (n_t pi_t), and selects ceil(sqrt(n_t pi_t)) new seeds among the rows that
-// were not seeds and have ReMasks left, with the same 64-bit key sort.
+// workspace. Per segment, the most confident masked rows above the threshold
+// are then drafted (at most B), Keep / Replace / ReMask applied to the previous
+// seeds, the updated state scored, the scores above their mean counted
+// (n_t pi_t), and ceil(sqrt(n_t pi_t)) new seeds selected among the rows that
+// were not seeds and have ReMasks left, with the same 64-bit keys: by the last
+// CTA of a segment up to 288 rows, in a launch of its own (decide_kernel) above.
 //
 // Streaming: a producer warp issues cp.async.bulk copies of 16 KB chunks of the row's aligned
 // 16-byte vectors into a 3-stage shared-memory ring (mbarrier full / empty), 8 consumer warps
@@ -623,7 +625,7 @@ __device__ __forceinline__ void top_select(uint64_t* keys, int n, int k, uint64_
     top_warps(keys, n, k, out);
 }
 
-// Sections 5.2 and 3, run by the last CTA of a segment: drafting and the
+// Sections 5.2 and 3 for a segment of any length, by one CTA: drafting and the
 // revision of the previous seeds. Updates tok, remask_cnt, flags (bit 1 marks
 // the rows drafted in this step; a drafted row loses bit 0) and ws_u (the
 // uncertainty of each row's updated token: ln Z for drafted and replaced rows).
@@ -1724,7 +1726,10 @@ int launch_rows(const ScoreParams& P, int N, size_t smem, int* status, cudaStrea
 // shared anyway and every further CTA only adds its start and reduction. us at 1 / 2 / 4 / 8 CTAs a
 // row, V = 126464: 32 rows 12.5 / 9.2 / 7.4 / 6.8, 64 rows 12.7 / 9.5 / 8.5 / 8.9, 128 rows 13.6 / 12.0
 // / 12.4 / 15.9, 152 rows 14.7 / 13.4 / 17.3 / 20.2, 200 rows 17.8 / 18.4 / 22.1 / 24.2. V = 32000:
-// 32 rows 6.4 / 6.3 / 5.9 / 5.5, 128 rows 7.0 / 7.2 / 7.7 / 11.5: halves of a short row do not pay.
+// 32 rows 6.4 / 6.3 / 5.9 / 5.5, 128 rows 7.0 / 7.2 / 7.7 / 11.5: halves of a short row do not pay. Where they
+// begin to, 1 / 2 CTAs a row: 100 rows of 60000 7.7 / 7.8, of 65536 7.7 / 7.7, of 80000 9.1 / 8.5; 152 rows 8.1 /
+// 8.3, 8.2 / 8.2, 9.6 / 9.2. Two CTAs a row that do not fit two to an SM: 154 rows of 80000 10.9 / 12.0, of 126464
+// 14.6 / 15.3.
 int row_split(int N, int V, int n_sm) {
   int c = kMaxSplit;
   while (c > 1 && (static_cast<long long>(N) * c > 2LL * n_sm || V < c * kMinSlice || (c == 2 && V < 65536))) c >>= 1;

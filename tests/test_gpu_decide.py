@@ -102,7 +102,7 @@ def check(di: W.DecideInputs, p, r, *, dio=True, draft_ok=True, fp64_rows=None, 
 
 @pytest.mark.parametrize("N,V,n_seq,block", [
     (1, 300, 1, 1), (16, 1000, 2, 4), (64, 4096, 4, 8), (96, 5003, 3, 16), (256, 2048, 1, 64),
-    (512, 1000, 2, 64),
+    (512, 1000, 2, 64), (100, 20001, 2, 16),   # the last: rows loaded to registers
 ])
 def test_decide_shapes(N, V, n_seq, block):
     for seed in range(3):
@@ -155,7 +155,7 @@ def test_decide_longest_segment_and_workspace_reuse():
         check(di, p, run_decide(di, p, workspace=ws), what="4096 rows")
 
 
-def test_decide_register_path_odd_vocab():
+def test_decide_odd_vocab():
     di = W.make_decide_inputs(48, 3001, 2, seed=29, block_len=8)   # V % 8 != 0: unaligned rows
     p = _params()
     check(di, p, run_decide(di, p), what="odd V")
