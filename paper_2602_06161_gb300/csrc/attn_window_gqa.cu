@@ -40,6 +40,8 @@
 #include <cuda_fp16.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "cluster.cuh"
 #include "context.cuh"
 #include "kernels.cuh"
@@ -643,15 +645,18 @@ int win_setup(WinSetup* out, size_t smem) {
   });
 }
 
-// Predicted microseconds of one call, fitted to calls measured back to back on
-// GB300 (Dream-shaped windows of 16 to 128 rows over 1024 keys, batches of 1 to 8, memories of
-// 2048 to 8192 keys; up to 19 % high, and the square kernel's up to 21 % low, over 22 shapes, on
-// all of which the faster kernel was taken): a packed CTA takes about 7 us plus
-// 1.5 us per KV step, and the clusters beyond those resident at once run in further waves (the
-// square kernel's prediction: window_square_us).
-double packed_us(const WinShape& w, const WinSetup& su) {
+// Predicted microseconds of one call, fitted to calls measured back to back on GB300 (250 windows of 1 to
+// 256 rows over 40 to 8192 keys, batches of 1 to 12, 16 / 2, 28 / 4 and 32 / 8 heads): a packed CTA takes
+// about 5.4 us, 1.2 us per KV step and 0.09 us per row that it combines from the cluster's splits, and the
+// clusters beyond those resident at once run in further waves. With the square kernel's prediction
+// (window_square_us) the slower kernel was taken on three of them, by at most 3 % (without the rows'
+// term, 7 us + 1.5 us per step, on thirty: 4, 28 / 4, 4 rows over 297 keys 9.7 instead of 7.9 us). The times
+// themselves are up to 26 % low (one KV tile, where the square kernel is ahead by more) and 30 % high (a
+// wave or two of clusters).
+double packed_us(const WinShape& w, int Lq, const WinSetup& su) {
   const long long waves = (w.clusters + su.max_clusters[w.nsplit] - 1) / su.max_clusters[w.nsplit];
-  return static_cast<double>(waves) * (7.0 + 1.5 * w.T);
+  const int owned = static_cast<int>((std::min<long long>(static_cast<long long>(w.G) * Lq, kBM) + w.nsplit - 1) / w.nsplit);
+  return static_cast<double>(waves) * (5.4 + 1.2 * w.T + 0.09 * owned);
 }
 
 bool packed_supported(const AttnArgs& a) {
@@ -680,7 +685,7 @@ WindowChoice window_gqa_model(const AttnArgs& a, int n_sm, const int* max_cluste
   c.clusters = w.clusters;
   // a cluster of nsplit CTAs that cannot be resident leaves only the square kernel
   c.resident = su.max_clusters[w.nsplit] >= 1;
-  c.packed_us = c.resident ? packed_us(w, su) : 0.0;
+  c.packed_us = c.resident ? packed_us(w, a.Lq, su) : 0.0;
   c.square_us = window_square_us(a, n_sm);
   c.packed = c.resident && c.packed_us < c.square_us;
   return c;

@@ -28,6 +28,13 @@ def _model(B, Hq, Hkv, Lk, Lq, q0=None, **gpu):
     (1, 32, 8, 8192, 64, True),      # 36.5 against 60.7 us
     (8, 32, 8, 2048, 64, False),     # 90.1 against 39.7 us
     (2, 16, 2, 2048, 32, True),      # 10.2 against 19.1 us
+    # two or three KV tiles, by the rows that a CTA combines
+    (4, 28, 4, 297, 4, True),        # 7.9 against 9.7 us
+    (8, 16, 2, 312, 7, True),        # 8.7 against 9.9 us
+    (2, 32, 8, 298, 10, True),       # 8.3 against 8.8 us
+    (2, 28, 4, 323, 11, False),      # 9.4 against 8.7 us
+    (1, 28, 4, 258, 18, False),      # 11.2 against 8.4 us
+    (2, 28, 4, 122, 4, False),       # 11.2 against 6.0 us
 ])
 def test_choice_on_the_measured_windows(B, Hq, Hkv, Lk, Lq, packed):
     c = _model(B, Hq, Hkv, Lk, Lq)
