@@ -209,9 +209,10 @@ __device__ __forceinline__ void raise_abort(AttnSmem& sm, int* status, int site)
 // kFault: the self-test instance that takes its wait limit and a planted missing load from
 // `flt`; the production instances wait up to one second and load every tile.
 // kPad: a split unit's halves may have an odd number of KV tiles between them, and a window's rows may be
-// packed heads. Without it are square launches whose units are not all split, which the compiler then
-// schedules 7 % faster on long sequences, and one-tile windows of unpacked heads over an even number of
-// KV tiles (8 x 32 heads, 64 rows over 2048 keys: 49.7 -> 49.5 us; 32 heads, 32 rows over 512: 7.98 -> 7.90).
+// packed heads. What needs neither runs without it: square launches that are not split over an odd number
+// of tiles, which the compiler then schedules 7 % faster on long sequences, and windows of unpacked heads
+// (8 x 32 heads, 64 rows over 2048 keys: 49.7 -> 49.5 us; 32 heads, 32 rows over 512: 7.98 -> 7.90; 3 x 32 heads,
+// 176 rows over 2493: 44.7 -> 43.7).
 template <int NQ, bool kWindow, bool kFault, bool kPad = kWindow>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_bf16_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
@@ -1109,6 +1110,10 @@ struct WindowPlan {
 // Before, a window was unpacked, with one tile a unit up to 128 rows and two above, and its keys were
 // split for an even number of KV tiles only: 2, 32/32, 3400, 100 (27 tiles) 42.2 -> 30.8; 1, 32/32,
 // 640, 64 (5 tiles) 11.5 -> 10.4; 8, 32/8, 1100, 64 (9 tiles) 34.4 -> 17.0.
+// The plain plan (unpacked, one tile up to 128 rows and two above) stays unless another is 8 % below it: in
+// one-tile units, predicted 5 and 7 % below, 5 x 32 heads, 178 rows over 813 keys took 36.5 instead of 35.1 us
+// and 6 x 32 heads, 157 over 488 28.3 instead of 27.6.
+constexpr double kPlanGain = 1.08;
 WindowPlan plan_window(const AttnArgs& a, int n_sm) {
   const int G = a.Hq / a.Hkv, nkv = (a.L + kBN - 1) / kBN;
   WindowPlan best{false, a.Lq <= kBM ? 1 : 2, 0.0};
@@ -1119,6 +1124,7 @@ WindowPlan plan_window(const AttnArgs& a, int n_sm) {
     return static_cast<double>((units + n_sm - 1) / n_sm) * (2.0 + 1.7 * steps) + 3.0;
   };
   best.us = us(best.pack, best.nq);
+  const WindowPlan plain = best;
   const auto consider = [&](bool pack, int nq) {
     const double t = us(pack, nq);
     if (t < best.us) best = WindowPlan{pack, nq, t};
@@ -1129,7 +1135,7 @@ WindowPlan plan_window(const AttnArgs& a, int n_sm) {
     consider(true, 2);
     consider(true, 1);
   }
-  return best;
+  return kPlanGain * best.us < plain.us ? best : plain;
 }
 
 }  // namespace
@@ -1179,7 +1185,8 @@ int launch_attn_bf16_sm103(const AttnArgs& args, int* status, cudaStream_t strea
                     attn_bf16_kernel<2, true, false>, attn_bf16_kernel<2, false, true>,
                     attn_bf16_kernel<1, true, true>, attn_bf16_kernel<2, true, true>,
                     attn_bf16_kernel<2, false, false, true>, attn_bf16_kernel<2, false, true, true>,
-                    attn_bf16_kernel<1, true, false, false>, attn_bf16_kernel<1, true, true, false>}) {
+                    attn_bf16_kernel<1, true, false, false>, attn_bf16_kernel<1, true, true, false>,
+                    attn_bf16_kernel<2, true, false, false>, attn_bf16_kernel<2, true, true, false>}) {
       if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return -3;
       // the register split inside the kernel assumes exactly kLaunchRegs per thread at launch;
@@ -1197,8 +1204,10 @@ int launch_attn_bf16_sm103(const AttnArgs& args, int* status, cudaStream_t strea
   // launches), two CTAs per unit; with an odd number of KV tiles only where it is the only round.
   const long long rounds = n_units / n_sm, n_last = n_units % n_sm;
   // One-tile units of a window are split inside their CTAs (both softmax warpgroups on the two
-  // halves of the keys).
-  const bool split_all = nq == 1 && nkv >= 2;
+  // halves of the keys); with three KV tiles only while they run in one round: halves of two tiles, one of
+  // them past the memory, save one step of three and cost the merge (7 x 32 heads, 18 rows over 268 keys, 224
+  // units: 17.9 against 17.1 us; 1 x 32 heads 8.4 against 8.7).
+  const bool split_all = nq == 1 && nkv >= 2 && (nkv != 3 || n_units <= n_sm);
   const int n_split = split_all ? static_cast<int>(n_units)
                       : (!window && nkv >= 2 && (nkv % 2 == 0 || rounds == 0) && n_last > 0 && 2 * n_last <= n_sm)
                           ? static_cast<int>(n_last) : 0;
@@ -1210,13 +1219,15 @@ int launch_attn_bf16_sm103(const AttnArgs& args, int* status, cudaStream_t strea
                     make_fastdiv(static_cast<uint32_t>(a.Hq)), make_fastdiv(static_cast<uint32_t>(a.Hq / a.Hkv)),
                     make_fastdiv(static_cast<uint32_t>(period))};
   const bool fault = a.fault_cta >= 0 || a.wait_ns > 0;
-  const bool pad = n_split > 0 && nkv % 2 != 0;
-  auto kernel = !window && pad ? (fault ? attn_bf16_kernel<2, false, true, true> : attn_bf16_kernel<2, false, false, true>)
-                : !window     ? (fault ? attn_bf16_kernel<2, false, true> : attn_bf16_kernel<2, false, false>)
-                : nq == 1 && nkv % 2 == 0 && !pack
-                    ? (fault ? attn_bf16_kernel<1, true, true, false> : attn_bf16_kernel<1, true, false, false>)
-                : nq == 1     ? (fault ? attn_bf16_kernel<1, true, true> : attn_bf16_kernel<1, true, false>)
-                              : (fault ? attn_bf16_kernel<2, true, true> : attn_bf16_kernel<2, true, false>);
+  // padding (kPad) for split units over an odd number of KV tiles, and the row wrap with it for packed heads
+  const bool pad = (n_split > 0 && nkv % 2 != 0) || pack;
+  auto kernel =
+      !window   ? pad ? (fault ? attn_bf16_kernel<2, false, true, true> : attn_bf16_kernel<2, false, false, true>)
+                      : (fault ? attn_bf16_kernel<2, false, true, false> : attn_bf16_kernel<2, false, false, false>)
+      : nq == 1 ? pad ? (fault ? attn_bf16_kernel<1, true, true, true> : attn_bf16_kernel<1, true, false, true>)
+                      : (fault ? attn_bf16_kernel<1, true, true, false> : attn_bf16_kernel<1, true, false, false>)
+                : pad ? (fault ? attn_bf16_kernel<2, true, true, true> : attn_bf16_kernel<2, true, false, true>)
+                      : (fault ? attn_bf16_kernel<2, true, true, false> : attn_bf16_kernel<2, true, false, false>);
   // programmatic dependent launch: the prologue overlaps the previous kernel's tail
   cudaLaunchAttribute attr[1];
   const cudaLaunchConfig_t cfg = pdl_config(dim3(static_cast<unsigned>(grid)), dim3(kThreads), smem, stream, attr);
