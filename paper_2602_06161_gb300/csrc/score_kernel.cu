@@ -17,7 +17,7 @@
 // the row kernel's CTA) the last CTA to finish a segment ranks them; it is found
 // with a self-resetting counter per segment, incremented with acquire-release
 // semantics. Longer segments' lists come from a launch of their own behind the
-// rows (topk_kernel), lists of one or two rows excepted.
+// rows (topk_kernel), lists of up to 8 rows excepted.
 //
 // Decision step (cover_score_decide_fwd, Sections 5.2, 3 and 5.3): the row
 // pass keeps u of the current token and ln Z (= u of the greedy token) in a
@@ -62,7 +62,7 @@ constexpr int kMaxPerSeq = 4096;            // rows per segment (the entry point
 constexpr int kRowLoads = 4;                // rows whose state a thread loads at once (general paths)
 constexpr int kRoundsMax = 32;              // selections up to this size by rounds or warp sorts (top_select)
 constexpr int kRoundsFew = 8;               // selections up to this size by per-warp rounds (top_rounds)
-constexpr int kFusedTopk = 2;               // longest list that the row kernel finds in segments longer than its CTAs
+constexpr int kFusedTopk = kRoundsFew;      // longest list that the row kernel finds in segments longer than its CTAs
 constexpr int kMaxWarps = 32;               // the selection kernels run up to 1024 threads
 constexpr int kMaxThreads = 32 * kMaxWarps;
 constexpr int kRankWarps = 16;              // top_small ranks the published keys of up to this many warps
@@ -1291,9 +1291,10 @@ __device__ __forceinline__ void topk_put(uint64_t key, size_t slot, int32_t* top
   if (topk_score != nullptr) topk_score[slot] = key != 0 ? order_key_inv(static_cast<uint32_t>(key >> 32)) : -INFINITY;
 }
 
-// The last CTA of a segment in the row kernel: ranks where every row has a thread, else a list of one or two.
+// The last CTA of a segment in a row kernel: ranks where every row has a thread of the bulk-copy kernel's,
+// else a list of a few.
 __device__ __forceinline__ void segment_topk(uint64_t* keys, int seg, const ScoreParams& P) {
-  if (P.per_seq <= static_cast<int>(blockDim.x)) {
+  if (P.per_seq <= kBulkThreads) {
     topk_rank(keys, seg, P.per_seq, P.topk, P.score, P.eligible, P.topk_idx, P.topk_score);
     return;
   }
@@ -1587,7 +1588,7 @@ __global__ void __launch_bounds__(kRegThreads, 2) score_reg_kernel(const ScorePa
     if (P.decide)
       decide_fast<false>(reg_keys, n / P.per_seq, P.per_seq, P);
     else
-      topk_rank(reg_keys, n / P.per_seq, P.per_seq, P.topk, P.score, P.eligible, P.topk_idx, P.topk_score);
+      segment_topk(reg_keys, n / P.per_seq, P);
   }
 }
 
@@ -1604,16 +1605,18 @@ __global__ void __launch_bounds__(kMaxThreads) decide_kernel(const ScoreParams P
   segment_decide(dec_keys, blockIdx.x, P.per_seq, P.sort_n, P);
 }
 
-// The top-k of such segments, likewise (for lists of more than kFusedTopk: one or two rows are found in
-// the row kernel's last CTA before this launch would start). How, by the rows and the list, with the us
-// that the launch adds behind rows of 1001 logits:
-//   rows           list       merged lists   ranks   rounds / warp sorts, 288 / 512 / 1024 threads   sort, 512 / 1024
-//   289            <= 32      2.6            3.9     k = 8: 4.2 / 4.1; k = 32: 6.1 / 6.9             9.4 / 10.2
-//   289, 400, 512  33 .. 200                 3.9, 5.4, 6.3                                           9.4, 9.6, 9.5 / 10.2, 9.8, 10.5
-//   640, 768, 1024 33 .. 200                 9.3, 13.0, 21.7                                         17.3, 17.5, 17.8 / 14.1, 14.3, 14.4
-//   1024           <= 32      3.6            21.7    k = 8: 4.9 / 4.9 / 6.1; k = 32: 6.1 / 8.4 / 16.1
-//   2048           <= 32                             k = 8: 6.0 / 5.5 / 6.7; k = 32: 8.6 / 8.1 / 16.2
-//   4096           <= 32                             k = 8: 8.4 / 7.3 / 8.4; k = 32: 14.2 / 12.0 / 16.5
+// The top-k of such segments, likewise, for lists of more than kFusedTopk. Shorter ones stay with the row
+// kernel's last CTA: rounds take it about as long as the second launch takes this kernel (600 rows of 1001
+// logits, k = 1 / 8: 6.3 / 8.3 us against 6.7 / 6.7), and a call of little work is bound by the host, where the
+// launch costs 2 us. How, by the rows and the list, with the us that the launch adds behind rows of 1001
+// logits:
+//   rows           list       merged lists   ranks             warp sorts, 288 / 512 / 1024 threads   sort, 512 / 1024
+//   289            <= 32      2.6            3.9               6.1 / 6.9                              9.4 / 10.2
+//   289, 400, 512  33 .. 200                 3.9, 5.4, 6.3                                            9.4, 9.6, 9.5 / 10.2, 9.8, 10.5
+//   640, 768, 1024 33 .. 200                 9.3, 13.0, 21.7                                          17.3, 17.5, 17.8 / 14.1, 14.3, 14.4
+//   1024           <= 32      3.6            21.7              6.1 / 8.4 / 16.1
+//   2048           <= 32                                       8.6 / 8.1 / 16.2
+//   4096           <= 32                                       14.2 / 12.0 / 16.5
 // In the row kernel's last CTA of 288 threads, lists of more than 32 rows were sorted: 1 x 512 rows of 20001
 // logits, k = 64: 20.7 us; a row kernel of 512 threads ranked them: 16.4; now 13.3 (1024 rows: 39.3, 35.2, 25.3).
 constexpr int kRankRows = 768;        // segments up to this size are ranked, for lists of more than kRoundsMax
@@ -1645,7 +1648,7 @@ __global__ void __launch_bounds__(kMaxThreads) topk_kernel(const ScoreParams P) 
     const uint64_t* best = topk_smem;
     topk_keys(topk_smem, seg, P.per_seq, P.sort_n, P.score, P.eligible);
     if (P.topk <= kRoundsMax) {
-      top_select(topk_smem, P.sort_n, P.topk, s_sel);
+      top_warps(topk_smem, P.sort_n, P.topk, s_sel);
       best = s_sel;
     } else {
       bitonic_sort_desc(topk_smem, P.sort_n);
@@ -1783,8 +1786,8 @@ int launch_score_impl(const ScoreArgs& a, const DecideArgs* d, int* status, cuda
   const int split = row_split(a.N, a.V, n_sm);
   if (loads_to_registers(a.N, a.V, split, n_sm)) {
     cudaLaunchAttribute attr[1];
-    const cudaLaunchConfig_t cfg =
-        pdl_config(dim3(static_cast<unsigned>(a.N)), dim3(kRegThreads), sizeof(uint64_t) * kRegThreads, stream, attr);
+    const cudaLaunchConfig_t cfg = pdl_config(dim3(static_cast<unsigned>(a.N)), dim3(kRegThreads),
+                                              sizeof(uint64_t) * std::max(sort_n, kRegThreads), stream, attr);
     rl = cudaLaunchKernelEx(&cfg, score_reg_kernel, rows) == cudaSuccess ? 0 : -3;
   } else {
     switch (split) {

@@ -164,12 +164,18 @@ def test_score_topk_fewer_eligible_than_k(per, k, frac):
         assert (r["topk_idx"][g, n_elig[g]:] == -1).all() and (r["topk_idx"][g, :n_elig[g]] >= 0).all()
 
 
+@pytest.mark.parametrize("N,k", [(304, 8), (304, 9), (288, 40), (200, 3)])
+def test_score_topk_of_rows_loaded_to_registers(N, k):
+    inp = W.make_score_inputs(N, 18435, 1, k, seed=N + k, eligible_frac=0.7)
+    check(inp, run_score(inp))
+
+
 @pytest.mark.parametrize("per,k", [
-    (289, 2), (1025, 2),                            # found in the row kernel
-    (289, 3), (512, 32), (513, 32), (1024, 32),     # the lists of 10 to 32 warps, merged
+    (289, 2), (289, 8), (1025, 8), (4096, 3),       # found in the row kernel
+    (289, 9), (512, 32), (513, 32), (1024, 32),     # the lists of 10 to 32 warps, merged
     (289, 33), (300, 300), (768, 33), (768, 700),   # ranks
     (769, 33), (1024, 1024), (1025, 33),            # sorts
-    (1025, 3), (1025, 32), (4096, 9),               # rounds, warp sorts on 512 threads
+    (1025, 9), (1025, 32), (4096, 32),              # warp sorts on 512 threads
 ])
 @pytest.mark.parametrize("frac", [1.0, 0.6, 0.005])
 def test_score_topk_of_long_segments(per, k, frac):
