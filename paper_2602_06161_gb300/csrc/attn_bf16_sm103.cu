@@ -1204,10 +1204,10 @@ int launch_attn_bf16_sm103(const AttnArgs& args, int* status, cudaStream_t strea
   // launches), two CTAs per unit; with an odd number of KV tiles only where it is the only round.
   const long long rounds = n_units / n_sm, n_last = n_units % n_sm;
   // One-tile units of a window are split inside their CTAs (both softmax warpgroups on the two
-  // halves of the keys); with three KV tiles only while they run in one round: halves of two tiles, one of
-  // them past the memory, save one step of three and cost the merge (7 x 32 heads, 18 rows over 268 keys, 224
-  // units: 17.9 against 17.1 us; 1 x 32 heads 8.4 against 8.7).
-  const bool split_all = nq == 1 && nkv >= 2 && (nkv != 3 || n_units <= n_sm);
+  // halves of the keys), except plain ones over three KV tiles: halves of two tiles, one of them past the memory,
+  // save one step of three and cost the merge (1 x 32 heads, 18 rows over 268 keys 8.4 against 8.7 us, but 7 x 32
+  // heads 17.9 against 17.1 and, with 53 seeds in the window, 2 x 28/4 heads, 105 rows over 351 13.9 against 13.1).
+  const bool split_all = nq == 1 && nkv >= 2 && (nkv != 3 || pack);
   const int n_split = split_all ? static_cast<int>(n_units)
                       : (!window && nkv >= 2 && (nkv % 2 == 0 || rounds == 0) && n_last > 0 && 2 * n_last <= n_sm)
                           ? static_cast<int>(n_last) : 0;
