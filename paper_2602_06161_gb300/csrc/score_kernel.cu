@@ -1740,18 +1740,21 @@ int row_split(int N, int V, int n_sm) {
 }
 
 // Whether unaligned rows go through the register-load kernel: with one or two unsplit rows per SM its 16
-// warps are ahead of the ring's 8, if a row is little more than whole batches of its CTA (16384 elements; the
-// rest goes a vector at a time) or long. us through the ring / registers:
-//   rows   V = 20001    26001        30001        36355        50257        80001          108602         152065
-//   77     4.3 / 3.9    4.7 / 4.5    4.9 / 5.1    5.4 / 4.6    6.6 / 6.3    (split)
-//   152    4.5 / 4.3    5.4 / 6.0    6.0 / 7.3    6.6 / 6.0    7.5 / 7.1    (split)
-//   153    5.0 / 5.2    5.8 / 6.5    6.6 / 7.8    7.3 / 6.7    8.6 / 7.8    11.1 / 10.9    13.3 / 12.7    16.8 / 15.6
-//   250    6.3 / 6.0    7.0 / 7.3    7.5 / 8.4    8.0 / 7.2    9.2 / 8.7    11.8 / 11.9    14.1 / 13.7    17.8 / 16.9
-//   320    8.2 / 8.9    9.2 / 11.2   10.0 / 13.0  10.9 / 10.8  12.8 / 12.9  17.4 / 18.3    21.4 / 21.8    27.8 / 27.0
-// and 4.0 / 4.1 at 153 rows of 8001, 4.4 / 4.9 of 16385.
+// warps are ahead of the ring's 8, except where much of a short row is left over whole batches of its CTA
+// (16384 elements; the rest goes a vector at a time). us through the ring / registers, by rows and V:
+//   rows   18435      20001      26001      30001      36355      45001      48001      53001      65001
+//   100    4.2 / 3.8  4.3 / 4.0  4.8 / 4.7  5.1 / 5.1  5.8 / 5.3  6.6 / 6.7  6.9 / 7.5  7.3 / 6.7  7.9 / 7.9
+//   153    4.7 / 5.0  5.0 / 5.2  5.8 / 6.5  6.6 / 7.8  7.2 / 6.6  7.9 / 7.9  8.4 / 8.4  8.6 / 7.8  9.5 / 9.1
+//   250    6.0 / 5.9  6.3 / 6.0  7.0 / 7.3  7.5 / 8.4  8.0 / 7.1  8.7 / 8.4  9.2 / 9.1  9.5 / 8.6  10.3 / 9.9
+//   rows   78001        85001        90125        95001        99001        113001       130001       152065
+//   153    10.7 / 10.6  11.4 / 10.3  11.7 / 11.0  12.1 / 12.2  12.4 / 11.0  13.5 / 12.9  15.0 / 13.6  16.8 / 15.6
+//   250    11.5 / 11.6  12.2 / 11.2  12.6 / 12.1  13.0 / 13.4  13.2 / 12.2  14.4 / 14.0  15.9 / 15.0  17.8 / 16.9
+// and with more rows 320 of 20001 8.2 / 8.9, of 50257 12.8 / 12.9, of 152065 27.8 / 27.0; 153 of 8001 4.0 / 4.1.
 bool loads_to_registers(int N, int V, int split, int n_sm) {
   constexpr int kBatch = kRegThreads * kRegUnroll * 8;
-  return V % 8 != 0 && split == 1 && N <= 2 * n_sm && V >= kBatch / 8 * 9 && (V % kBatch <= kBatch / 4 || V >= 6 * kBatch);
+  const int left = V % kBatch;
+  return V % 8 != 0 && split == 1 && N <= 2 * n_sm &&
+         (V >= 6 * kBatch || (V >= 2 * kBatch && left <= 3 * kBatch / 4) || (V >= 9 * kBatch / 8 && left <= kBatch / 4));
 }
 
 int launch_score_impl(const ScoreArgs& a, const DecideArgs* d, int* status, cudaStream_t stream) {

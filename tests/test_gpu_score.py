@@ -65,7 +65,8 @@ def test_score_shapes(N, V, n_seq, k):
     (77, 65544), (152, 65537),    # two
     (153, 65544),                 # one
     (100, 20001), (153, 36355), (304, 18435), (160, 98305),   # loaded to registers
-    (305, 20001), (100, 20481), (100, 18427),                 # and on the other side of that rule
+    (153, 45055),
+    (305, 20001), (100, 20481), (100, 18427), (153, 45057),   # and on the other side of that rule
 ])
 def test_score_split_rows(N, V):
     """Rows split over a cluster: sums and, with the maximum in several slices, its first index."""
